@@ -4,10 +4,11 @@
 // The paper counts the eigenvalues of each slice from the inertia of
 // D - b_i I at both ends of the slice (Section 3.2, "Validation and Other
 // Details"), using a band LDL^H that keeps no L.  Here the count is computed
-// for many shifts at once (one thread block per shift).  The active
-// (b+1)-column window of the band lives in shared memory when it fits,
-// otherwise in a per-shift slice of the workspace (L2 resident); each step
-// eliminates one column with a rank-1 update of the trailing b x b triangle.
+// for many shifts at once: a thread-block cluster of 1 to 16 CTAs per shift
+// eliminates panels of 8 columns with the active window in (distributed) shared
+// memory (inertia_panel_kernel); bands too wide for that keep the window in a
+// per-shift slice of the workspace (L2 resident), one CTA per shift and one
+// column at a time (inertia_kernel).
 //
 // Every floating-point operation is an explicitly rounded __dmul_rn /
 // __dsub_rn / __ddiv_rn (no contraction), in the same order as the CPU
@@ -16,10 +17,17 @@
 //   W(i,j) -= l_i * conj(W(j,k))  for k < j <= i <= k+b,
 // with t = l*conj(a) formed as (l.re*a.re + l.im*a.im, l.im*a.re - l.re*a.im)
 // and only the real part applied on the diagonal.
+#include <cooperative_groups.h>
 #include <float.h>
 
+#include <algorithm>
+#include <map>
+#include <mutex>
+#include <tuple>
 
 #include "common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace pdeshep {
 
@@ -105,9 +113,14 @@ __device__ __forceinline__ void load_row(typename InertiaElem<CPLX>::T* W, int b
   }
 }
 
-// One CTA per shift.  Shared memory: pair table (s,u) packed as int32, the
-// multipliers L[0..b], the ring heads h[0..b] and (if `gwin` is null) the
-// window rings W[(b+1)(b+2)/2].
+// One CTA per shift, one column per step.  Shared memory: pair table (s,u)
+// packed as int32, the multipliers L[0..b], the ring heads h[0..b] and (if
+// `gwin` is null) the window rings W[(b+1)(b+2)/2].  It serves calls with enough
+// shifts to fill the GPU: its half-square window lets four CTAs of b = 64 complex
+// share an SM and hide each other's barriers, and it spends fewer FP64
+// instructions per column than the panel kernel below (504 shifts, n = 4096,
+// b = 64 complex: 23.5 us per column against 28.1).  Bands that no cluster's
+// shared memory holds also come here (window in the workspace).
 template <bool CPLX>
 __global__ void __launch_bounds__(256) inertia_kernel(int64_t n, int b, const double* __restrict__ band,
                                                       int64_t ldab, const double* __restrict__ sigmas,
@@ -228,6 +241,317 @@ __global__ void __launch_bounds__(256) inertia_kernel(int64_t n, int b, const do
   if (threadIdx.x == 0) neg_out[sid] = neg;
 }
 
+// The pivot in use (zero -> -pivmin), counted in neg if negative; on the bits, since an FP64
+// comparison costs 64 clocks of the step's chain.
+__device__ __forceinline__ double pivot(double dk, double pivmin, int64_t& neg) {
+  long long bits = __double_as_longlong(dk);
+  if ((bits << 1) == 0) {
+    dk = -pivmin;
+    bits = __double_as_longlong(dk);
+  }
+  neg += bits < 0 && (unsigned long long)(bits << 1) <= 0xffe0000000000000ull;  // negative, not NaN
+  return dk;
+}
+
+// ---------------------------------------------------------------------------
+// Panel elimination on a thread-block cluster.  FP64 is the scarce resource
+// (about 1.7 lanes per clock and SM; a warp instruction holds its quadrant's
+// pipe for 64 clocks however few lanes are active, a division takes about 600),
+// so one CTA per shift left 143 of 152 SMs idle at 9 shifts, and one column at a
+// time paid four barriers and the latency of a band row per column.  Here
+//  * a cluster of G CTAs shares one shift: row i of the window belongs to CTA
+//    i mod G (cyclic: every CTA keeps an even share of the shrinking triangle),
+//    which holds its b + 1 entries (i, i-d) at offset d of a row slot;
+//  * kPan = 8 columns are eliminated per round, with two cluster barriers: every
+//    CTA factors the panel's 8 x 8 triangle redundantly together with its own
+//    rows' 8 entries, sends those rows' entries (the a of W -= l conj(a)) to the
+//    other CTAs through distributed shared memory, then applies the 8 updates to
+//    its rows in registers, one read and one write of the window per 8 columns;
+//  * real and imaginary parts are separate lanes (4 FP64 operations each per
+//    update) and the triangle's rows are paired shortest with longest, so that
+//    the lanes of a warp are all in use;
+//  * band rows arrive by cp.async one round ahead.
+// Each entry sees the same rounded operations in the same (ascending column)
+// order as with one column at a time, so counts and pivots keep their bits.
+// Measured against one CTA per shift and one column per step (us per column, all
+// shifts of the call): b = 64 complex, 1 shift 1.5 against 6.7, 9 shifts 2.0
+// against 6.7, 63 shifts 4.5 against 6.8; b = 128 complex, 17 shifts 5.4 against
+// 22.6; b = 32 real, 64 shifts 1.2 against 1.55.  What remains at few shifts is
+// the chain of a column: a division and four dependent operations, about 1.2k of
+// 3k clocks, then the share of the updates (1k) and two cluster barriers per 8.
+// ---------------------------------------------------------------------------
+constexpr int kPan = 8;
+constexpr int kPanThreads = 256;
+static_assert(kPan * 32 == kPanThreads, "one warp per panel column");
+
+struct PanelShape {
+  int nslot;   // row slots of one CTA
+  int rown;    // own rows below a panel, at most
+  int chunks;  // warps that hold one panel column (a lane per entry and part)
+  size_t smem;
+};
+static PanelShape panel_shape(int b, int cplx, int G) {
+  PanelShape s;
+  s.nslot = (int)ceil_div(b + 2 * kPan, G);  // rows k .. k+b+2 kPan-1 are live during panel k
+  s.rown = (int)ceil_div(b, G);
+  const size_t np = cplx ? 2 : 1;
+  s.chunks = (int)ceil_div((kPan + s.rown) * (int64_t)np, 32);
+  s.smem = sizeof(double) * np *
+           ((size_t)s.nslot * (b + 1) + (size_t)kPan * kPan + (size_t)2 * (kPan + s.rown) * kPan +
+            (G > 1 ? (size_t)b * kPan : 0));
+  return s;
+}
+
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
+}
+
+// v - t with t = l a (real) or the `part` (0: real, 1: imaginary) of l conj(a):
+// re: l.re a.re + l.im a.im, im: l.im a.re - l.re a.im, every operation rounded
+__device__ __forceinline__ double sub_prod(double v, double l, double a) { return __dsub_rn(v, __dmul_rn(l, a)); }
+__device__ __forceinline__ double sub_prod(double v, double2 l, double2 a, int part) {
+  const double l1 = part ? l.y : l.x, l2 = part ? -l.x : l.y;
+  return __dsub_rn(v, __dadd_rn(__dmul_rn(l1, a.x), __dmul_rn(l2, a.y)));
+}
+
+// a / d rounded to nearest; zeros (the division's slow path) are handled on the bits
+__device__ __forceinline__ double quotient(double a, double d) {
+  const long long ab = __double_as_longlong(a), db = __double_as_longlong(d);
+  const bool zero = (ab << 1) == 0;
+  const double q = __ddiv_rn(zero ? 1.0 : a, d);
+  const bool nan = (unsigned long long)(db << 1) > 0xffe0000000000000ull;
+  return zero && !nan ? __longlong_as_double((ab ^ db) & (long long)0x8000000000000000ull) : q;
+}
+
+template <bool CPLX, int NC>
+__global__ void __launch_bounds__(kPanThreads)
+    inertia_panel_kernel(int64_t n, int b, const double* __restrict__ band, int64_t ldab,
+                         const double* __restrict__ sigmas, const unsigned long long* amax_bits,
+                         int64_t* __restrict__ neg_out, double* __restrict__ piv_out, int nslot, int rown,
+                         int chunks) {
+  using T = typename InertiaElem<CPLX>::T;
+  constexpr int NP = CPLX ? 2 : 1;
+  extern __shared__ __align__(16) char smem[];
+  cg::cluster_group cl = cg::this_cluster();
+  const int G = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int sid = blockIdx.x / G;
+  const int tid = threadIdx.x;
+  const int rl = (b + 1) * NP;                      // doubles of a row slot
+  double* W = (double*)smem;                        // [nslot][b + 1][NP]
+  double* Tri = W + (size_t)nslot * rl;             // [kPan][kPan][NP]: panel rows (r, c), r >= c
+  const int lda = kPan + rown;
+  T* L = (T*)(Tri + kPan * kPan * NP);              // [kPan][lda]: column c's l of the panel rows, then own rows
+  T* A = L + (size_t)lda * kPan;                    // the same for the a of column c
+  T* Ap = G > 1 ? A + (size_t)lda * kPan : A + kPan;  // column c, row k + kPan + j, of all CTAs at c * ldp + j
+  const int ldp = G > 1 ? b : lda;
+  __shared__ double sh_d;                              // the pivot of the next column
+  const int warp = tid >> 5, lane = tid & 31;
+  const double sigma = sigmas[sid];
+  const double amax = __longlong_as_double((long long)*amax_bits);
+  const double a2 = __dmul_rn(amax, amax);
+  const double pivmin = DBL_MIN * (a2 > 1.0 ? a2 : 1.0);
+
+  const int lg = 31 - __clz(G);  // G is a power of two
+  auto first_own = [&](int64_t i) -> int64_t {  // the first row >= i of this CTA
+    return i + ((rank - (int)i) & (G - 1));
+  };
+  auto slot_of = [&](int64_t i) -> int { return (int)((unsigned)(i >> lg) % (unsigned)nslot); };
+  // own rows r0 <= r < r0 + cnt requested (8-byte copies: the band is only known to be 8-byte aligned)
+  auto request_rows = [&](int64_t r0, int cnt) {
+    const int64_t r1 = r0 + cnt < n ? r0 + cnt : n;
+    int64_t r = first_own(r0);
+    if (r >= r1) return;
+    int q = slot_of(r);
+    for (int x = 0; r < r1; r += G, ++x) {  // row number x: its diagonal entry is copied by thread x mod 256
+      double* s = W + (size_t)q * rl;
+      for (int d = (tid - x) & (kPanThreads - 1); d <= b; d += kPanThreads) {
+        const int64_t j = r - d;
+        if (j < 0) break;
+        const double* p = band + NP * (d + j * ldab);
+        cp_async8(s + NP * d, p);
+        if (CPLX) cp_async8(s + NP * d + 1, p + 1);
+      }
+      q = q + 1 == nslot ? 0 : q + 1;
+    }
+  };
+  // ... and finished: the thread that copied a diagonal entry shifts it (own copies are visible to it)
+  auto finish_rows = [&](int64_t r0, int cnt) {
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    const int64_t r1 = r0 + cnt < n ? r0 + cnt : n;
+    const int64_t r = first_own(r0);
+    for (int x = tid; r + (int64_t)x * G < r1; x += kPanThreads) {
+      double* s = W + (size_t)slot_of(r + (int64_t)x * G) * rl;
+      s[0] = __dsub_rn(s[0], sigma);
+      if (CPLX) s[1] = 0.0;
+    }
+  };
+  auto csync = [&]() {
+    if (G > 1)
+      cl.sync();
+    else
+      __syncthreads();
+  };
+  // rows k .. k+kPan-1, columns k .. of them, to every CTA's triangle; q: the slot of the first own one
+  auto send_triangle = [&](int64_t k, int q) {
+    for (int i = (rank - (int)k) & (G - 1); i < kPan && k + i < n; i += G) {
+      const double* s = W + (size_t)q * rl;
+      for (int e = tid; e < (kPan * NP << lg); e += kPanThreads) {
+        const int part = e % NP, c = (e / NP) % kPan, g = e / (NP * kPan);
+        if (c > i) continue;
+        const double v = i - c <= b ? s[NP * (i - c) + part] : 0.0;
+        double* t = G > 1 ? cl.map_shared_rank(Tri, g) : Tri;
+        t[(i * kPan + c) * NP + part] = v;
+      }
+      q = q + 1 == nslot ? 0 : q + 1;
+    }
+  };
+  request_rows(0, b + kPan);
+  finish_rows(0, b + kPan);
+  csync();
+  send_triangle(0, 0);
+  csync();
+
+  int64_t neg = 0;
+  for (int64_t k = 0; k < n; k += kPan) {
+    const int pk = (int)(n - k < kPan ? n - k : kPan);
+    const int nrows = (int)(n - k - pk < b ? n - k - pk : b);  // rows k+kPan .. of the panel
+    const int64_t i0 = first_own(k + kPan);
+    const int off0 = (int)(i0 - (k + kPan));
+    const int s0 = slot_of(i0);
+    auto own = [&](int t) -> double* {  // slot of own row i0 + t G
+      const int q = s0 + t;
+      return W + (size_t)(q >= nslot ? q - nslot : q) * rl;
+    };
+    const int T0 = off0 < nrows ? ((nrows - 1 - off0) >> lg) + 1 : 0;  // own rows among them: i0 + t G
+    const int64_t new0 = k + kPan + b;
+    request_rows(new0, kPan);
+    // ---- the panel.  Its entries live in registers: chunk u of column j (32 lanes of rows: the
+    // triangle's, then the own ones) belongs to warp (j + u) mod 8, so the divisions of a column and
+    // the updates of the others spread over the SM's four FP64 pipes.
+    double v[NC];
+    int rho[NC];  // row - k of this lane's entry in chunk u; past every reach if there is none
+    const int part = lane % NP;
+#pragma unroll
+    for (int u = 0; u < NC; ++u) {
+      const int r = (32 * u + lane) / NP, j = (warp - u) & (kPan - 1), t = r - kPan;
+      const double* src = Tri;
+      rho[u] = 1 << 30;
+      if (r < kPan) {
+        if (r < pk) rho[u] = r;
+        src = Tri + (r * kPan + j) * NP;
+      } else if (t < T0) {
+        rho[u] = kPan + off0 + t * G;
+        if (rho[u] - j <= b) src = own(t) + NP * (rho[u] - j);
+      }
+      v[u] = src[part];
+      if (NC > 1 && u == 0 && warp == 0 && lane == 0) sh_d = v[u];
+    }
+    if (NC > 1) __syncthreads();
+#pragma unroll 1
+    for (int c = 0; c < pk; ++c) {
+      // With one chunk per column the warp of column c has the pivot among its lanes and goes on to the
+      // division at once; the other warps' updates by column c - 1 run beside it.
+      if (NC > 1 || warp == c) {
+        const double dk = pivot(NC > 1 ? sh_d : __shfl_sync(0xffffffffu, v[0], c * NP), pivmin, neg);
+        const bool first = NC > 1 ? tid == 0 : lane == 0;
+        if (piv_out && first && rank == 0) piv_out[(int64_t)sid * n + k + c] = dk;
+#pragma unroll
+        for (int u = 0; u < NC; ++u)
+          if (((warp - u) & (kPan - 1)) == c && u < chunks) {
+            const bool on = rho[u] > c && rho[u] - c <= b;
+            const double l = quotient(on ? v[u] : 1.0, dk);
+            if (on) {
+              const int e = (c * lda + (32 * u + lane) / NP) * NP + part;
+              ((double*)A)[e] = v[u];
+              ((double*)L)[e] = l;
+            }
+          }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < NC; ++u) {
+        const int j = (warp - u) & (kPan - 1);
+        if (j > c && u < chunks) {
+          const bool on = rho[u] > c && rho[u] - c <= b;
+          const T l = L[c * lda + (on ? (32 * u + lane) / NP : 0)], a = A[c * lda + j];
+          double x;
+          if constexpr (CPLX)
+            x = sub_prod(v[u], l, a, part);
+          else
+            x = sub_prod(v[u], l, a);
+          // (an update past the panel's end or above the diagonal changes only entries nothing reads;
+          // the imaginary part of the diagonal is not read either)
+          if (on) v[u] = x;
+          if (NC > 1 && u == 0 && j == c + 1 && lane == (c + 1) * NP) sh_d = v[u];
+        }
+      }
+      if (NC > 1) __syncthreads();
+    }
+    // ---- own rows' panel entries to every CTA
+    if (G > 1) {
+      for (int e = tid; e < (T0 * kPan << lg); e += kPanThreads) {
+        const int g = e & (G - 1), c = (e >> lg) % kPan, t = (e >> lg) / kPan;
+        if (kPan + off0 + t * G - c > b) continue;
+        cl.map_shared_rank(Ap, g)[c * ldp + off0 + t * G] = A[c * lda + kPan + t];
+      }
+    }
+    csync();
+    // ---- the eight updates of the own rows' columns k+kPan .. i
+    if (T0 > 0) {
+      const int len0 = off0 + 1, lenT = off0 + (T0 - 1) * G + 1;
+      const int width = (len0 + lenT) * NP;
+      const int total = ((T0 + 1) / 2) * width;
+      for (int e0 = tid & ~31; e0 < total; e0 += kPanThreads) {
+        const int e = e0 + (tid & 31);
+        bool on = e < total;
+        int t = on ? e / width : 0;
+        int x = on ? e - t * width : 0;
+        const int lt = (off0 + t * G + 1) * NP;
+        if (x >= lt) {
+          x -= lt;
+          if (2 * t == T0 - 1) on = false;  // an odd count: the middle row has no partner
+          t = T0 - 1 - t;
+        }
+        const int part = x % NP, j = x / NP;  // column k + kPan + j
+        const int ri = off0 + t * G;          // row k + kPan + ri
+        if (CPLX && part == 1 && j == ri) on = false;
+        const int c0 = on ? (ri + kPan - b > 0 ? ri + kPan - b : 0) : kPan;  // first column that reaches the row
+        const int cs = __reduce_min_sync(0xffffffffu, c0);
+        double* w = own(t) + NP * (ri - j) + part;
+        double v = on ? *w : 0.0;
+        const T* lp = L + kPan + t;
+        const T* ap = Ap + j;
+#pragma unroll
+        for (int c = 0; c < kPan; ++c) {
+          if (c < cs) continue;
+          if (c < c0) continue;
+          if constexpr (CPLX)
+            v = sub_prod(v, lp[c * lda], ap[c * ldp], part);
+          else
+            v = sub_prod(v, lp[c * lda], ap[c * ldp]);
+        }
+        if (on) *w = v;
+      }
+    }
+    finish_rows(new0, kPan);
+    __syncthreads();
+    if (k + kPan < n) send_triangle(k + kPan, s0);
+    csync();
+  }
+  if (NC > 1) {
+    if (tid == 0 && rank == 0) neg_out[sid] = neg;
+  } else {  // every warp counted the pivots of its column
+    long long* sums = (long long*)A;
+    if (lane == 0) sums[warp] = neg;
+    __syncthreads();
+    if (tid == 0 && rank == 0) {
+      long long total = 0;
+      for (int w = 0; w < kPan; ++w) total += sums[w];
+      neg_out[sid] = total;
+    }
+  }
+}
+
 static size_t window_bytes(int b, int cplx) {
   return (size_t)(b + 1) * (b + 2) / 2 * (cplx ? 16 : 8);
 }
@@ -236,9 +560,8 @@ static size_t inertia_smem_base(int b, int cplx) {
   return ((npairs * 4 + 15) & ~size_t(15)) + (size_t)(b + 1) * (cplx ? 16 : 8) +
          (((size_t)(b + 1) * sizeof(int) + 15) & ~size_t(15));
 }
-static bool window_in_smem(int b, int cplx) {
-  return inertia_smem_base(b, cplx) + window_bytes(b, cplx) <= 226 * 1024;
-}
+static size_t single_smem(int b, int cplx) { return inertia_smem_base(b, cplx) + window_bytes(b, cplx); }
+static bool window_in_smem(int b, int cplx) { return single_smem(b, cplx) <= 226 * 1024; }
 
 // Workspace layout: amax bits, nonfinite flag, sigma[], neg[], global windows.
 struct InertiaWs {
@@ -279,23 +602,130 @@ int launch_band_amax(int64_t n, int b, int cplx, const void* band, int64_t ldab,
   return 0;
 }
 
-// Batched inertia with sigma already on the device; results into d_neg.  Async.
+using PanelKernel = void (*)(int64_t, int, const double*, int64_t, const double*, const unsigned long long*, int64_t*,
+                            double*, int, int, int);
+template <bool CPLX>
+static PanelKernel panel_kernel(int chunks) {
+  return chunks <= 1   ? (PanelKernel)inertia_panel_kernel<CPLX, 1>
+         : chunks <= 2 ? (PanelKernel)inertia_panel_kernel<CPLX, 2>
+         : chunks <= 4 ? (PanelKernel)inertia_panel_kernel<CPLX, 4>
+         : chunks <= 8 ? (PanelKernel)inertia_panel_kernel<CPLX, 8>
+                       : nullptr;
+}
+
+static cudaLaunchConfig_t panel_config(int G, unsigned grid, size_t smem, cudaStream_t st, cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kPanThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = G;
+  attr->val.clusterDim.y = 1;
+  attr->val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// Clusters of G CTAs of the panel kernel that run at once (0: this shape does not fit), cached per
+// device and shape.
+template <bool CPLX>
+static int panel_clusters(int b, int G) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, int, int>, int> known;
+  const PanelShape s = panel_shape(b, CPLX, G);
+  PanelKernel kern = panel_kernel<CPLX>(s.chunks);
+  int dev = 0;
+  if (!kern || s.smem > 226 * 1024 || cudaGetDevice(&dev) != cudaSuccess) return 0;
+  std::lock_guard<std::mutex> lk(mu);
+  const auto key = std::make_tuple(dev, b, G);
+  auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  int nc = 0;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t cfg = panel_config(G, (unsigned)G, s.smem, nullptr, &attr);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&nc, kern, &cfg);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    nc = 0;
+  }
+  if (known.size() > 4096) known.clear();
+  known[key] = nc;
+  return nc;
+}
+
+// The cluster size for nsigma shifts, or 0 for one CTA per shift and one column per step
+// (inertia_kernel): the least estimated clocks per column of a fit to measured times.  Panel kernel:
+// the panel's chain (a division and an update, in one warp per column or through two barriers), the
+// rest of a round (barriers, row entry, triangle), the CTA's share of the updates at 76 clocks per
+// warp instruction and FP64 pipe; CTAs that share an SM share its pipes.  `sms` is what clusters of G
+// reach at one CTA per SM.  At b = 64 complex the measured times cross at about 110 shifts.
+template <bool CPLX>
+static int panel_cluster_size(int b, int nsigma, bool single_ok) {
+  static const int sms[5] = {152, 152, 144, 120, 112};
+  const double np = CPLX ? 2.0 : 1.0, ops = CPLX ? 4.0 : 2.0;
+  const double work = 0.5 * b * (b + 1.0) * np / 32.0 * ops * 19.0;  // all updates of one column
+  int best = -1;
+  double best_t = 0.0;
+  if (single_ok) {
+    const double div = np * 9.0 * 19.0 * ceil_div(b, 32);
+    const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(8, 227 * 1024 / (single_smem(b, CPLX) + 1024)));
+    const int waves = (int)ceil_div(nsigma, 152 * per_sm);
+    const double co = (double)ceil_div(std::min(nsigma, 152 * per_sm), 152);
+    best_t = waves * std::max(work + div + 2150.0 + 64.0 * ops, co * 1.1 * (work + div));
+    best = 0;
+  }
+  for (int G = 1, q = 0; G <= 16; G *= 2, ++q) {
+    const int nc = panel_clusters<CPLX>(b, G);
+    if (nc < 1) continue;
+    const int chunks = panel_shape(b, CPLX, G).chunks;
+    const int waves = (int)ceil_div(nsigma, nc);
+    const double co = (double)ceil_div((int64_t)std::min(nsigma, nc) * G, sms[q]);
+    const double upd = 1.2 * work / G, pan = chunks * (9.0 + 3.5 * ops) * 19.0 + 150.0;
+    const double chain = (chunks == 1 ? 1000.0 + 115.0 * ops : 1300.0 + 175.0 * ops) + 750.0;
+    const double t = waves * std::max((co > 1 ? 1.25 : 1.0) * (chain + upd), co * (upd + pan));
+    if (best < 0 || t < best_t) {
+      best = G;
+      best_t = t;
+    }
+  }
+  return best;
+}
+
+template <bool CPLX>
+static int launch_panel(int64_t n, int b, const void* band, int64_t ldab, int nsigma, const double* d_sigma,
+                        const unsigned long long* amax, int64_t* d_neg, double* d_piv, int G, cudaStream_t st) {
+  const PanelShape s = panel_shape(b, CPLX, G);
+  PanelKernel kern = panel_kernel<CPLX>(s.chunks);
+  PD_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
+  if (G > 8) PD_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t cfg = panel_config(G, (unsigned)nsigma * (unsigned)G, s.smem, st, &attr);
+  PD_CK(cudaLaunchKernelEx(&cfg, kern, n, b, (const double*)band, ldab, d_sigma, amax, d_neg, d_piv, s.nslot, s.rown,
+                           s.chunks));
+  count_launch();
+  return 0;
+}
+
+// Batched inertia with sigma already on the device; results into d_neg.  Async.  gwin (the window in
+// the workspace) serves only bands that no cluster's shared memory holds.
 int launch_inertia(int64_t n, int b, int cplx, const void* band, int64_t ldab, int nsigma,
                    const double* d_sigma, const unsigned long long* amax, int64_t* d_neg,
                    double* d_piv, char* gwin, size_t gwin_stride, cudaStream_t st) {
   if (nsigma <= 0) return 0;
-  size_t smem = inertia_smem_base(b, cplx) + (gwin ? 0 : window_bytes(b, cplx));
-  if (cplx) {
-    PD_CK(cudaFuncSetAttribute(inertia_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem));
-    inertia_kernel<true><<<nsigma, 256, smem, st>>>(n, b, (const double*)band, ldab, d_sigma, amax,
-                                                    d_neg, d_piv, gwin, gwin_stride);
-  } else {
-    PD_CK(cudaFuncSetAttribute(inertia_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem));
-    inertia_kernel<false><<<nsigma, 256, smem, st>>>(n, b, (const double*)band, ldab, d_sigma, amax,
-                                                     d_neg, d_piv, gwin, gwin_stride);
-  }
+  const bool single = window_in_smem(b, cplx);
+  const int G = cplx ? panel_cluster_size<true>(b, nsigma, single) : panel_cluster_size<false>(b, nsigma, single);
+  if (G > 0)
+    return cplx ? launch_panel<true>(n, b, band, ldab, nsigma, d_sigma, amax, d_neg, d_piv, G, st)
+                : launch_panel<false>(n, b, band, ldab, nsigma, d_sigma, amax, d_neg, d_piv, G, st);
+  const size_t smem = single ? single_smem(b, cplx) : inertia_smem_base(b, cplx);
+  auto kern = cplx ? inertia_kernel<true> : inertia_kernel<false>;
+  PD_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  kern<<<nsigma, 256, smem, st>>>(n, b, (const double*)band, ldab, d_sigma, amax, d_neg, d_piv,
+                                  single ? nullptr : gwin, gwin_stride);
   PD_CK_LAUNCH();
   return 0;
 }

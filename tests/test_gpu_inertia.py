@@ -83,3 +83,41 @@ def test_bisection_enclosures(device):
         glo, ghi = pk.gershgorin(to_dev(ab2, device))
         olo, ohi = oracle.gershgorin(ab2)
         assert (glo, ghi) == (olo, ohi), (glo - olo, ghi - ohi)
+
+
+# The panel kernel eliminates 8 columns per round on a cluster whose size depends on b and the number
+# of shifts: orders and bandwidths around multiples of 8, bands narrower than a panel, n <= b, and
+# shift counts that reach the largest cluster (1 shift), smaller ones and one CTA per shift.
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("n,b,nsig", [(7, 2, 1), (8, 8, 1), (9, 9, 40), (17, 16, 2), (63, 5, 1), (64, 24, 90),
+                                      (65, 25, 1), (130, 31, 60), (129, 33, 1), (143, 66, 1), (150, 57, 30),
+                                      (31, 70, 2), (200, 149, 1), (190, 129, 20), (210, 200, 1)])
+def test_panel_edges_bit_exact(device, n, b, nsig, cplx):
+    import paper_2012_00506_gb300 as pk
+    ab = synth.random_band(n, b, 900 + n + b, cplx)
+    lo, hi = oracle.gershgorin(ab)
+    sig = np.random.default_rng(n).uniform(lo, hi, nsig)
+    neg, piv = pk.inertia(to_dev(ab, device), sig, pivots=True)
+    piv = piv.cpu().numpy()
+    for i, s in enumerate(sig):
+        c, d = oracle.inertia(ab, s, return_pivots=True)
+        assert neg[i] == c
+        assert np.array_equal(piv[i], d)
+
+
+def test_panel_zero_pivots_and_nan(device):
+    """Exactly zero pivots (a diagonal band whose entries meet the shift, a band of zeros below the
+    diagonal) become -pivmin and count as negative; a NaN in the band is reported."""
+    import paper_2012_00506_gb300 as pk
+    for b in (3, 20):
+        ab = np.zeros((100, b + 1))
+        ab[:, 0] = np.arange(100) % 7 - 3.0
+        sig = [-3.0, 0.0, 0.5, 3.0]
+        neg, piv = pk.inertia(to_dev(ab, device), sig, pivots=True)
+        for i, s in enumerate(sig):
+            c, d = oracle.inertia(ab, s, return_pivots=True)
+            assert neg[i] == c and np.array_equal(piv[i].cpu().numpy(), d)
+        ab[50, 1] = np.nan
+        with pytest.raises(pk.PdeshepError) as e:
+            pk.inertia(to_dev(ab, device), sig)
+        assert e.value.status == 4
