@@ -9,24 +9,28 @@
 // the pivots equal those of LAPACK's gbtrf (first maximum of |Re|+|Im|).
 // The U factor fills to 2b superdiagonals (2bt tiles).
 //
-// factor_kernel: one thread block per shifted system (the L2 level of the
-//   paper's parallelism is the batch dimension).  Per block column K: the
-//   panel ((bt+1)T x T) is factored in shared memory (warp-shuffle pivot
-//   search, row swaps, rank-1 updates); the panel permutation is gathered
-//   into each trailing block column on load; the top tile is multiplied by
-//   the inverted unit-lower diagonal block and the tiles below get the
-//   T-deep Schur update.  The inverses of the diagonal blocks are stored so
-//   that every solve step is a tile product.
+// factor_kernel: a thread-block cluster per shifted system (the L2 level of the
+//   paper's parallelism is the batch dimension; the cluster is the L3 level,
+//   inside one factorization).  Per block column K: the panel ((bt+1)T x T) is
+//   factored in registers; the panel permutation is gathered into each trailing
+//   block column on load; the top tile is multiplied by the inverted unit-lower
+//   diagonal block and the tiles below get the T-deep Schur update.
+// diag_inverse_kernel: the inverses of the diagonal blocks, so that every solve
+//   step is a tile product.
 // solve kernels: one thread block per (system, 32-column block of right-hand
 //   sides); forward L sweep then backward U sweep (trans = 0), or U^H then
 //   L^H and the inverse permutation (trans = 1, the conjugate node conj(z)
 //   of a Hermitian band).  Factor tiles stream from L2/HBM through shared
 //   memory; each is reused by the 32 right-hand sides of the block.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <type_traits>
 #include <vector>
 
 #include "band_lu.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace pdeshep {
 
@@ -93,249 +97,668 @@ __global__ void __launch_bounds__(kThreads) init_factor_kernel(FactorGeom g, int
   }
 }
 
-// (value, index) of the warp's largest value, the lowest index on ties, in every lane
+// ---------------------------------------------------------------------------
+// factorization.  The chain of a block column is its panel: 32 columns of pivot
+// search, row interchange and elimination, in which the next column waits for the
+// last.  One CTA per system spent 88 us (b = 64) to 150 us (b = 128) per block
+// column on it and on what followed it (serial inverses of the diagonal blocks,
+// updates through shared memory), with all but a few SMs idle when a call has few
+// systems.  Here
+//  * a cluster of G CTAs shares a system: CTA 0 updates the next block column and
+//    factors it while the others apply the current panel to the block columns
+//    right of it (look-ahead of one); one cluster barrier per block column.  In
+//    FP64, where the updates of a block column take longer than a barrier, its
+//    columns are spread over the cluster as well (`spread`, a second barrier);
+//  * the panel lives in registers, and a column takes one barrier: each warp's
+//    candidate pivot (integer warp reductions on the bits of |re| + |im|) writes its
+//    row and its reciprocal beside its value, so after the barrier every thread has
+//    all it needs.  Rows do not move: each carries its logical index.  complex64: a
+//    thread per row (panel_lu_rows); complex128, where the FP64 pipes of all four
+//    quadrants are needed, a row in four threads (panel_lu_parts);
+//  * a warp updates NC columns on its own (gathered through the permutation,
+//    rows in registers), without barriers;
+//  * the inverses of the diagonal blocks that only the solves need are left to
+//    diag_inverse_kernel, parallel over blocks and systems.
+// Every entry sees the operations of the one-CTA form in the same order
+// (complex64 factors keep their bits; in FP64 the top block comes from forward
+// substitution instead of the product with the inverse).
+// Measured, us per block column against one CTA with a panel in shared memory: complex64 b = 64, 8
+// systems 24.5 against 88, 64 systems 25 against 89, 256 systems 54 (two waves of 89 before); b = 128, 16
+// systems 30 against 151; complex128 b = 32, 8 systems 145 against 454, b = 128, 2 systems 282 against
+// 1558.  What remains (b = 64) is the panel: 32 columns of about 1200 clocks, each a search (300), a
+// reciprocal (two dependent divisions, 170), two barriers and the row's updates (440).
+// ---------------------------------------------------------------------------
+// a b with each rounding spelled out, so that the factors' bits do not depend on how the compiler
+// contracts the expression: (a.x b.x - [a.y b.y], a.x b.y + [a.y b.x]), products in brackets rounded.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+template <typename C>
+__device__ __forceinline__ C cmul_rn(C a, C b) {
+  return cmk<C>(fma(a.x, b.x, -mul_rn(a.y, b.y)), fma(a.x, b.y, mul_rn(a.y, b.x)));
+}
+
+// order-preserving integer key of v >= 0 (0 for NaN, which is never a pivot; > 1 if v > 0)
+__device__ __forceinline__ unsigned long long pivot_key(float v) {
+  return v == v ? (unsigned long long)__float_as_uint(v) + 1 : 0ull;
+}
+__device__ __forceinline__ unsigned long long pivot_key(double v) {
+  return v == v ? (unsigned long long)__double_as_longlong(v) + 1 : 0ull;
+}
 template <typename R>
-__device__ __forceinline__ void warp_argmax(R& best, int& idx) {
-  for (int o = 16; o > 0; o >>= 1) {
-    const R ob = __shfl_xor_sync(0xffffffffu, best, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-    if (ob > best || (ob == best && oi < idx)) {
-      best = ob;
-      idx = oi;
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k) {
+  if constexpr (sizeof(R) == 4) return __reduce_max_sync(0xffffffffu, (unsigned)k);
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32));
+  const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32) == hi ? (unsigned)k : 0u);
+  return ((unsigned long long)hi << 32) | lo;
+}
+__device__ __forceinline__ float2 shfl_c(float2 v, int src) {
+  return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+__device__ __forceinline__ double2 shfl_c(double2 v, int src) {
+  return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+
+// One warp's candidate for the pivot of a column: its row (columns from the current one on), the
+// reciprocal of its entry, its key and logical row.
+template <typename C>
+struct alignas(16) PivotSlot {
+  C row[kTile];
+  C inv;
+  unsigned long long key;
+  int log, pad;
+};
+
+constexpr int kRowsMax = 256;  // panel rows that panel_lu_rows takes
+
+// shared memory of one CTA
+template <typename C>
+struct FactorSmem {
+  C* Pan;   // [T][ldp] panel: packed L\U of the top block and L below, logical row r at perm[r]
+            // (panel_lu_rows: multipliers only) or at r (panel_lu_parts)
+  C* Li;    // [T][T+1] rows of the inverse of the unit lower top block (complex64)
+  C* top;   // [warps][2][NC][T] top rows of a warp's columns
+  int* perm;            // [Pmax]
+  PivotSlot<C>* slot;   // panel_lu_parts: [2][warps]
+  C* U;                 // panel_lu_rows: [T][T+2] pivot rows, each from its column on
+  C* col;               // ... [2][kRowsMax] the rows' entries of the current column
+  unsigned* key;        // ... [2][kRowsMax] and their keys
+  int* log;             // ... [kRowsMax] logical rows
+  int* win;             // ... [T] pivot row of each column
+};
+
+template <typename C, bool ROWS>
+__host__ __device__ inline size_t factor_cluster_smem(int Pmax, int nw, int nc) {
+  const size_t base = sizeof(C) * ((size_t)kTile * (Pmax + 1) + (size_t)kTile * (kTile + 1) + (size_t)nw * 2 * nc * kTile) +
+                      sizeof(int) * Pmax + 64;
+  return base + (ROWS ? sizeof(C) * (kTile * (kTile + 2) + 2 * kRowsMax) + sizeof(int) * (3 * kRowsMax + kTile)
+                      : sizeof(PivotSlot<C>) * 2 * nw);
+}
+
+// complex64: LU with partial pivoting of the panel of block column K (rows K .. K+nbb), thread r holding
+// panel row r.  The row's registers move down one place per column (w[0] is the current column), which
+// the elimination does for free by its choice of destination and which keeps the loop rolled: four
+// stages of 8 columns, their widths 32, 24, 16 and 8 (unrolled over 32 columns the code would not stay
+// in the instruction cache).  Per column, every row's entry of that column is in shared memory; each warp
+// searches all of them and takes the reciprocal itself, while the pivot row's thread writes its row
+// out: one round of warp reductions and two short barriers (a search per warp and then one among the
+// warps took as long at b = 64 and 3% longer at b = 128).  Multipliers go to sm.Pan at the row's own place, pivot rows to
+// sm.U.  The pivot of a column is the largest |re| + |im|, the lowest logical row on ties.
+// A warp of its own (unit_lower_rows) follows with the inverse of the unit lower top block, whose row c
+// needs no more than the pivot row of column c.
+// The steps after which that warp may go on; each has a named barrier of its own (2 ..), on which the
+// panel's warps only arrive, so that it may lag behind them.
+constexpr unsigned kHelperSteps = 1u << 7 | 1u << 15 | 1u << 19 | 1u << 23 | 1u << 25 | 1u << 27 | 1u << 29 | 1u << 30 |
+                                  1u << 31;
+__device__ __forceinline__ int helper_barrier(int c) { return 2 + __popc(kHelperSteps & ((1u << c) - 1)); }
+__device__ __forceinline__ void helper_arrive(int c, int nthreads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(helper_barrier(c)), "r"(nthreads) : "memory");
+}
+__device__ __forceinline__ void panel_barrier(int nthreads) {
+  asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
+}
+// order-preserving key of a candidate pivot (0: a row that is done, or NaN; > 1: a positive pivot)
+__device__ __forceinline__ unsigned candidate_key(float2 a, bool active) {
+  const float v = cabs1(a);
+  return active && v == v ? __float_as_uint(v) + 1 : 0u;
+}
+constexpr int kURow = kTile + 2;  // a pivot row in sm.U, from its column on: 16-byte words
+// NQ: rows / 32, at most
+template <int W, int NQ>
+__device__ __forceinline__ void panel_stage(float2 (&w)[kTile], int& mylog, int nwp, int ldp,
+                                            const FactorSmem<float2>& sm, int64_t k0, int64_t n, int* sh_status,
+                                            int32_t* ipiv) {
+  constexpr int T = kTile;
+  const int tid = threadIdx.x, lane = tid & 31;
+#pragma unroll 1
+  for (int c = T - W; c < T - W + 8; ++c) {
+    const unsigned* keys = sm.key + (c & 1) * kRowsMax;
+    panel_barrier(nwp * 32);
+    unsigned k[NQ], key = 0;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) k[q] = keys[q * 32 + lane];  // (0 past the last row)
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) key = max(key, k[q]);
+    const unsigned best = __reduce_max_sync(0xffffffffu, key);
+    unsigned hits = 0;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) hits |= (k[q] == best ? 1u : 0u) << q;
+    int r = 32 * (__ffs(hits) - 1) + lane;
+    unsigned who = __ballot_sync(0xffffffffu, hits != 0);
+    if (__ballot_sync(0xffffffffu, (hits & (hits - 1)) != 0) | (who & (who - 1))) {  // equal keys: the lowest logical row
+      int lg = 0x7fffffff;
+#pragma unroll 1
+      for (int q = 0; q < nwp; ++q) {
+        const int l = sm.log[q * 32 + lane];
+        if (keys[q * 32 + lane] == best && l >= c && l < lg) {
+          lg = l;
+          r = q * 32 + lane;
+        }
+      }
+      who = __ballot_sync(0xffffffffu, lg == __reduce_min_sync(0xffffffffu, lg));
+    }
+    r = __shfl_sync(0xffffffffu, r, __ffs(who) - 1);  // the pivot row (nothing but NaN: row c, no interchange)
+    if (tid == r) {
+#pragma unroll
+      for (int q = 0; q < W; q += 2)
+        *(float4*)&sm.U[c * kURow + q] = make_float4(w[q].x, w[q].y, w[q + 1].x, w[q + 1].y);
+      sm.win[c] = r;
+    }
+    const float2 a = sm.col[(c & 1) * kRowsMax + r];
+    const int p = sm.log[r];
+    const bool ok = best > 1;  // a positive pivot
+    // 1 / a with Smith's scaling (crecip), the parts' divisions in lanes 0 and 1
+    const bool big = fabsf(a.x) >= fabsf(a.y);
+    const float rr = (big ? a.y : a.x) / (big ? a.x : a.y);
+    const float den = big ? fmaf(a.y, rr, a.x) : fmaf(a.x, rr, a.y);
+    const float q2 = (lane == 0 ? (big ? 1.f : rr) : (big ? -rr : -1.f)) / den;
+    const float2 inv = make_float2(__shfl_sync(0xffffffffu, q2, 0), __shfl_sync(0xffffffffu, q2, 1));
+    const int nlog = mylog == p ? c : (mylog == c ? p : mylog);
+    const int nx = ((c + 1) & 1) * kRowsMax + tid;
+    panel_barrier(nwp * 32);
+    const float2* u = sm.U + c * kURow;
+    if (ok) {
+      const float2 l = cmul_rn(w[0], inv);
+      w[0] = w[1];
+      cfms(w[0], l, u[1]);
+      sm.key[nx] = candidate_key(w[0], nlog > c);
+      sm.col[nx] = w[0];
+      sm.Pan[tid + c * ldp] = l;
+#pragma unroll
+      for (int q = 2; q < W; q += 2) {
+        const float4 v = *(const float4*)&u[q];
+        w[q - 1] = w[q];
+        cfms(w[q - 1], l, make_float2(v.x, v.y));
+        w[q] = w[q + 1 < W ? q + 1 : q];
+        cfms(w[q], l, make_float2(v.z, v.w));
+      }
+    } else {
+      sm.Pan[tid + c * ldp] = w[0];
+#pragma unroll
+      for (int q = 0; q < W - 1; ++q) w[q] = w[q + 1];
+      sm.key[nx] = candidate_key(w[0], nlog > c);
+      sm.col[nx] = w[0];
+      if (tid == 0 && *sh_status == 0) *sh_status = (int)(k0 + c + 1);
+    }
+    if (nlog != mylog) sm.log[tid] = nlog;
+    mylog = nlog;
+    if ((kHelperSteps >> c) & 1u) helper_arrive(c, nwp * 32 + 32);
+    if (ipiv && tid == 0 && k0 + c < n) ipiv[k0 + c] = (int32_t)(k0 + p);
+  }
+}
+
+// Rows of the inverse X of the unit lower top block, those up to column c once the panel's warps have
+// passed step c of kHelperSteps: lane = column, X(c, j) = -sum_{k=j}^{c-1} L(c, k) X(k, j), terms in
+// ascending k.
+__device__ __forceinline__ void unit_lower_rows(int nwp, int ldp, const FactorSmem<float2>& sm) {
+  constexpr int T = kTile;
+  const int j = threadIdx.x & 31;
+  int c = 0;
+  for (int e = 0; e < T; ++e) {
+    if (!((kHelperSteps >> e) & 1u)) continue;
+    asm volatile("bar.sync %0, %1;" ::"r"(helper_barrier(e)), "r"(nwp * 32 + 32) : "memory");
+    for (; c <= e; ++c) {
+      const float2* L = sm.Pan + sm.win[c];
+      float2 s = make_float2(0.f, 0.f);
+#pragma unroll 8
+      for (int k = 0; k < c; ++k) {
+        const float2 a = L[k * ldp], x = sm.Li[k * (T + 1) + j];
+        if (k >= j) cfma(s, a, x);
+      }
+      sm.Li[c * (T + 1) + j] = j == c ? make_float2(1.f, 0.f) : j < c ? make_float2(-s.x, -s.y) : make_float2(0.f, 0.f);
+      __syncwarp();
     }
   }
 }
 
-// ---------------------------------------------------------------------------
-// factorization: one thread block per system
-// ---------------------------------------------------------------------------
-template <typename C>
-__global__ void __launch_bounds__(kThreads) factor_kernel(FactorGeom g, const SysDesc* sys,
-                                                         char* arena, int* status, int32_t* ipiv) {
-  using R = typename real_of<C>::type;
-  extern __shared__ __align__(16) char smem[];
-  const int T = kTile;
-  const int bt = g.bt;
-  const int Pmax = (bt + 1) * T;
-  const int ldp = Pmax + 1;
-  C* Pan = (C*)smem;
-  C* Cb = Pan + (size_t)ldp * T;
-  C* Li = Cb + (size_t)ldp * T;
-  C* Ui = Li + T * T;
-  int* perm = (int*)(Ui + T * T);
-  int* pos = perm + Pmax;  // [2][Pmax]
-  __shared__ R wbest[64];
-  __shared__ int widx[64];
-  __shared__ int sh_status;
-
-  const int sidx = blockIdx.x;
-  const SysDesc d = sys[sidx];
-  FactorPtr<C> f = factor_ptr<C>(g, arena + d.factor_off);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) sh_status = 0;
-
-  for (int K = 0; K < g.Nb; ++K) {
-    const int nbb = min(bt, g.Nb - 1 - K);
-    const int nbr = min(2 * bt, g.Nb - 1 - K);
-    const int P = (nbb + 1) * T;
-    // load panel tiles (K+q, K)
-    for (int e = tid; e < P * T; e += blockDim.x) {
-      const int q = (e / (T * T)), w = e % (T * T);
-      const int r = w % T, c = w / T;
-      const C* tile = f.tiles + g.tile_index(K + q, K) * g.tile_elems;
-      Pan[q * T + r + c * ldp] = tile[w];
-    }
-    for (int r = tid; r < P; r += blockDim.x) {
-      perm[r] = r;
-      pos[r] = r;
-    }
-    __syncthreads();
-    // panel LU with partial pivoting, one CTA barrier per column.  Rows are addressed through
-    // pos[] (logical -> physical row), so an interchange moves no data; a thread owns logical rows
-    // tid, tid + blockDim.x, ...: it eliminates them and, in the same phase, takes their part of the
-    // next column's pivot search (warp maxima in wbest/widx; every thread then reduces the warp
-    // maxima itself).  The pivot is the largest |re| + |im| with the lowest row on ties, and every
-    // element sees the same operations in the same order as with physical interchanges.
-    {
-      const int nw = blockDim.x >> 5;
-      // the pivot search of column 0
-      {
-        R best = R(-1);
-        int idx = 0x7fffffff;
-        for (int r = tid; r < P; r += blockDim.x) {
-          const R v = cabs1(Pan[r]);
-          if (v > best) {
-            best = v;
-            idx = r;
-          }
-        }
-        warp_argmax(best, idx);
-        if (lane == 0) {
-          wbest[warp] = best;
-          widx[warp] = idx;
-        }
-      }
-      __syncthreads();
-      for (int c = 0; c < T; ++c) {
-        const int cur = c & 1;
-        const int* posc = pos + cur * Pmax;
-        int* posn = pos + (cur ^ 1) * Pmax;
-        R best = R(-1);
-        int p = 0x7fffffff;
-        for (int w = 0; w < nw; ++w) {
-          const R ob = wbest[cur * 32 + w];
-          const int oi = widx[cur * 32 + w];
-          if (ob > best || (ob == best && oi < p)) {
-            best = ob;
-            p = oi;
-          }
-        }
-        const int pp = posc[p], pc = posc[c];  // physical rows of the pivot and of logical row c
-        if (tid == 0) {
-          if (p != c) {
-            int tp = perm[c];
-            perm[c] = perm[p];
-            perm[p] = tp;
-          }
-          const int64_t k = (int64_t)K * T + c;
-          if (ipiv && k < g.n) ipiv[(int64_t)sidx * g.n + k] = (int32_t)((int64_t)K * T + p);
-          if (!(best > R(0)) && sh_status == 0) sh_status = (int)(k + 1);
-        }
-        const bool ok = best > R(0);
-        const C inv = ok ? crecip(Pan[pp + c * ldp]) : cmk<C>(0, 0);
-        R nb = R(-1);
-        int ni = 0x7fffffff;
-        for (int r = tid; r < P; r += blockDim.x) {
-          const int phys = r == c ? pp : (r == p ? pc : posc[r]);
-          posn[r] = phys;
-          if (r <= c) continue;
-          if (ok) {
-            const C l = cmul(Pan[phys + c * ldp], inv);
-            Pan[phys + c * ldp] = l;
-            for (int j = c + 1; j < T; ++j) cfms(Pan[phys + j * ldp], l, Pan[pp + j * ldp]);
-          }
-          if (c + 1 < T) {
-            const R v = cabs1(Pan[phys + (c + 1) * ldp]);
-            if (v > nb) {
-              nb = v;
-              ni = r;
-            }
-          }
-        }
-        warp_argmax(nb, ni);
-        if (lane == 0) {
-          wbest[(cur ^ 1) * 32 + warp] = nb;
-          widx[(cur ^ 1) * 32 + warp] = ni;
-        }
-        __syncthreads();
-      }
-      // rows back in logical order (pos of column T, an even count: buffer 0)
-      for (int e = tid; e < P * T; e += blockDim.x) {
-        const int r = e % P, cc = e / P;
-        Cb[r + cc * ldp] = Pan[pos[r] + cc * ldp];
-      }
-      __syncthreads();
-      C* tmp = Pan;
-      Pan = Cb;
-      Cb = tmp;
-    }
-    // write back the panel (L multipliers and the packed diagonal block)
-    for (int e = tid; e < P * T; e += blockDim.x) {
-      const int q = (e / (T * T)), w = e % (T * T);
-      const int r = w % T, c = w / T;
-      C* tile = f.tiles + g.tile_index(K + q, K) * g.tile_elems;
-      tile[w] = Pan[q * T + r + c * ldp];
-    }
-    {
-      int16_t* pg = f.perm + (int64_t)K * Pmax;
-      for (int r = tid; r < Pmax; r += blockDim.x) pg[r] = (int16_t)(r < P ? perm[r] : r);
-    }
-    // inverses of the unit-lower and upper diagonal blocks
-    if (tid < T) {
-      const int j = tid;
-      for (int i = 0; i < T; ++i) Li[i + j * T] = cmk<C>(i == j ? R(1) : R(0), R(0));
-      for (int i = j + 1; i < T; ++i) {
-        C s = cmk<C>(0, 0);
-        for (int k = j; k < i; ++k) cfma(s, Pan[i + k * ldp], Li[k + j * T]);
-        Li[i + j * T] = cmk<C>(-s.x, -s.y);
-      }
-    } else if (tid >= 32 && tid < 32 + T) {
-      const int j = tid - 32;
-      for (int i = 0; i < T; ++i) Ui[i + j * T] = cmk<C>(0, 0);
-      Ui[j + j * T] = crecip(Pan[j + j * ldp]);
-      for (int i = j - 1; i >= 0; --i) {
-        C s = cmk<C>(0, 0);
-        for (int k = i + 1; k <= j; ++k) cfma(s, Pan[i + k * ldp], Ui[k + j * T]);
-        const C ri = crecip(Pan[i + i * ldp]);
-        Ui[i + j * T] = cmk<C>(-(s.x * ri.x - s.y * ri.y), -(s.x * ri.y + s.y * ri.x));
-      }
-    }
-    __syncthreads();
-    {
-      C* li = f.inv + (int64_t)(2 * K) * g.tile_elems;
-      C* ui = f.inv + (int64_t)(2 * K + 1) * g.tile_elems;
-      for (int e = tid; e < T * T; e += blockDim.x) {
-        li[e] = Li[e];
-        ui[e] = Ui[e];
-      }
-    }
-    // trailing block columns K+1 .. K+nbr: warp w owns columns w, w+8, w+16, w+24 of every block
-    // column through the gather (rows in panel order), U(K, Jc) = Linv Cb[0:T], the rows below
-    // (Cb[T:P] -= L U) and the scatter, so the warps need no barrier between them
-    for (int jb = 1; jb <= nbr; ++jb) {
-      const int Jc = K + jb;
+template <int NQ>
+__device__ void panel_lu_rows(const FactorGeom& g, const FactorPtr<float2>& f, int K, const FactorSmem<float2>& sm,
+                              int* sh_status, int32_t* ipiv) {
+  constexpr int T = kTile;
+  const int tid = threadIdx.x;
+  const int nbb = min(g.bt, g.Nb - 1 - K);
+  const int P = (nbb + 1) * T, Pmax = (g.bt + 1) * T, ldp = Pmax + 1, nwp = P / 32;
+  if (tid < P) {
+    float2 w[T];
+    const float2* src = f.tiles + g.tile_index(K + tid / T, K) * g.tile_elems + (tid & (T - 1));
 #pragma unroll
-      for (int jj = 0; jj < 4; ++jj) {
-        const int c = warp + 8 * jj;
-        for (int r = lane; r < P; r += 32) {
-          const int sr = perm[r];
-          const int q = sr / T, rr = sr % T;
-          const C* tile = f.tiles + g.tile_index(K + q, Jc) * g.tile_elems;
-          Cb[r + c * ldp] = tile[rr + c * T];
-        }
-      }
-      __syncwarp();
-      // top block: U(K, Jc) = Linv * Cb[0:T]
-      C acc[4];
-#pragma unroll
-      for (int jj = 0; jj < 4; ++jj) acc[jj] = cmk<C>(0, 0);
-      for (int k = 0; k < T; ++k) {
-        const C a = Li[lane + k * T];
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) cfma(acc[jj], a, Cb[k + (warp + 8 * jj) * ldp]);
-      }
-      __syncwarp();
-#pragma unroll
-      for (int jj = 0; jj < 4; ++jj) Cb[lane + (warp + 8 * jj) * ldp] = acc[jj];
-      __syncwarp();
-      // rows below: Cb[T:P] -= L(panel rows T:P) * U(K, Jc)
-      for (int q = 1; q <= nbb; ++q) {
-        const int r = q * T + lane;
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) acc[jj] = Cb[r + (warp + 8 * jj) * ldp];
-        for (int k = 0; k < T; ++k) {
-          const C a = Pan[r + k * ldp];
-#pragma unroll
-          for (int jj = 0; jj < 4; ++jj) cfms(acc[jj], a, Cb[k + (warp + 8 * jj) * ldp]);
-        }
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) Cb[r + (warp + 8 * jj) * ldp] = acc[jj];
-      }
-      __syncwarp();
-#pragma unroll
-      for (int jj = 0; jj < 4; ++jj) {
-        const int c = warp + 8 * jj;
-        for (int r = lane; r < P; r += 32) {
-          const int q = r / T, rr = r % T;
-          C* tile = f.tiles + g.tile_index(K + q, Jc) * g.tile_elems;
-          tile[rr + c * T] = Cb[r + c * ldp];
-        }
-      }
-      __syncwarp();
-    }
-    __syncthreads();  // block column K+1 (the next panel) and the tiles below are written
+    for (int i = 0; i < T; ++i) w[i] = src[i * T];
+    int mylog = tid;
+    sm.log[tid] = tid;
+    sm.col[tid] = w[0];
+    sm.key[tid] = candidate_key(w[0], true);
+    for (int q = nwp; q < NQ; ++q)  // no rows here
+      if (tid < 32) sm.key[q * 32 + tid] = sm.key[kRowsMax + q * 32 + tid] = 0;
+    const int64_t k0 = (int64_t)K * T;
+    panel_stage<32, NQ>(w, mylog, nwp, ldp, sm, k0, g.n, sh_status, ipiv);
+    panel_stage<24, NQ>(w, mylog, nwp, ldp, sm, k0, g.n, sh_status, ipiv);
+    panel_stage<16, NQ>(w, mylog, nwp, ldp, sm, k0, g.n, sh_status, ipiv);
+    panel_stage<8, NQ>(w, mylog, nwp, ldp, sm, k0, g.n, sh_status, ipiv);
+    sm.perm[mylog] = tid;
+  } else if (tid < P + 32) {
+    unit_lower_rows(nwp, ldp, sm);
   }
-  if (tid == 0) status[sidx] = sh_status;
+  __syncthreads();
+}
+// ... and its results to global memory (L\U of the top block, L below, in logical row order; the inverse of
+// the unit lower block; the permutation), with every thread of the CTA
+__device__ void store_panel_rows(const FactorGeom& g, const FactorPtr<float2>& f, int K,
+                                 const FactorSmem<float2>& sm) {
+  constexpr int T = kTile;
+  const int nbb = min(g.bt, g.Nb - 1 - K);
+  const int P = (nbb + 1) * T, Pmax = (g.bt + 1) * T, ldp = Pmax + 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  float2* li = f.inv + (int64_t)(2 * K) * g.tile_elems + lane;
+  for (int c = warp; c < T; c += nw) li[c * T] = sm.Li[lane * (T + 1) + c];
+  for (int q = 0; q <= nbb; ++q) {
+    const float2* L = sm.Pan + sm.perm[q * T + lane];
+    float2* dst = f.tiles + g.tile_index(K + q, K) * g.tile_elems + lane;
+#pragma unroll 4
+    for (int c = warp; c < T; c += nw)
+      dst[c * T] = q == 0 && lane <= c ? sm.U[lane * kURow + c - lane] : L[c * ldp];
+  }
+  int16_t* pg = f.perm + (int64_t)K * Pmax;
+  for (int e = threadIdx.x; e < Pmax; e += blockDim.x) pg[e] = (int16_t)(e < P ? sm.perm[e] : e);
+}
+
+// The same with a row in PARTS threads (columns i PARTS + part): complex128, and complex64 panels of
+// more than kRowsMax rows.  Results in sm.Pan (logical row order) / sm.perm and in global memory.
+template <typename C, int PARTS>
+__device__ void panel_lu_parts(const FactorGeom& g, const FactorPtr<C>& f, int K, const FactorSmem<C>& sm, int* sh_status,
+                         int32_t* ipiv) {
+  using R = typename real_of<C>::type;
+  constexpr int T = kTile, NI = T / PARTS, RPW = 32 / PARTS;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nbb = min(g.bt, g.Nb - 1 - K);
+  const int P = (nbb + 1) * T, Pmax = (g.bt + 1) * T, ldp = Pmax + 1;
+  const int nwp = (P + RPW - 1) / RPW;  // warps that hold rows
+  const int part = lane / RPW, r = warp * RPW + (lane & (RPW - 1));
+  const bool has = r < P;
+  C w[NI];
+#pragma unroll
+  for (int i = 0; i < NI; ++i)
+    w[i] = has ? f.tiles[g.tile_index(K + r / T, K) * g.tile_elems + (r & (T - 1)) + (i * PARTS + part) * T]
+               : cmk<C>(0, 0);
+  int mylog = has ? r : 0x7fffffff;
+  int par = 0;
+#pragma unroll
+  for (int i = 0; i < NI; ++i) {
+#pragma unroll 1
+    for (int pc = 0; pc < PARTS; ++pc, par ^= 1) {
+      const int c = i * PARTS + pc;
+      PivotSlot<C>* slots = sm.slot + par * (blockDim.x >> 5);
+      if (warp < nwp) {
+        const unsigned long long key = (part == pc && has && mylog >= c) ? pivot_key(cabs1(w[i])) : 0ull;
+        const unsigned long long m = warp_max_key<R>(key);
+        const int lg = __reduce_min_sync(0xffffffffu, key == m && key > 0 ? mylog : 0x7fffffff);
+        PivotSlot<C>& sl = slots[warp];
+        if (m > 0 && mylog == lg) {
+#pragma unroll
+          for (int q = i; q < NI; ++q) sl.row[q * PARTS + part] = w[q];
+        }
+        {
+          // reciprocal of the candidate (Smith's form), its parts' divisions in two lanes at once
+          const unsigned at = __ballot_sync(0xffffffffu, m > 0 && mylog == lg && part == pc);
+          const C a = shfl_c(w[i], at ? __ffs(at) - 1 : 0);
+          const bool big = fabs(a.x) >= fabs(a.y);
+          const R r0 = (big ? a.y : a.x) / (big ? a.x : a.y);
+          const R den = big ? a.x + a.y * r0 : a.x * r0 + a.y;
+          const R q = (lane == 0 ? (big ? R(1) : r0) : (big ? -r0 : R(-1))) / den;
+          if (lane < 2) ((R*)&sl.inv)[lane] = m > 1 ? q : R(0);
+        }
+        if (lane == 0) {
+          sl.key = m;
+          sl.log = lg;
+        }
+      }
+      __syncthreads();
+      if (warp < nwp) {
+        const unsigned long long kq = lane < nwp ? slots[lane].key : 0ull;
+        const int lq = lane < nwp ? slots[lane].log : 0x7fffffff;
+        const unsigned long long m = warp_max_key<R>(kq);
+        int p = __reduce_min_sync(0xffffffffu, kq == m && m > 0 ? lq : 0x7fffffff);
+        const unsigned who = __ballot_sync(0xffffffffu, kq == m && lq == p);
+        const bool ok = m > 1;  // a positive pivot
+        if (m == 0) p = c;      // nothing but NaN: no interchange
+        if (tid == 0) {
+          const int64_t k = (int64_t)K * T + c;
+          if (ipiv && k < g.n) ipiv[k] = (int32_t)((int64_t)K * T + p);
+          if (!ok && *sh_status == 0) *sh_status = (int)(k + 1);
+        }
+        if (ok) {
+          const PivotSlot<C>& sl = slots[__ffs(who) - 1];
+          C l = cmul_rn(w[i], sl.inv);
+          l = shfl_c(l, pc * RPW + (lane & (RPW - 1)));
+          if (has && mylog >= c && mylog != p) {
+            if (part == pc)
+              w[i] = l;
+            else if (part > pc)
+              cfms(w[i], l, sl.row[i * PARTS + part]);
+#pragma unroll
+            for (int q = i + 1; q < NI; ++q) cfms(w[q], l, sl.row[q * PARTS + part]);
+          }
+        }
+        mylog = mylog == p ? c : (mylog == c ? p : mylog);
+      }
+    }
+  }
+  if (has) {
+#pragma unroll
+    for (int i = 0; i < NI; ++i) sm.Pan[mylog + (i * PARTS + part) * ldp] = w[i];
+    if (part == 0) sm.perm[mylog] = r;
+  }
+  __syncthreads();
+  for (int e = tid; e < P * T; e += blockDim.x) {
+    const int q = e / (T * T), x = e % (T * T);
+    f.tiles[g.tile_index(K + q, K) * g.tile_elems + x] = sm.Pan[q * T + x % T + (x / T) * ldp];
+  }
+  int16_t* pg = f.perm + (int64_t)K * Pmax;
+  for (int e = tid; e < Pmax; e += blockDim.x) pg[e] = (int16_t)(e < P ? sm.perm[e] : e);
+}
+
+// Inverse of the panel's unit lower top block into sm.Li and global memory: lane = row, a warp takes
+// 4 columns at a time; X(i, j) = -sum_{k=j}^{i-1} L(i, k) X(k, j), terms in ascending k, each X(k, j)
+// passed on by a shuffle once it is final.
+template <typename C>
+__device__ void unit_lower_inverse(const FactorGeom& g, const FactorPtr<C>& f, int K, const FactorSmem<C>& sm) {
+  using R = typename real_of<C>::type;
+  constexpr int T = kTile;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int ldp = (g.bt + 1) * T + 1;
+  const C* L = sm.Pan + lane;
+  C* out = f.inv + (int64_t)(2 * K) * g.tile_elems;
+  for (int j0 = 4 * warp; j0 < T; j0 += 4 * nw) {
+    C s[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s[q] = cmk<C>(0, 0);
+#pragma unroll 4
+    for (int k = 0; k < T - 1; ++k) {
+      const C a = L[k * ldp];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        C x = shfl_c(s[q], k);
+        x = k == j0 + q ? cmk<C>(R(1), R(0)) : cmk<C>(-x.x, -x.y);
+        if (lane > k && k >= j0 + q) cfma(s[q], a, x);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int j = j0 + q;
+      const C x = lane == j ? cmk<C>(R(1), R(0)) : (lane > j ? cmk<C>(-s[q].x, -s[q].y) : cmk<C>(0, 0));
+      sm.Li[lane * (T + 1) + j] = x;
+      out[lane + j * T] = x;
+    }
+  }
+}
+
+// Panel K applied to columns c0 .. c0+NC-1 of block column Jc by one warp: rows gathered through the
+// panel's permutation, U(K, Jc) = L^{-1} (top rows), then rows below -= L U.
+template <typename C, int NC, bool ROWS>
+__device__ __forceinline__ void update_columns(const FactorGeom& g, const FactorPtr<C>& f, int K, int Jc, int c0,
+                                               const FactorSmem<C>& sm) {
+  constexpr int T = kTile;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nbb = min(g.bt, g.Nb - 1 - K);
+  const int ldp = (g.bt + 1) * T + 1;
+  C* top = sm.top + (size_t)warp * 2 * NC * T;  // the top block in use
+  C* raw = top + NC * T;                        // the top rows before the permutation
+  auto at = [&](int row, int c) -> C* {  // window row `row` of the block column
+    return f.tiles + g.tile_index(K + (row >> 5), Jc) * g.tile_elems + (row & 31) + c * T;
+  };
+  // A row below the top block is either where it was or an old top row (interchanges bring rows up
+  // only as pivots), so only old top rows are read after their place is written: from `raw`.
+  auto request = [&](int q, int sr, C (&v)[NC]) {
+    if (sr >= T) {
+#pragma unroll
+      for (int j = 0; j < NC; ++j) v[j] = *at(sr, c0 + j);
+    }
+  };
+  auto complete = [&](int sr, C (&v)[NC]) {
+    if (sr < T) {
+#pragma unroll
+      for (int j = 0; j < NC; ++j) v[j] = raw[j * T + sr];
+    }
+  };
+  C x[NC], nx[NC];
+  const int s0 = sm.perm[lane];
+  int s1 = nbb > 0 ? sm.perm[T + lane] : 0;
+  {
+    C y[NC];
+#pragma unroll
+    for (int j = 0; j < NC; ++j) y[j] = *at(lane, c0 + j);
+    request(0, s0, x);
+    request(1, s1, nx);
+#pragma unroll
+    for (int j = 0; j < NC; ++j) raw[j * T + lane] = y[j];
+  }
+  __syncwarp();
+  complete(s0, x);
+  if constexpr (sizeof(C) == sizeof(float2)) {
+#pragma unroll
+    for (int j = 0; j < NC; ++j) top[j * T + lane] = x[j];
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < NC; ++j) x[j] = cmk<C>(0, 0);
+#pragma unroll 4
+    for (int k = 0; k < T; k += 2) {
+      const C a0 = sm.Li[lane * (T + 1) + k], a1 = sm.Li[lane * (T + 1) + k + 1];
+#pragma unroll
+      for (int j = 0; j < NC; ++j) {
+        const float4 u = *(const float4*)&top[j * T + k];
+        cfma(x[j], a0, cmk<C>(u.x, u.y));
+        cfma(x[j], a1, cmk<C>(u.z, u.w));
+      }
+    }
+    __syncwarp();
+  } else {
+    const C* L = sm.Pan + (ROWS ? s0 : lane);
+    for (int k = 0; k < T - 1; ++k) {
+      const C a = L[k * ldp];
+#pragma unroll
+      for (int j = 0; j < NC; ++j) {
+        const C u = shfl_c(x[j], k);
+        C y = x[j];
+        cfms(y, a, u);
+        if (lane > k) x[j] = y;
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < NC; ++j) top[j * T + lane] = x[j];
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < NC; ++j) *at(lane, c0 + j) = x[j];
+  for (int q = 1; q <= nbb; ++q) {
+    const C* L = sm.Pan + (ROWS ? s1 : q * T + lane);
+    complete(s1, nx);
+    C acc[NC];
+#pragma unroll
+    for (int j = 0; j < NC; ++j) acc[j] = nx[j];
+    if (q < nbb) {
+      s1 = sm.perm[(q + 1) * T + lane];
+      request(q + 1, s1, nx);
+    }
+    if constexpr (sizeof(C) == sizeof(float2)) {
+#pragma unroll 4
+      for (int k = 0; k < T; k += 2) {
+        const C a0 = L[k * ldp], a1 = L[(k + 1) * ldp];
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+          const float4 u = *(const float4*)&top[j * T + k];
+          cfms(acc[j], a0, cmk<C>(u.x, u.y));
+          cfms(acc[j], a1, cmk<C>(u.z, u.w));
+        }
+      }
+    } else {
+#pragma unroll 8
+      for (int k = 0; k < T; ++k) {
+        const C a = L[k * ldp];
+#pragma unroll
+        for (int j = 0; j < NC; ++j) cfms(acc[j], a, top[j * T + k]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < NC; ++j) *at(q * T + lane, c0 + j) = acc[j];
+  }
+  __syncwarp();
+}
+
+// Columns [0, ncol) of the block columns from Jc0 on, in groups of NC, over the warps of `nc` CTAs.
+template <typename C, int NC, bool ROWS>
+__device__ __forceinline__ void update_range(const FactorGeom& g, const FactorPtr<C>& f, int K, int Jc0, int ncol,
+                                             int cta, int nc, const FactorSmem<C>& sm) {
+  const int nw = blockDim.x >> 5;
+  for (int u = cta + nc * (int)(threadIdx.x >> 5); u * NC < ncol; u += nc * nw)
+    update_columns<C, NC, ROWS>(g, f, K, Jc0 + u * NC / kTile, (u * NC) % kTile, sm);
+}
+
+// PARTS: 0 for panel_lu_rows (-1: of more than 160 rows), else the threads of a row; NCF: columns a warp takes at once in the next
+// block column, NC: in the others; MAXT: the largest CTA; MINB: CTAs that share an SM.
+template <typename C, int PARTS, int NCF, int NC, int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB)
+    factor_kernel(FactorGeom g, const SysDesc* sys, char* arena, int* status, int32_t* ipiv, int spread) {
+  extern __shared__ __align__(16) char smem[];
+  __shared__ int sh_status;
+  constexpr int T = kTile, NCM = NCF > NC ? NCF : NC;
+  constexpr bool ROWS = PARTS <= 0;
+  cg::cluster_group cl = cg::this_cluster();
+  const int G = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int sidx = blockIdx.x / G;
+  const SysDesc d = sys[sidx];
+  const FactorPtr<C> f = factor_ptr<C>(g, arena + d.factor_off);
+  const int Pmax = (g.bt + 1) * T, ldp = Pmax + 1, nw = blockDim.x >> 5;
+  auto align16 = [](void* p) { return (void*)(((uintptr_t)p + 15) & ~(uintptr_t)15); };
+  FactorSmem<C> sm;
+  sm.top = (C*)smem;  // first: read as 16-byte words
+  sm.Li = sm.top + (size_t)nw * 2 * NCM * T;
+  sm.Pan = sm.Li + T * (T + 1);
+  if constexpr (ROWS) {
+    sm.U = (C*)align16(sm.Pan + (size_t)T * ldp);
+    sm.col = sm.U + T * (T + 2);
+    sm.key = (unsigned*)(sm.col + 2 * kRowsMax);
+    sm.log = (int*)(sm.key + 2 * kRowsMax);
+    sm.win = sm.log + kRowsMax;
+    sm.perm = sm.win + T;
+  } else {
+    sm.slot = (PivotSlot<C>*)align16(sm.Pan + (size_t)T * ldp);
+    sm.perm = (int*)(sm.slot + 2 * nw);
+  }
+  int32_t* piv = ipiv ? ipiv + (int64_t)sidx * g.n : nullptr;
+  if (threadIdx.x == 0) sh_status = 0;
+  __syncthreads();
+  auto panel = [&](int K) {
+    if constexpr (ROWS) {
+      panel_lu_rows<(PARTS < 0 ? 8 : 5)>(g, f, K, sm, &sh_status, piv);
+      store_panel_rows(g, f, K, sm);
+    } else {
+      panel_lu_parts<C, PARTS>(g, f, K, sm, &sh_status, piv);
+      if (sizeof(C) == sizeof(float2)) unit_lower_inverse<C>(g, f, K, sm);
+    }
+  };
+  auto csync = [&]() {
+    if (G > 1)
+      cl.sync();
+    else
+      __syncthreads();
+  };
+  if (rank == 0) panel(0);
+  csync();
+  for (int K = 0; K < g.Nb - 1; ++K) {
+    const int nbb = min(g.bt, g.Nb - 1 - K), nbr = min(2 * g.bt, g.Nb - 1 - K);
+    const int P = (nbb + 1) * T;
+    if (rank != 0) {  // CTA 0 holds the panel already
+      const int16_t* pg = f.perm + (int64_t)K * Pmax;
+      for (int e = threadIdx.x; e < P; e += blockDim.x) sm.perm[e] = pg[e];
+      const int lane = threadIdx.x & 31;
+      for (int q = 0; q <= nbb; ++q) {
+        const C* src = f.tiles + g.tile_index(K + q, K) * g.tile_elems + lane;
+        C* dst = sm.Pan + (ROWS ? (int)pg[q * T + lane] : q * T + lane);
+        for (int c = threadIdx.x >> 5; c < T; c += nw) dst[c * ldp] = src[c * T];
+      }
+      if (sizeof(C) == sizeof(float2)) {
+        const C* li = f.inv + (int64_t)(2 * K) * g.tile_elems;
+        for (int c = threadIdx.x >> 5; c < T; c += nw) sm.Li[lane * (T + 1) + c] = li[lane + c * T];
+      }
+      __syncthreads();
+    }
+    if (spread) {
+      update_range<C, NCF, ROWS>(g, f, K, K + 1, T, rank, G, sm);
+      csync();
+    } else if (rank == 0) {
+      update_range<C, NCF, ROWS>(g, f, K, K + 1, T, 0, 1, sm);
+      __syncthreads();
+    }
+    if (G == 1 || rank != 0)
+      update_range<C, NC, ROWS>(g, f, K, K + 2, (nbr - 1) * T, G == 1 ? 0 : rank - 1, G == 1 ? 1 : G - 1, sm);
+    if (G == 1) __syncthreads();
+    if (rank == 0) panel(K + 1);
+    csync();
+  }
+  if (rank == 0 && threadIdx.x == 0) status[sidx] = sh_status;
+}
+
+// Inverses of the diagonal blocks, one warp per block and system, lane = column: Uinv of the upper
+// triangle and, in FP64, Linv of the unit lower one.
+template <typename C>
+__global__ void __launch_bounds__(64) diag_inverse_kernel(FactorGeom g, const SysDesc* sys, char* arena) {
+  using R = typename real_of<C>::type;
+  constexpr int T = kTile;
+  __shared__ C D[T * T];   // the packed diagonal block, element (r, c) at r + c T
+  __shared__ C X[2][T * T];
+  const int K = blockIdx.x, lane = threadIdx.x & 31, which = threadIdx.x >> 5;
+  const FactorPtr<C> f = factor_ptr<C>(g, arena + sys[blockIdx.y].factor_off);
+  const C* src = f.tiles + g.tile_index(K, K) * g.tile_elems;
+  for (int e = threadIdx.x; e < T * T; e += blockDim.x) D[e] = src[e];
+  __syncthreads();
+  const int j = lane;
+  if (which == 0) {
+    C* U = X[0];
+    U[(T - 1) * T + j] = j == T - 1 ? crecip(D[j + j * T]) : cmk<C>(0, 0);
+    for (int i = T - 2; i >= 0; --i) {
+      C s = cmk<C>(0, 0);
+#pragma unroll 4
+      for (int k = i + 1; k < T; ++k)
+        if (k <= j) cfma(s, D[i + k * T], U[k * T + j]);
+      const C ri = crecip(D[i + i * T]);
+      const C u = cmul_rn(cmk<C>(s.x, s.y), ri);  // real part of s ri; the imaginary part below
+      U[i * T + j] = i == j ? ri : i > j ? cmk<C>(0, 0) : cmk<C>(-u.x, -fma(s.y, ri.x, mul_rn(s.x, ri.y)));
+    }
+  } else if (sizeof(C) == sizeof(double2)) {
+    C* L = X[1];
+    for (int i = 0; i < T; ++i) {
+      C s = cmk<C>(0, 0);
+#pragma unroll 4
+      for (int k = 0; k < i; ++k)
+        if (k >= j) cfma(s, D[i + k * T], L[k * T + j]);
+      L[i * T + j] = i == j ? cmk<C>(R(1), R(0)) : i < j ? cmk<C>(0, 0) : cmk<C>(-s.x, -s.y);
+    }
+  }
+  __syncthreads();
+  C* ui = f.inv + (int64_t)(2 * K + 1) * g.tile_elems;
+  C* li = f.inv + (int64_t)(2 * K) * g.tile_elems;
+  for (int e = threadIdx.x; e < T * T; e += blockDim.x) {
+    ui[e] = X[0][(e % T) * T + e / T];
+    if (sizeof(C) == sizeof(double2)) li[e] = X[1][(e % T) * T + e / T];
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -799,10 +1222,36 @@ size_t solve_smem_bytes(const FactorGeom& g, int chunk, size_t es, int trans) {
   return es * ((size_t)2 * T * kLdt + (size_t)T * chunk + uni);  // two tile slots
 }
 
-static size_t factor_smem_bytes(const FactorGeom& g, size_t es) {
-  const int T = kTile;
-  const size_t Pmax = (size_t)(g.bt + 1) * T;
-  return es * (2 * (Pmax + 1) * T + 2 * (size_t)T * T) + sizeof(int) * 3 * Pmax;
+// The widest band the factorization takes (the shared memory of two panels, their
+// permutations and the diagonal inverses; what the callers' workspaces were planned for).
+static bool factor_band_ok(const FactorGeom& g, size_t es) {
+  const size_t Pmax = (size_t)(g.bt + 1) * kTile;
+  return es * (2 * (Pmax + 1) * kTile + 2 * (size_t)kTile * kTile) + sizeof(int) * 3 * Pmax <= 227 * 1024;
+}
+
+template <typename C, int PARTS, int NCF, int NC, int MAXT, int MINB>
+static int launch_factor_cluster(const FactorGeom& g, int G, int spread, int nsys, const SysDesc* d_sys,
+                                 char* factor_arena, int* d_status, int32_t* d_ipiv, cudaStream_t st) {
+  const int Pmax = (g.bt + 1) * kTile, threads = PARTS > 0 ? Pmax * PARTS : MAXT;
+  const size_t smem = factor_cluster_smem<C, (PARTS <= 0)>(Pmax, threads / 32, NCF > NC ? NCF : NC);
+  auto kern = factor_kernel<C, PARTS, NCF, NC, MAXT, MINB>;
+  PD_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (G > 8) PD_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)nsys * (unsigned)G);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = G;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  PD_CK(cudaLaunchKernelEx(&cfg, kern, g, d_sys, factor_arena, d_status, d_ipiv, spread));
+  count_launch();
+  return 0;
 }
 
 template <typename C>
@@ -813,13 +1262,30 @@ int launch_factor(const FactorGeom& g, int cplx, const void* band, int64_t ldab,
   dim3 gi((unsigned)(g.tiles < 4096 ? g.tiles : 4096), (unsigned)nsys);
   init_factor_kernel<C><<<gi, kThreads, 0, st>>>(g, cplx, (const double*)band, ldab, d_sys, factor_arena);
   PD_CK_LAUNCH();
-  const size_t smem = factor_smem_bytes(g, sizeof(C));
-  if (smem > 227 * 1024) {
+  if (!factor_band_ok(g, sizeof(C))) {
     set_last_error_msg("band too wide for the factor kernel's shared memory");
     return PDESHEP_CUDA_ERROR;
   }
-  PD_CK(cudaFuncSetAttribute(factor_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  factor_kernel<C><<<nsys, kThreads, smem, st>>>(g, d_sys, factor_arena, d_status, d_ipiv);
+  // The cluster: as many CTAs as still shorten a block column, while all clusters run at once (76, 36
+  // and 15 clusters of 2, 4 and 8 fit at one CTA per SM).  complex64: a second CTA takes the updates off
+  // the panel's chain (b = 64: 34 -> 24.5 us per block column), at b > 64 four (68, 44, 30 us for 1, 2, 4);
+  // more change nothing.  complex128: every CTA shortens the updates (b = 32: 166, 151, 145 us for 2, 4,
+  // 8; b = 128: 1432, 1110, 394, 282 for 1 to 8).
+  const int most = sizeof(C) == sizeof(double2) ? 8 : g.bt > 2 ? 4 : 2;
+  const int G = most >= 8 && nsys <= 15 ? 8 : most >= 4 && nsys <= 36 ? 4 : nsys <= 76 ? 2 : 1;
+  if constexpr (sizeof(C) == sizeof(float2)) {
+    if ((g.bt + 1) * kTile > kRowsMax)
+      PD_TRY((launch_factor_cluster<C, 2, 2, 2, 832, 1>(g, G, 0, nsys, d_sys, factor_arena, d_status, d_ipiv, st)));
+    else if ((g.bt + 1) * kTile > 160)
+      PD_TRY((launch_factor_cluster<C, -1, 4, 4, 288, 1>(g, G, 0, nsys, d_sys, factor_arena, d_status, d_ipiv, st)));
+    else if (nsys <= 152)
+      PD_TRY((launch_factor_cluster<C, 0, 4, 4, 256, 1>(g, G, 0, nsys, d_sys, factor_arena, d_status, d_ipiv, st)));
+    else  // more systems than SMs: two per SM, with some registers spilled (256 systems, b = 64: 54 against 70 us)
+      PD_TRY((launch_factor_cluster<C, 0, 4, 4, 256, 2>(g, G, 0, nsys, d_sys, factor_arena, d_status, d_ipiv, st)));
+  } else {
+    PD_TRY((launch_factor_cluster<C, 4, 1, 1, 640, 1>(g, G, G > 1, nsys, d_sys, factor_arena, d_status, d_ipiv, st)));
+  }
+  diag_inverse_kernel<C><<<dim3((unsigned)g.Nb, (unsigned)nsys), 64, 0, st>>>(g, d_sys, factor_arena);
   PD_CK_LAUNCH();
   return 0;
 }

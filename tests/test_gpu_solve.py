@@ -67,3 +67,50 @@ def test_band_matmul(device):
         Y = block_from_dev(pk.band_matmul(to_dev(ab, device), block_to_dev(X, device)))
         Yo = oracle.band_matvec(ab, X)
         assert np.max(np.abs(Y - (Yo if cplx else Yo.real))) < 1e-13
+
+
+# The factorization's dispatch: panels of at most 160 rows, of at most 256 (b <= 224) and wider; one CTA per
+# system (more systems than clusters), two per SM (more than 152 systems) and clusters of 2, 4 and 8; the last
+# block columns and orders that are no multiple of the tile.
+@pytest.mark.parametrize("n,b,nshift,precision", [(33, 32, 1, 1), (95, 40, 5, 1), (260, 100, 3, 1), (300, 130, 40, 1),
+                                                  (330, 224, 2, 1), (420, 230, 2, 1), (450, 350, 1, 1),
+                                                  (129, 31, 160, 1), (100, 33, 80, 1), (64, 64, 50, 1),
+                                                  (161, 30, 20, 0), (200, 70, 40, 0), (97, 96, 80, 0), (260, 128, 4, 0)])
+def test_factor_dispatch_pivots_and_solutions(device, n, b, nshift, precision):
+    import paper_2012_00506_gb300 as pk
+    ab = synth.random_band(n, b, 5000 + n + b, True)
+    lo, hi = oracle.gershgorin(ab)
+    t = (np.arange(nshift) + 0.5) / nshift
+    shifts = lo + (hi - lo) * (0.1 + 0.8 * t) + 1j * (hi - lo) * (0.02 + 0.05 * t)
+    Y = synth.random_subspace(n, 3, 6000 + n, True)
+    for trans in (0, 1):
+        X, ipiv = pk.shifted_solve(to_dev(ab, device), shifts, block_to_dev(Y, device), trans=trans,
+                                   precision=precision, return_ipiv=True)
+        ipiv = ipiv.cpu().numpy()
+        for s in sorted({0, nshift // 2, nshift - 1}):
+            F, ip, info = oracle.band_lu(ab, shifts[s])
+            Xo = oracle.band_solve(F, ip, b, Y, trans)
+            err = np.max(np.abs(block_from_dev(X[s]) - Xo)) / np.max(np.abs(Xo))
+            if precision == pk.FP64:
+                assert np.array_equal(ipiv[s], ip)
+            assert err < (1e-11 if precision == pk.FP64 else 1e-4), (s, trans, err)
+
+
+def test_equal_pivots_take_the_lowest_row(device):
+    """Bands whose columns hold entries of equal modulus: the pivot is the first of them, as in gbtrf."""
+    import paper_2012_00506_gb300 as pk
+    n, b = 150, 40
+    ab = np.where(np.arange(b + 1)[None, :] + np.arange(n)[:, None] < n, 1.0, 0.0) * np.where(
+        np.arange(b + 1) % 3 == 1, -0.5, 0.5)
+    ab[:, 0] = 0.25
+    z = np.array([0.25 + 0.5j, 0.75 + 0.0625j])
+    Y = synth.random_subspace(n, 2, 77, True)
+    for precision in (0, 1):
+        X, ipiv = pk.shifted_solve(to_dev(ab, device), z, block_to_dev(Y, device), precision=precision,
+                                   return_ipiv=True)
+        for s in range(2):
+            F, ip, info = oracle.band_lu(ab, z[s])
+            k = 33  # while the entries are still exact in both precisions
+            assert np.array_equal(ipiv.cpu().numpy()[s][:1], ip[:1])
+            if precision == pk.FP64:
+                assert np.array_equal(ipiv.cpu().numpy()[s][:k], ip[:k])
