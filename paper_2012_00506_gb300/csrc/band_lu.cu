@@ -1189,7 +1189,8 @@ __device__ void solve_c_body(const FactorGeom& g, const SysDesc& d, int col0, co
 
 // Persistent solve: the grid holds as many blocks as fit on the GPU at once;
 // each block takes (system, column block) items from a shared counter until
-// the list is exhausted, so systems of uneven m0 keep every SM busy.
+// the list is exhausted, so systems of uneven m0 keep every SM busy.  A column
+// block of 8 (complex128) takes the items of 16 columns in halves.
 template <typename C, int CW, int TRANS>
 __global__ void __launch_bounds__(kThreads) solve_kernel(FactorGeom g, const SysDesc* sys, const char* arena,
                                                         const C* rhs, C* out, const int2* items, int nitems,
@@ -1202,8 +1203,10 @@ __global__ void __launch_bounds__(kThreads) solve_kernel(FactorGeom g, const Sys
     const int item = sh_item;
     __syncthreads();  // every thread has its item before thread 0 fetches the next one
     if (item >= nitems) return;
-    const int2 w = items[item];
+    int2 w = items[CW == 8 ? item >> 1 : item];
+    if (CW == 8) w.y += 8 * (item & 1);
     const SysDesc d = sys[w.x];
+    if (w.y >= d.ncols) continue;  // (the same for every thread)
     if (TRANS == 0)
       solve_n_body<C, CW>(g, d, w.y, arena, rhs, out, smem);
     else
@@ -1303,6 +1306,7 @@ size_t solve_queue_bytes(int nsys, int max_cols) {
 // the queue scratch (counter first, then the items).  Returns the item count.
 int upload_solve_items(int nsys, const SysDesc* h_sys, int chunk, void* queue, cudaStream_t st, int* nitems) {
   if (chunk == kTcChunk) chunk = kTmChunk;  // the tensor-core solve also takes 128 right-hand sides per item
+  if (chunk == 8) chunk = 16;               // halves of 16-column items
   std::vector<int2> it;
   for (int s = 0; s < nsys; ++s)
     for (int c = 0; c < h_sys[s].ncols; c += chunk) it.push_back(make_int2(s, c));
@@ -1327,6 +1331,7 @@ static int launch_solve_cw(const FactorGeom& g, int nitems, const SysDesc* d_sys
   Arena qa(queue, ~size_t(0));
   int* counter = qa.take<int>(1);
   const int2* d_items = qa.take<int2>((size_t)nitems);
+  if (CW == 8) nitems *= 2;
   auto kern = solve_kernel<C, CW, TRANS>;
   PD_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0, dev = 0, sms = 0;
@@ -1352,6 +1357,11 @@ int launch_solve_queued(const FactorGeom& g, int trans, int nitems, const SysDes
     set_last_error_msg("the tensor-memory and tensor-core solves are complex64 only");
     return PDESHEP_CUDA_ERROR;
   }
+  if constexpr (std::is_same<C, double2>::value) {
+    if (chunk == 8)
+      return trans ? launch_solve_cw<C, 8, 1>(g, nitems, d_sys, factor_arena, rhs_arena, out_arena, queue, st)
+                   : launch_solve_cw<C, 8, 0>(g, nitems, d_sys, factor_arena, rhs_arena, out_arena, queue, st);
+  }
   switch (chunk * 2 + (trans ? 1 : 0)) {
     case 32: return launch_solve_cw<C, 16, 0>(g, nitems, d_sys, factor_arena, rhs_arena, out_arena, queue, st);
     case 33: return launch_solve_cw<C, 16, 1>(g, nitems, d_sys, factor_arena, rhs_arena, out_arena, queue, st);
@@ -1365,13 +1375,38 @@ int launch_solve_queued(const FactorGeom& g, int trans, int nitems, const SysDes
   }
 }
 
+// The column block of the tiled solve for these systems: the least waves of items over 152 SMs times an
+// item's time.  complex128 is bound by its SM's FP64 pipe, an item's time by its columns (b = 32: 1.34,
+// 2.58, 5.04, 10.0 us per row for 8, 16, 32, 64 columns; 152 items of 8 run 3.8 times as fast as 40 of
+// 32).  complex64 items are bound by the chain of a step while they are alone on an SM (b = 64: 0.31, 0.42,
+// 0.69 us per row for 16, 32, 64) and by the SM's throughput when several share it (0.215, 0.35, 0.7 each);
+// 64 columns, and the 128 of the tensor-memory kernel (1.14), never won.
+int solve_width(const FactorGeom& g, size_t es, int nsys, const SysDesc* h_sys) {
+  const bool dbl = es == sizeof(double2);
+  int best = 16;
+  double best_t = 1e300;
+  for (int cw = dbl ? 8 : 16; cw <= (dbl ? 64 : 32); cw *= 2) {
+    if (cw > 16 && solve_smem_bytes(g, cw, es, 0) > 227 * 1024) break;
+    int64_t items = 0;
+    for (int s = 0; s < nsys; ++s) items += ceil_div(h_sys[s].ncols, cw);
+    const double waves = (double)ceil_div(items, 152);
+    const double t = dbl ? waves * (0.1 + 0.155 * cw)
+                         : std::max(cw == 16 ? 0.31 : 0.42, waves * (cw == 16 ? 0.215 : 0.35));
+    if (t < best_t) {
+      best_t = t;
+      best = cw;
+    }
+  }
+  return best;
+}
+
 template <typename C>
 int launch_solve(const FactorGeom& g, int trans, int nsys, const SysDesc* h_sys, const SysDesc* d_sys,
                  const char* factor_arena, const C* rhs_arena, C* out_arena, int chunk, void* queue,
                  cudaStream_t st) {
   if (nsys <= 0) return 0;
-  if (chunk <= 0) chunk = 32;
-  if (chunk != 16 && chunk != 32 && chunk != 64 && chunk != kTmChunk && chunk != kTcChunk) {
+  if (chunk <= 0) chunk = solve_width(g, sizeof(C), nsys, h_sys);
+  if (chunk != 8 && chunk != 16 && chunk != 32 && chunk != 64 && chunk != kTmChunk && chunk != kTcChunk) {
     set_last_error_msg("right-hand-side block width must be 16, 32, 64, 128 or 256");
     return PDESHEP_CUDA_ERROR;
   }

@@ -87,13 +87,15 @@ int launch_factor(const FactorGeom& g, int cplx, const void* band, int64_t ldab,
 
 // trans = 0: X = (zI-B)^{-1} Y;  trans = 1: X = (zI-B)^{-H} Y.  Y and X hold C.
 // h_sys: the same descriptors on the host (their column counts build the work
-// list).  chunk: right-hand sides per work item (16, 32 or 64; 0 = 32; 128 = the
-// tensor-memory kernel of solve_tm.cu, complex64 only).
+// list).  chunk: right-hand sides per work item (16, 32 or 64; complex128 also 8; 0 =
+// solve_width's choice; 128 = the tensor-memory kernel of solve_tm.cu, complex64 only).
 // queue: device scratch of solve_queue_bytes(nsys, max columns).
 template <typename C>
 int launch_solve(const FactorGeom& g, int trans, int nsys, const SysDesc* h_sys, const SysDesc* d_sys,
                  const char* factor_arena, const C* rhs_arena, C* out_arena, int chunk, void* queue,
                  cudaStream_t st);
+
+int solve_width(const FactorGeom& g, size_t es, int nsys, const SysDesc* h_sys);
 
 // The same in two steps: the work list is uploaded once (a host-to-device
 // copy, outside any stream capture), then launches replay it (capturable).

@@ -616,23 +616,30 @@ struct Feast {
   // steps run to 7 iterations; two or three passes are slower).  An explicit rhs_chunk serves every
   // pass.
   int rhs_chunk = 32;  // width of the current pass
-  int chunk_late = 32, chunk_early = 0;
+  int chunk_late = 0, chunk_early = 0;  // late 0: solve_width's choice for the pass's active systems
   int iter_now = 1;
   static constexpr int kTcIterations = 4;
-  int pass_chunk() const { return (chunk_early && iter_now <= kTcIterations) ? chunk_early : chunk_late; }
+  int pass_chunk() const {
+    if (chunk_early && iter_now <= kTcIterations) return chunk_early;
+    if (chunk_late) return chunk_late;
+    std::vector<SysDesc> sd;  // only the column counts matter
+    for (int s : active)
+      for (int j = 0; j < ne; ++j) {
+        SysDesc d = {};
+        d.ncols = m0[s];
+        sd.push_back(d);
+      }
+    return solve_width(g, es, (int)sd.size(), sd.data());
+  }
   int gram_splits = 0;  // 0: heuristic
   bool tune_solve = false, tune_gram = false;
 
-  // the default solve: the tensor-memory kernel for complex64 factors when its window fits
-  int default_chunk() const {
-    return (o->precision == PDESHEP_MIXED && solve_tm_supported(g)) ? kTmChunk : 32;
-  }
   void setup_tuning() {
     if (o->rhs_chunk > 0) {
       chunk_late = o->rhs_chunk;
       chunk_early = 0;
     } else {
-      chunk_late = default_chunk();
+      chunk_late = 0;
       chunk_early = (o->precision == PDESHEP_MIXED && solve_tc_supported(g)) ? kTcChunk : 0;
     }
     rhs_chunk = pass_chunk();
@@ -1047,8 +1054,9 @@ struct FeastRun : Feast<S, C> {
       PD_CK(cudaEventCreate(&t0));
       PD_CK(cudaEventCreate(&t1));
       float best = 1e30f, t_tc = 1e30f;
-      int best_cw = this->default_chunk();
-      for (int cw : {16, 32, 64, kTmChunk, kTcChunk}) {
+      int best_cw = 32;
+      for (int cw : {8, 16, 32, 64, kTmChunk, kTcChunk}) {
+        if (cw == 8 && sizeof(C) != sizeof(double2)) continue;
         if (cw == kTmChunk   ? !(sizeof(C) == sizeof(float2) && solve_tm_supported(g))
             : cw == kTcChunk ? !(sizeof(C) == sizeof(float2) && solve_tc_supported(g))
                              : solve_smem_bytes(g, cw, sizeof(C), 0) > 227 * 1024)

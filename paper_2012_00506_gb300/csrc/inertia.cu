@@ -663,8 +663,12 @@ static int panel_clusters(int b, int G) {
 // rest of a round (barriers, row entry, triangle), the CTA's share of the updates at 76 clocks per
 // warp instruction and FP64 pipe; CTAs that share an SM share its pipes.  `sms` is what clusters of G
 // reach at one CTA per SM.  At b = 64 complex the measured times cross at about 110 shifts.
+// beside: the counts run on a side stream next to factorizations that need whole SMs, and nobody waits
+// for them until two filter passes are done, so they keep to about 20 CTAs (9 shifts of n = 8192, b = 64
+// complex on 112 SMs stretched a factorization of 64 systems from 6.4 to 18 ms).
+constexpr int kBesideCtas = 20;
 template <bool CPLX>
-static int panel_cluster_size(int b, int nsigma, bool single_ok) {
+static int panel_cluster_size(int b, int nsigma, bool single_ok, bool beside) {
   static const int sms[5] = {152, 152, 144, 120, 112};
   const double np = CPLX ? 2.0 : 1.0, ops = CPLX ? 4.0 : 2.0;
   const double work = 0.5 * b * (b + 1.0) * np / 32.0 * ops * 19.0;  // all updates of one column
@@ -681,6 +685,7 @@ static int panel_cluster_size(int b, int nsigma, bool single_ok) {
   for (int G = 1, q = 0; G <= 16; G *= 2, ++q) {
     const int nc = panel_clusters<CPLX>(b, G);
     if (nc < 1) continue;
+    if (beside && best >= 0 && (int64_t)nsigma * G > kBesideCtas) break;
     const int chunks = panel_shape(b, CPLX, G).chunks;
     const int waves = (int)ceil_div(nsigma, nc);
     const double co = (double)ceil_div((int64_t)std::min(nsigma, nc) * G, sms[q]);
@@ -714,10 +719,11 @@ static int launch_panel(int64_t n, int b, const void* band, int64_t ldab, int ns
 // the workspace) serves only bands that no cluster's shared memory holds.
 int launch_inertia(int64_t n, int b, int cplx, const void* band, int64_t ldab, int nsigma,
                    const double* d_sigma, const unsigned long long* amax, int64_t* d_neg,
-                   double* d_piv, char* gwin, size_t gwin_stride, cudaStream_t st) {
+                   double* d_piv, char* gwin, size_t gwin_stride, cudaStream_t st, bool beside = false) {
   if (nsigma <= 0) return 0;
   const bool single = window_in_smem(b, cplx);
-  const int G = cplx ? panel_cluster_size<true>(b, nsigma, single) : panel_cluster_size<false>(b, nsigma, single);
+  const int G = cplx ? panel_cluster_size<true>(b, nsigma, single, beside)
+                     : panel_cluster_size<false>(b, nsigma, single, beside);
   if (G > 0)
     return cplx ? launch_panel<true>(n, b, band, ldab, nsigma, d_sigma, amax, d_neg, d_piv, G, st)
                 : launch_panel<false>(n, b, band, ldab, nsigma, d_sigma, amax, d_neg, d_piv, G, st);
@@ -736,7 +742,7 @@ size_t inertia_ws_bytes(int b, int cplx, int nsigma) {
   return a.used();
 }
 
-// Asynchronous counts: everything is enqueued on st; the counts (nsigma int64)
+// Asynchronous counts beside other work: everything is enqueued on st; the counts (nsigma int64)
 // and the non-finite flag (int) stay in the workspace at *d_neg / *d_bad.
 int inertia_counts_async(int64_t n, int b, int cplx, const void* band, int64_t ldab, int nsigma,
                          const double* h_sigma, void* work, size_t wbytes, cudaStream_t st,
@@ -747,7 +753,7 @@ int inertia_counts_async(int64_t n, int b, int cplx, const void* band, int64_t l
   PD_TRY(launch_band_amax(n, b, cplx, band, ldab, w.amax, w.nonfinite, st));
   PD_CK(cudaMemcpyAsync(w.sigma, h_sigma, sizeof(double) * nsigma, cudaMemcpyHostToDevice, st));
   PD_TRY(launch_inertia(n, b, cplx, band, ldab, nsigma, w.sigma, w.amax, w.neg, nullptr, w.gwin,
-                        w.gwin_stride, st));
+                        w.gwin_stride, st, true));
   *d_neg = w.neg;
   *d_bad = w.nonfinite;
   return 0;

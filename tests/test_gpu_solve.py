@@ -114,3 +114,25 @@ def test_equal_pivots_take_the_lowest_row(device):
             assert np.array_equal(ipiv.cpu().numpy()[s][:1], ip[:1])
             if precision == pk.FP64:
                 assert np.array_equal(ipiv.cpu().numpy()[s][:k], ip[:k])
+
+
+# The default column block: 8 (halves of 16-column items), 16, 32 and 64 in FP64, 16 and 32 in complex64 beyond
+# the tensor-core solve's bands; column counts at the edges of the blocks.
+@pytest.mark.parametrize("precision,b,nshift,nrhs", [(0, 20, 1, 1), (0, 20, 2, 8), (0, 33, 3, 9), (0, 20, 9, 150),
+                                                     (0, 20, 70, 33), (0, 20, 152, 65), (1, 140, 2, 17),
+                                                     (1, 140, 40, 70)])
+def test_default_solve_width(device, precision, b, nshift, nrhs):
+    import paper_2012_00506_gb300 as pk
+    n = 150
+    ab = synth.random_band(n, b, 7000 + b, True)
+    lo, hi = oracle.gershgorin(ab)
+    t = (np.arange(nshift) + 0.5) / nshift
+    shifts = lo + (hi - lo) * t + 0.1j * (hi - lo)
+    Y = synth.random_subspace(n, nrhs, 8000 + nrhs, True)
+    for trans in (0, 1):
+        X = pk.shifted_solve(to_dev(ab, device), shifts, block_to_dev(Y, device), trans=trans, precision=precision)
+        for s in sorted({0, nshift - 1}):
+            F, ip, _ = oracle.band_lu(ab, shifts[s])
+            Xo = oracle.band_solve(F, ip, b, Y, trans)
+            err = np.max(np.abs(block_from_dev(X[s]) - Xo)) / np.max(np.abs(Xo))
+            assert err < (1e-11 if precision == pk.FP64 else 1e-4), (s, trans, err)
