@@ -12,6 +12,8 @@
 
 #include <algorithm>
 #include <map>
+#include <mutex>
+#include <tuple>
 #include <vector>
 
 #include "dense.cuh"
@@ -673,8 +675,28 @@ struct Rot {
   int p, q;
 };
 
-// Rotation of the pair (p, q) of one round.  Indices >= m (the dummy player of
-// an odd m) are stored as -1; a pair without rotation keeps c = 1, s = 0, u = 1.
+// Rotation that annihilates A(p,q) given app = A(p,p), aqq = A(q,q); c = 1, s = 0, u = 1 if it is
+// negligible.
+template <typename S>
+__device__ __forceinline__ void rotation(S apq, typename real_t<S>::type app, typename real_t<S>::type aqq,
+                                         typename real_t<S>::type& rc, typename real_t<S>::type& rs, S& ru) {
+  using R = typename real_t<S>::type;
+  rc = R(1);
+  rs = R(0);
+  ru = sc<S>::from_re(R(1));
+  // |A(p,q)| without squaring: in FP32 the square of an element below ~1e-19
+  // is subnormal, and a modulus taken from it makes the rotation non-unitary
+  const R g = sc<S>::absv(apq);
+  const R tiny = sizeof(R) == 8 ? R(1e-290) : R(1e-30);
+  if (!(g > tiny)) return;
+  ru = sc<S>::scale(apq, R(1) / g);
+  const R th = (aqq - app) / (R(2) * g);
+  const R t = (th >= R(0) ? R(1) : R(-1)) / (fabs(th) + sqrt(th * th + R(1)));
+  rc = R(1) / sqrt(t * t + R(1));
+  rs = t * rc;
+}
+
+// Rotation of the pair (p, q) of one round.  Indices >= m (the dummy player of an odd m) are stored as -1.
 template <typename S>
 __device__ __forceinline__ void make_rot(const S* A, int m, int p, int q, Rot<S>& r) {
   using R = typename real_t<S>::type;
@@ -684,18 +706,357 @@ __device__ __forceinline__ void make_rot(const S* A, int m, int p, int q, Rot<S>
   r.s = R(0);
   r.u = sc<S>::from_re(R(1));
   if (p >= m || q >= m) return;
-  const S apq = A[p + (int64_t)q * m];
-  // |A(p,q)| without squaring: in FP32 the square of an element below ~1e-19
-  // is subnormal, and a modulus taken from it makes the rotation non-unitary
-  const R g = sc<S>::absv(apq);
-  const R tiny = sizeof(R) == 8 ? R(1e-290) : R(1e-30);
-  if (!(g > tiny)) return;
-  r.u = sc<S>::scale(apq, R(1) / g);
-  const R app = sc<S>::re(A[p + (int64_t)p * m]), aqq = sc<S>::re(A[q + (int64_t)q * m]);
-  const R th = (aqq - app) / (R(2) * g);
-  const R t = (th >= R(0) ? R(1) : R(-1)) / (fabs(th) + sqrt(th * th + R(1)));
-  r.c = R(1) / sqrt(t * t + R(1));
-  r.s = t * r.c;
+  rotation<S>(A[p + (int64_t)q * m], sc<S>::re(A[p + (int64_t)p * m]), sc<S>::re(A[q + (int64_t)q * m]), r.c, r.s, r.u);
+}
+
+// conj(a) b with the roundings spelled out (the two Jacobi kernels give the same bits; left to itself the
+// compiler contracts the expression differently in each): re = a.x b.x + [a.y b.y], im = -a.y b.x + [a.x b.y].
+__device__ __forceinline__ float mul_cj(float a, float b) { return a * b; }
+__device__ __forceinline__ double mul_cj(double a, double b) { return a * b; }
+__device__ __forceinline__ float2 mul_cj(float2 a, float2 b) {
+  return make_float2(__fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)), __fmaf_rn(-a.y, b.x, __fmul_rn(a.x, b.y)));
+}
+__device__ __forceinline__ double2 mul_cj(double2 a, double2 b) {
+  return make_double2(__fma_rn(a.x, b.x, __dmul_rn(a.y, b.y)), __fma_rn(-a.y, b.x, __dmul_rn(a.x, b.y)));
+}
+
+// The rotated 2 x 2 block x (rows of pair i, columns of pair k): columns [x_p, x_q] <- [x_p u c - x_q s,
+// x_p u s + x_q c] (pair k), rows [x_p; x_q] <- [conj(u c) x_p - s x_q; conj(u s) x_p + c x_q] (pair i).
+template <typename S, typename R>
+__device__ __forceinline__ void rotate_block(S (&x)[2][2], R ic, R is, S iuc, S ius, R kc, R ks, S uck, S usk) {
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const S xp = x[a][0], xq = x[a][1];
+    x[a][0] = sc<S>::sub(sc<S>::mul(xp, uck), sc<S>::scale(xq, ks));
+    x[a][1] = sc<S>::add(sc<S>::mul(xp, usk), sc<S>::scale(xq, kc));
+  }
+#pragma unroll
+  for (int b2 = 0; b2 < 2; ++b2) {
+    const S xp = x[0][b2], xq = x[1][b2];
+    x[0][b2] = sc<S>::sub(mul_cj(iuc, xp), sc<S>::scale(xq, is));
+    x[1][b2] = sc<S>::add(mul_cj(ius, xp), sc<S>::scale(xq, ic));
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The same rounds with the matrix in (distributed) shared memory.  In global memory a round cost 7 to 10 us,
+// almost all of it L2 latency and the cluster barrier's wait for global stores, against 1 us of work.
+// Here the pairs of a round have places 0 .. np-1, CTA g of the cluster holds the columns (of A and of V)
+// of places [g w, (g+1) w), and from one round to the next every column moves by one place: the first
+// players' row to the left, the others' to the right (the circle method), so a CTA passes one column to
+// each neighbour per round.  A round: every CTA derives its own pairs' rotations and sends them to all,
+// cluster barrier, the 2 x 2 blocks of its columns and its columns of V in place, the two columns to the
+// neighbours' free slots, cluster barrier.  Same pairs, formulas and stopping test as jacobi_kernel, which
+// remains for orders whose columns do not fit.
+// Measured (FP32 stage of pdeshep_eigh): 8 blocks of 267 complex columns 16.1 -> 8.8 ms, one of 150 real ones
+// 3.9 -> 2.8, two of 20 0.32 -> 0.18.  A round of 267 columns on 16 CTAs is now about 9000 clocks: rotations
+// 1200, two barriers with their skew 2100, A 1900, V 1400, columns to the neighbours 600.
+// ---------------------------------------------------------------------------
+template <typename S>
+struct RingRot {  // the rotation and the products its users need
+  S uc, us;
+  typename real_t<S>::type c, s;
+};
+
+constexpr int kRingThreads = 512;
+
+template <typename S>
+static size_t ring_smem(int m, int w) {
+  using R = typename real_t<S>::type;
+  const int np = (m + 1) / 2;
+  return sizeof(S) * (size_t)2 * (2 * w + 2) * m + sizeof(RingRot<S>) * (size_t)np + sizeof(R) * (size_t)m +
+         sizeof(double) * 64 + sizeof(int) * (size_t)(4 * w + 16) + 64;
+}
+// places per CTA (at least two, so that the fixed player's neighbour place is in the same CTA)
+__host__ __device__ inline int ring_places(int m, int G) {
+  const int np = (m + 1) / 2, w = (np + G - 1) / G;
+  return w < 2 ? 2 : w;
+}
+
+template <typename S>
+__global__ void __launch_bounds__(kRingThreads, sizeof(S) <= 8 ? 2 : 1)
+    jacobi_ring_kernel(const SmallDesc* desc, const S* Aall, S* Vout, double* lamall, double tol, int max_sweeps,
+                       int* sweeps_out) {
+  using R = typename real_t<S>::type;
+  extern __shared__ __align__(16) char smem[];
+  __shared__ double red[2][kRingThreads / 32];
+  cg::cluster_group cl = cg::this_cluster();
+  const int G = (int)cl.num_blocks(), g = (int)cl.block_rank();
+  const int t = blockIdx.x / G;
+  const SmallDesc d = desc[t];
+  const int m = d.m, M = m + (m & 1), np = M / 2, M1 = M - 1;
+  const int w = ring_places(m, G), i0 = g * w, wl = max(0, min(w, np - i0)), last = (np - 1) / w;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int NW = kRingThreads / 32;
+  S* colA = (S*)smem;                           // [2 w + 2][m]
+  S* colV = colA + (size_t)(2 * w + 2) * m;     // [2 w + 2][m]
+  RingRot<S>* rot = (RingRot<S>*)(colV + (size_t)(2 * w + 2) * m);  // [np]
+  double* part = (double*)(((uintptr_t)(rot + np) + 7) & ~(uintptr_t)7);  // [16][2]
+  R* lam = (R*)(part + 32);                     // [m]
+  int* slots = (int*)(((uintptr_t)(lam + m) + 3) & ~(uintptr_t)3);  // [2][2 w + 2]: slots of the first and second players,
+                                                // then the free slots for a column from the right / from the left
+  int* nb = slots + 2 * (2 * w + 2);            // [0]: the left neighbour's free slot, [1]: the right neighbour's
+  auto csync = [&]() {
+    if (G > 1)
+      cl.sync();
+    else
+      __syncthreads();
+  };
+  auto first_of = [&](int r, int i) { return r + i >= M1 ? r + i - M1 : r + i; };             // player at place i
+  auto second_of = [&](int r, int i) { return i == 0 ? M1 : (r - i < 0 ? r - i + M1 : r - i); };
+
+  // tasks (place j, 32 rows or row pairs ch) of a warp: warp, warp + NW, ...
+  const int lgG = 31 - __clz(G), nch = (np + 31) >> 5, nvc = (m + 31) >> 5;
+  const int ja = warp / nch, ca = warp % nch, jv = warp / nvc, cv = warp % nvc;
+  const int qa = NW / nch, ra = NW % nch, qv = NW / nvc, rv = NW % nvc;
+  auto step = [&](int& j, int& ch, int n) {
+    ch += n == nch ? ra : rv;
+    j += n == nch ? qa : qv;
+    if (ch >= n) {
+      ch -= n;
+      ++j;
+    }
+  };
+  const S* A = Aall + d.off;
+  for (int e = tid; e < 2 * wl; e += kRingThreads) slots[e < wl ? e : w + e - wl] = e;
+  if (tid == 0) {
+    slots[2 * w] = 2 * wl;
+    slots[2 * w + 1] = 2 * wl + 1;
+  }
+  for (int c = warp; c < 2 * wl; c += NW) {
+    const int pl = c < wl ? first_of(0, i0 + c) : second_of(0, i0 + c - wl);
+    for (int k = lane; k < m; k += 32) {
+      colA[(size_t)c * m + k] = pl < m ? A[k + (int64_t)pl * m] : sc<S>::zero();
+      colV[(size_t)c * m + k] = sc<S>::from_re(k == pl ? R(1) : R(0));
+    }
+  }
+  csync();
+  int sweeps = 0, converged = 0, par = 0;
+  for (;; ++sweeps) {
+    // off-norm and Frobenius norm (deterministic: per-CTA partials summed in rank order); at the start of a
+    // sweep every column is where round 0 has it
+    const int* sl = slots + par * (2 * w + 2);
+    double off = 0.0, fro = 0.0;
+    for (int c = warp; c < 2 * wl; c += NW) {
+      const int pl = c < wl ? first_of(0, i0 + c) : second_of(0, i0 + c - wl);
+      const S* col = colA + (size_t)sl[c < wl ? c : w + c - wl] * m;
+      if (pl < m)
+        for (int k = lane; k < m; k += 32) {
+          const double a2 = (double)sc<S>::abs2(col[k]);
+          fro += a2;
+          if (k != pl) off += a2;
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      off += __shfl_down_sync(0xffffffffu, off, o);
+      fro += __shfl_down_sync(0xffffffffu, fro, o);
+    }
+    if (lane == 0) {
+      red[0][warp] = off;
+      red[1][warp] = fro;
+    }
+    __syncthreads();
+    if (tid < 2 * G) {
+      double sum = 0.0;
+      for (int q = 0; q < NW; ++q) sum += red[tid & 1][q];
+      double* dst = G > 1 ? cl.map_shared_rank(part, tid >> 1) : part;
+      dst[2 * g + (tid & 1)] = sum;
+    }
+    csync();
+    double so = 0.0, sf = 0.0;
+    for (int c = 0; c < G; ++c) {
+      so += part[2 * c];
+      sf += part[2 * c + 1];
+    }
+    if (sqrt(so) <= tol * sqrt(sf) || sf == 0.0) {
+      converged = 1;
+      break;
+    }
+    if (sweeps >= max_sweeps) break;
+    for (int r = 0; r < M1; ++r, par ^= 1) {
+      const int* cur = slots + par * (2 * w + 2);
+      int* nxt = slots + (par ^ 1) * (2 * w + 2);
+      // rotations of the own pairs, one copy per CTA of the cluster
+      for (int e = tid; e < (wl << lgG); e += kRingThreads) {
+        const int j = e >> lgG, to = e & (G - 1);
+        const int p = first_of(r, i0 + j), q = second_of(r, i0 + j);
+        RingRot<S> x;
+        x.c = R(1);
+        x.s = R(0);
+        S u = sc<S>::from_re(R(1));
+        if (p < m && q < m) {
+          const S* cp = colA + (size_t)cur[j] * m;
+          const S* cq = colA + (size_t)cur[w + j] * m;
+          rotation<S>(cq[p], sc<S>::re(cp[p]), sc<S>::re(cq[q]), x.c, x.s, u);
+        }
+        x.uc = sc<S>::scale(u, x.c);
+        x.us = sc<S>::scale(u, x.s);
+        RingRot<S>* dst = G > 1 ? cl.map_shared_rank(rot, to) : rot;
+        dst[i0 + j] = x;
+      }
+      if (tid == 0 && wl > 0) {  // where the neighbours may put their columns
+        if (g < last) cl.map_shared_rank(nb, g + 1)[0] = cur[2 * w];
+        if (g > 0) cl.map_shared_rank(nb, g - 1)[1] = cur[2 * w + 1];
+      }
+      csync();
+      // A <- J^H A J on the own columns: the block of rows (p_i, q_i) and columns (p_k, q_k) needs the
+      // rotations of pairs i and k only; a warp takes 32 row pairs of one column pair
+      for (int j = ja, ch = ca; j < wl; step(j, ch, nch)) {
+        const int i = ch * 32 + lane;
+        if (i >= np) continue;
+        const RingRot<S> ri = rot[i], rk = rot[i0 + j];
+        const int p = first_of(r, i), q = second_of(r, i);
+        S* cp = colA + (size_t)cur[j] * m;
+        S* cq = colA + (size_t)cur[w + j] * m;
+        S x[2][2];
+        x[0][0] = p < m ? cp[p] : sc<S>::zero();
+        x[0][1] = p < m ? cq[p] : sc<S>::zero();
+        x[1][0] = q < m ? cp[q] : sc<S>::zero();
+        x[1][1] = q < m ? cq[q] : sc<S>::zero();
+        rotate_block<S, R>(x, ri.c, ri.s, ri.uc, ri.us, rk.c, rk.s, rk.uc, rk.us);
+        if (i == i0 + j && p < m && q < m) {  // the rotated pivot block: exact zeros, real diagonal
+          x[0][1] = sc<S>::zero();
+          x[1][0] = sc<S>::zero();
+          x[0][0] = sc<S>::from_re(sc<S>::re(x[0][0]));
+          x[1][1] = sc<S>::from_re(sc<S>::re(x[1][1]));
+        }
+        if (p < m) {
+          cp[p] = x[0][0];
+          cq[p] = x[0][1];
+        }
+        if (q < m) {
+          cp[q] = x[1][0];
+          cq[q] = x[1][1];
+        }
+      }
+      // V <- V J
+      for (int j = jv, ch = cv; j < wl; step(j, ch, nvc)) {
+        const int k = ch * 32 + lane;
+        if (k >= m) continue;
+        const RingRot<S> rk = rot[i0 + j];
+        S* vp = colV + (size_t)cur[j] * m + k;
+        S* vq = colV + (size_t)cur[w + j] * m + k;
+        const S a = *vp, b = *vq;
+        *vp = sc<S>::sub(sc<S>::mul(a, rk.uc), sc<S>::scale(b, rk.s));
+        *vq = sc<S>::add(sc<S>::mul(a, rk.us), sc<S>::scale(b, rk.c));
+      }
+      __syncthreads();
+      // the outer columns to the neighbours, and the places of the next round
+      if (wl > 0) {
+        const int out_t = cur[0], out_b = cur[w + wl - 1];
+        const bool left = (warp & 2) == 0;  // warps 0, 1 (mod 4): A, V to the left; 2, 3: to the right
+        if (left ? g > 0 : g < last) {
+          S* base = (warp & 1) ? colV : colA;
+          S* dst = cl.map_shared_rank(base, left ? g - 1 : g + 1) + (size_t)nb[left ? 0 : 1] * m;
+          const S* src = base + (size_t)(left ? out_t : out_b) * m;
+          for (int k = (warp >> 2) * 32 + lane; k < m; k += NW * 8) dst[k] = src[k];
+        }
+        // first players move left, second ones right; CTA 0 keeps the fixed player at place 0 and turns
+        // its leftmost first player into a second one, the last CTA its rightmost second into a first
+        for (int j = tid; j < wl; j += kRingThreads) {
+          if (np == 1) {  // one pair: nobody moves
+            nxt[0] = cur[0];
+            nxt[w] = cur[w];
+            continue;
+          }
+          nxt[j] = j + 1 < wl ? cur[j + 1] : (g == last ? out_b : cur[2 * w]);
+          if (g == 0)
+            nxt[w + j] = j == 0 ? cur[w] : (j == 1 ? out_t : cur[w + j - 1]);
+          else
+            nxt[w + j] = j == 0 ? cur[2 * w + 1] : cur[w + j - 1];
+        }
+        if (tid == 0) {
+          // the slots the sent columns leave are the free ones of the next round
+          nxt[2 * w] = g == 0 ? out_b : out_t;
+          nxt[2 * w + 1] = g == last ? out_t : out_b;
+        }
+      }
+      csync();
+    }
+  }
+  // sort ascending by eigenvalue (rank sort, ties by index), phase-normalise
+  const int* sl = slots + par * (2 * w + 2);
+  for (int e = tid; e < 2 * wl * G; e += kRingThreads) {
+    const int c = e % (2 * wl), to = e / (2 * wl);
+    const int pl = c < wl ? first_of(0, i0 + c) : second_of(0, i0 + c - wl);
+    if (pl >= m) continue;
+    R* dst = G > 1 ? cl.map_shared_rank(lam, to) : lam;
+    dst[pl] = sc<S>::re(colA[(size_t)sl[c < wl ? c : w + c - wl] * m + pl]);
+  }
+  csync();
+  for (int c = warp; c < 2 * wl; c += NW) {
+    const int pl = c < wl ? first_of(0, i0 + c) : second_of(0, i0 + c - wl);
+    if (pl >= m) continue;
+    const R li = lam[pl];
+    int rank = 0;
+    for (int j = lane; j < m; j += 32) rank += (lam[j] < li) || (lam[j] == li && j < pl);
+    const S* v = colV + (size_t)sl[c < wl ? c : w + c - wl] * m;
+    // phase of the first largest-magnitude component
+    R best = R(-1);
+    int kb = m;
+    for (int k = lane; k < m; k += 32) {
+      const R a = sc<S>::abs2(v[k]);
+      if (a > best) {
+        best = a;
+        kb = k;
+      }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      rank += __shfl_xor_sync(0xffffffffu, rank, o);
+      const R ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int ok = __shfl_xor_sync(0xffffffffu, kb, o);
+      if (ob > best || (ob == best && ok < kb)) {
+        best = ob;
+        kb = ok;
+      }
+    }
+    if (kb >= m) kb = 0;  // (nothing but NaN)
+    const R nb2 = sqrt(best);
+    S ph = sc<S>::from_re(R(1));
+    if (nb2 > R(0)) ph = sc<S>::scale(sc<S>::conj(v[kb]), R(1) / nb2);
+    S* vo = Vout + d.off + (int64_t)rank * m;
+    for (int k = lane; k < m; k += 32) vo[k] = k == kb && nb2 > R(0) ? sc<S>::from_re(nb2) : sc<S>::mul(v[k], ph);
+    if (lane == 0) lamall[d.voff + rank] = (double)li;
+  }
+  if (g == 0 && tid == 0) sweeps_out[t] = converged ? sweeps : -1;
+}
+
+// Clusters of the ring kernel that run at once for the largest order max_m on clusters of G (0: the columns
+// do not fit), cached per device and shape.
+template <typename S>
+static int ring_clusters(int max_m, int G) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, int, int>, int> known;
+  const size_t smem = ring_smem<S>(max_m, ring_places(max_m, G));
+  int dev = 0;
+  if (smem > 224 * 1024 || cudaGetDevice(&dev) != cudaSuccess) return 0;
+  std::lock_guard<std::mutex> lk(mu);
+  const auto key = std::make_tuple(dev, max_m, G);
+  const auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  auto kern = jacobi_ring_kernel<S>;
+  int nc = 0;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)G);
+  cfg.blockDim = dim3(kRingThreads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = G;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&nc, kern, &cfg);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    nc = 0;
+  }
+  if (known.size() > 4096) known.clear();
+  known[key] = nc;
+  return nc;
 }
 
 template <typename S>
@@ -794,22 +1155,8 @@ __global__ void __launch_bounds__(512) jacobi_kernel(const SmallDesc* desc, S* A
 #pragma unroll
           for (int b2 = 0; b2 < 2; ++b2)
             x[a][b2] = (ra[a] >= 0 && cb[b2] >= 0) ? A[ra[a] + (int64_t)cb[b2] * m] : sc<S>::zero();
-        // columns: [x_p, x_q] <- [x_p u c - x_q s, x_p u s + x_q c] (pair k)
-        const S uck = sc<S>::scale(rk.u, rk.c), usk = sc<S>::scale(rk.u, rk.s);
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-          const S xp = x[a][0], xq = x[a][1];
-          x[a][0] = sc<S>::sub(sc<S>::mul(xp, uck), sc<S>::scale(xq, rk.s));
-          x[a][1] = sc<S>::add(sc<S>::mul(xp, usk), sc<S>::scale(xq, rk.c));
-        }
-        // rows: [x_p; x_q] <- [conj(u c) x_p - s x_q; conj(u s) x_p + c x_q] (pair i)
-        const S ucc = sc<S>::conj(sc<S>::scale(ri.u, ri.c)), usc = sc<S>::conj(sc<S>::scale(ri.u, ri.s));
-#pragma unroll
-        for (int b2 = 0; b2 < 2; ++b2) {
-          const S xp = x[0][b2], xq = x[1][b2];
-          x[0][b2] = sc<S>::sub(sc<S>::mul(ucc, xp), sc<S>::scale(xq, ri.s));
-          x[1][b2] = sc<S>::add(sc<S>::mul(usc, xp), sc<S>::scale(xq, ri.c));
-        }
+        rotate_block<S, R>(x, ri.c, ri.s, sc<S>::scale(ri.u, ri.c), sc<S>::scale(ri.u, ri.s), rk.c, rk.s,
+                           sc<S>::scale(rk.u, rk.c), sc<S>::scale(rk.u, rk.s));
         if (i == k && ri.p >= 0 && ri.q >= 0) {  // the rotated pivot block: exact zeros, real diagonal
           x[0][1] = sc<S>::zero();
           x[1][0] = sc<S>::zero();
@@ -875,6 +1222,32 @@ template <typename S>
 int launch_jacobi(int nblk, const SmallDesc* d_desc, int max_m, S* A, S* Aalt, S* Vwork, S* Vout, double* lam,
                   double tol, int max_sweeps, int* sweeps_out, double* scratch, cudaStream_t st) {
   if (nblk <= 0) return 0;
+  // The ring kernel on the smallest cluster whose CTAs have about one 2 x 2 block per thread (a barrier costs
+  // as much as a block), fewer CTAs when the blocks' clusters would not all be resident; more when
+  // only that makes the columns fit.
+  int G = 1;
+  const int64_t np = (max_m + 1) / 2;
+  while (G < 16 && np * np >= 2 * (int64_t)G * kRingThreads) G *= 2;
+  while (G > 1 && ring_clusters<S>(max_m, G) < nblk && ring_clusters<S>(max_m, G / 2) > 0) G /= 2;
+  while (G < 16 && ring_clusters<S>(max_m, G) < 1) G *= 2;
+  if (ring_clusters<S>(max_m, G) > 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nblk * (unsigned)G);
+    cfg.blockDim = dim3(kRingThreads);
+    cfg.dynamicSmemBytes = ring_smem<S>(max_m, ring_places(max_m, G));
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = G;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    PD_CK(cudaLaunchKernelEx(&cfg, jacobi_ring_kernel<S>, d_desc, (const S*)A, Vout, lam, tol, max_sweeps, sweeps_out));
+    count_launch();
+    g_last_ctas = G;
+    return 0;
+  }
   const size_t smem = sizeof(Rot<S>) * (size_t)((max_m + 2) / 2);
   if (smem > 48 * 1024) PD_CK(cudaFuncSetAttribute(jacobi_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   return launch_cluster_t(false, jacobi_kernel<S>, nblk, smem, 512, st, d_desc, A, Aalt, Vwork, Vout, lam, tol, max_sweeps,
@@ -1170,7 +1543,7 @@ int small_gemm(bool conjA, const std::vector<SmallDesc>& blk, int max_m, S* cons
 // others are left to the cluster treatment.
 template <typename S>
 __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall, const S* Pall, double* lamall,
-                                                  double* est_out, double* reach_all) {
+                                                  double* est_out, double* reach_all, int balanced) {
   // One refinement step (Ogita and Aishima, 2018) for block t, given S = V^H A V
   // and P = V^H V of the current approximate eigenvectors V:
   //   lambda_i = S_ii / P_ii, R = I - P, c_ij = S_ij + lambda_j R_ij,
@@ -1185,6 +1558,10 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
   // being separated, or -inf.  Grid (blocks, kOaSplit): CTA y of a block handles
   // columns y*nw + warp (stride kOaSplit*nw); est_out[block * kOaSplit + y] is its
   // partial maximum.  Every CTA computes the (identical) lambda itself.
+  // balanced (for a last step after coarser ones): E_ij as R_ij / 2 + (S_ij + (lambda_i + lambda_j)/2 R_ij) /
+  // (lambda_j - lambda_i), the same value with an exactly antihermitian second term, so that its rounding does
+  // not touch the orthogonality; and couplings below 1e-14 max|lambda| of pairs far apart (|gap| > 1e8 |c_ij|)
+  // are corrected as well: the coarser steps leave some of that size.
   const SmallDesc d = desc[blockIdx.x];
   const int m = d.m;
   S* Sm = Sall + d.off;
@@ -1230,11 +1607,16 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
         const double gap = lj - li;
         if (ca > tiny) {
           if (fabs(gap) > 4.0 * ca) {
-            ev = sc<S>::scale(c, 1.0 / gap);
+            if (balanced)
+              ev = sc<S>::add(ev, sc<S>::scale(sc<S>::add(Sm[e], sc<S>::scale(r, 0.5 * (li + lj))), 1.0 / gap));
+            else
+              ev = sc<S>::scale(c, 1.0 / gap);
             emax = fmax(emax, sqrt(sc<S>::abs2(ev)));
           } else if (li >= lj) {
             rj = fmax(rj, li);
           }
+        } else if (balanced && fabs(gap) > 1e8 * ca) {
+          ev = sc<S>::add(ev, sc<S>::scale(sc<S>::add(Sm[e], sc<S>::scale(r, 0.5 * (li + lj))), 1.0 / gap));
         }
       }
       Sm[e] = ev;
@@ -1420,6 +1802,11 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
   // separated pairs.  A block leaves the batch after the step whose correction was
   // below kRefineTol (what remains is of the order of its square); at most
   // kRefineSteps steps.
+  // w.rough: steps whose correction will be above kRefineTol by the square of the last one run their products
+  // in float-float: the next step corrects what that leaves (a block leaves only after a step in FP64, so S, P,
+  // lambda and the last correction are computed as before).  One of three or four steps is then in FP64
+  // (8 blocks of 267 complex columns: 4.4 ms a step against 2.4).
+  double est_max = 1.0;
   S* V = w.Vd;
   S* Vn = w.Vw;
   std::vector<double> drel(nblk, 1.0), est(nblk), estp((size_t)nblk * kOaSplit);
@@ -1427,6 +1814,8 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
   for (int t = 0; t < nblk; ++t) act[t] = t;
   for (int it = 0; it < kRefineSteps && !act.empty(); ++it) {
     const int na = (int)act.size();
+    const bool rough = w.rough && it + 1 < kRefineSteps && est_max * est_max > kRefineTol;
+    const int ff = w.ff || rough;
     std::vector<SmallDesc> sub_d(na);
     for (int q = 0; q < na; ++q) sub_d[q] = all[act[q]];
     const SmallDesc* dd = d_desc;
@@ -1436,17 +1825,17 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
     }
     {
       S* abc[3] = {A, V, w.T};  // T = A V
-      PD_TRY(small_gemm<S>(false, sub_d, max_m, abc, 0, 0, w.items, st, w.ff));
+      PD_TRY(small_gemm<S>(false, sub_d, max_m, abc, 0, 0, w.items, st, ff));
     }
     {
       S* abc[3] = {V, w.T, w.W64};  // S = V^H A V  (in W64)
-      PD_TRY(small_gemm<S>(true, sub_d, max_m, abc, 1, 0, w.items, st, w.ff));
+      PD_TRY(small_gemm<S>(true, sub_d, max_m, abc, 1, 0, w.items, st, ff));
     }
     {
       S* abc[3] = {V, V, w.T};  // P = V^H V  (in T)
-      PD_TRY(small_gemm<S>(true, sub_d, max_m, abc, 1, 0, w.items, st, w.ff));
+      PD_TRY(small_gemm<S>(true, sub_d, max_m, abc, 1, 0, w.items, st, ff));
     }
-    oa_kernel<S><<<dim3(na, kOaSplit), 256, 0, st>>>(dd, w.W64, w.T, w.lam32, w.delta, w.reach);
+    oa_kernel<S><<<dim3(na, kOaSplit), 256, 0, st>>>(dd, w.W64, w.T, w.lam32, w.delta, w.reach, w.rough);
     PD_CK_LAUNCH();
     for (auto& b : sub_d)
       PD_CK(cudaMemcpyAsync(Vn + b.off, V + b.off, sizeof(S) * (size_t)b.m * b.m, cudaMemcpyDeviceToDevice, st));
@@ -1459,7 +1848,7 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
         it2[q] = GemmItem<S>{V + o, w.W64 + o, Vn + o, m, m, m, m, m, m, 0};
       }
       PD_CK(cudaMemcpyAsync(w.items, it2.data(), sizeof(GemmItem<S>) * na, cudaMemcpyHostToDevice, st));
-      PD_TRY(launch_gemm<S>(false, na, w.items, max_m, max_m, max_m, one, one, 1, nullptr, 0, st, 0, 0, w.ff));
+      PD_TRY(launch_gemm<S>(false, na, w.items, max_m, max_m, max_m, one, one, 1, nullptr, 0, st, 0, 0, ff));
     }
     for (auto& b : sub_d)
       PD_CK(cudaMemcpyAsync(V + b.off, Vn + b.off, sizeof(S) * (size_t)b.m * b.m, cudaMemcpyDeviceToDevice, st));
@@ -1471,9 +1860,13 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
     }
     if (rep) rep->refine_steps += 1;
     std::vector<int> next;
+    est_max = 0.0;
     for (int q = 0; q < na; ++q) {
       drel[act[q]] = est[q];
-      if (!(est[q] < kRefineTol)) next.push_back(act[q]);
+      if (!(est[q] < kRefineTol) || (rough && !w.ff)) {
+        next.push_back(act[q]);
+        est_max = std::max(est_max, est[q]);
+      }
     }
     act.swap(next);
   }

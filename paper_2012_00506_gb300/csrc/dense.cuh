@@ -93,6 +93,7 @@ struct EighScratch {
   int* csweeps;
   double* cjscratch;
   int ff = 0;               // float-float products in the refinement (set by the caller)
+  int rough = 0;            // FP64 refinement with its first steps in float-float (set by the caller)
 };
 // columns i0..i0+c-1 of the m x m block at element offset off (eigenvalues at voff)
 struct ClusterRef {

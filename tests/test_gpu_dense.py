@@ -71,3 +71,43 @@ def test_eigh_matches_oracle(device, cplx):
         for k in range(len(lo)):
             if gaps[k] > 1e-6 * nrm:
                 assert np.max(np.abs(V[:, k] - Vo[:, k])) < 1e-10 * nrm / gaps[k]
+
+
+# The ring form of the Jacobi stage: orders around one and two places per CTA, odd ones (a dummy player),
+# uneven blocks in one call, an order whose columns do not fit the cluster (complex 460), and the tiles of the
+# products (16 and 32 x 64) at their edges.
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("sizes", [[1], [2, 3, 4, 5], [15, 16, 17, 31, 33], [65, 7, 66], [129, 128, 200, 1], [271],
+                                   [460]])
+def test_eigh_orders(device, sizes, cplx):
+    import torch
+    import paper_2012_00506_gb300 as pk
+    rng = np.random.default_rng(sum(sizes))
+    mats = []
+    for m in sizes:
+        A = rng.normal(size=(m, m)) + (1j * rng.normal(size=(m, m)) if cplx else 0)
+        mats.append(0.5 * (A + A.conj().T))
+    out = pk.eigh([torch.from_numpy(A).to(device) for A in mats])
+    for A, (lam, V) in zip(mats, out):
+        lam, V = lam.cpu().numpy(), V.cpu().numpy()
+        nrm = max(1.0, np.linalg.norm(A))
+        assert np.max(np.abs(lam - np.linalg.eigvalsh(A))) < 1e-13 * nrm
+        assert np.max(np.abs(A @ V - V * lam)) < 1e-12 * nrm
+        assert np.max(np.abs(V.conj().T @ V - np.eye(A.shape[0]))) < 1e-12
+
+
+def test_eigh_degenerate_spectra(device):
+    """Multiple eigenvalues, a diagonal block and one far from the others in scale."""
+    import torch
+    import paper_2012_00506_gb300 as pk
+    rng = np.random.default_rng(3)
+    Q, _ = np.linalg.qr(rng.normal(size=(90, 90)))
+    mats = [np.eye(40), np.diag(np.arange(33.0) // 3), Q @ np.diag(np.repeat(np.arange(9.0), 10)) @ Q.T,
+            1e6 * np.outer(Q[0], Q[0]) + np.diag(np.linspace(0, 1, 90))]
+    mats = [0.5 * (A + A.T) for A in mats]
+    for A, (lam, V) in zip(mats, pk.eigh([torch.from_numpy(A).to(device) for A in mats])):
+        lam, V = lam.cpu().numpy(), V.cpu().numpy()
+        nrm = max(1.0, np.linalg.norm(A))
+        assert np.max(np.abs(lam - np.linalg.eigvalsh(A))) < 1e-13 * nrm
+        assert np.max(np.abs(A @ V - V * lam)) < 1e-12 * nrm
+        assert np.max(np.abs(V.T @ V - np.eye(A.shape[0]))) < 1e-12
