@@ -23,16 +23,20 @@ namespace cg = cooperative_groups;
 namespace pdeshep {
 
 // ---------------------------------------------------------------------------
-// batched GEMM, 32 x 32 output tiles, 32-deep k tiles, 256 threads (2 x 2 each).
+// batched GEMM, 16 x 16 output tiles, 32-deep k tiles, 256 threads (one output each).
 // FP64 runs at about 2 FMA per clock per SM on this part, so shared-memory
 // bandwidth is never the limit and small tiles cost nothing; they cut the
-// padding of m0 x m0 outputs (m0 = 267 pads to 288 instead of 320).
-// herm: the product is Hermitian (Gram, projection): only tiles with
-//   ti <= tj are computed and the lower triangle is filled by conjugation.
+// padding of m0 x m0 outputs (m0 = 267 pads to 272) and spread the few tiles of
+// one or two blocks over the SMs (one 267 x 267 complex block: 32 x 32 tiles
+// occupy 81 SMs for 311 us, 16 x 16 tiles all of them for 160 us).
+// herm: the product is Hermitian (Gram, projection): only the tiles of 32 x 32
+//   blocks on or above the diagonal are computed and the blocks below it are
+//   filled by conjugation.
 // triB: B is upper triangular (R^{-1}): the k loop stops at the tile's last
 //   column.
 // ---------------------------------------------------------------------------
-constexpr int GBM = 32, GBN = 32, GBK = 32;
+constexpr int GBM = 16, GBN = 16, GBK = 32;
+constexpr int GHB = 32 / GBM;  // tiles per block of the Hermitian shortcut
 
 template <typename S, bool CA>
 __global__ void __launch_bounds__(256) gemm_kernel(const GemmItem<S>* items, S alpha, S beta, int splits,
@@ -43,18 +47,14 @@ __global__ void __launch_bounds__(256) gemm_kernel(const GemmItem<S>* items, S a
   const int tm = (it.m + GBM - 1) / GBM, tn = (it.n + GBN - 1) / GBN;
   if ((int)blockIdx.x >= tm * tn) return;
   const int ti = blockIdx.x % tm, tj = blockIdx.x / tm;
-  if (herm && ti > tj) return;
+  if (herm && ti / GHB > tj / GHB) return;
   const int i0 = ti * GBM, j0 = tj * GBN;
   const int split = blockIdx.z;
-  const int klim = triB ? min(it.k, j0 + GBN) : it.k;
+  const int klim = triB ? min(it.k, (tj / GHB + 1) * 32) : it.k;
   const int kper = ((klim + splits - 1) / splits + GBK - 1) / GBK * GBK;
   const int kb = split * kper, ke = min(klim, kb + kper);
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  S acc[2][2];
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int c = 0; c < 2; ++c) acc[a][c] = sc<S>::zero();
+  S acc = sc<S>::zero();
   for (int k0 = kb; k0 < ke; k0 += GBK) {
     for (int e = tid; e < GBM * GBK; e += 256) {
       int i, kk;
@@ -79,31 +79,21 @@ __global__ void __launch_bounds__(256) gemm_kernel(const GemmItem<S>* items, S a
     __syncthreads();
 #pragma unroll 8
     for (int kk = 0; kk < GBK; ++kk) {
-      const S a0 = As[kk][ty], a1 = As[kk][ty + 16];
-      const S b0 = Bs[kk][tx], b1 = Bs[kk][tx + 16];
-      sc<S>::fma_(acc[0][0], a0, b0);
-      sc<S>::fma_(acc[0][1], a0, b1);
-      sc<S>::fma_(acc[1][0], a1, b0);
-      sc<S>::fma_(acc[1][1], a1, b1);
+      sc<S>::fma_(acc, As[kk][tx], Bs[kk][ty]);
     }
     __syncthreads();
   }
-#pragma unroll
-  for (int q = 0; q < 2; ++q)
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int i = i0 + ty + 16 * q, j = j0 + tx + 16 * r;
-      if (i >= it.m || j >= it.n) continue;
-      if (splits > 1) {
-        part[split * part_stride + it.part_off + i + (int64_t)j * it.m] = acc[q][r];
-      } else {
-        S* cp = it.C + i + (int64_t)j * it.ldc;
-        S v = sc<S>::mul(alpha, acc[q][r]);
-        if (sc<S>::re(beta) != 0.0 || sc<S>::abs2(beta) != 0.0) v = sc<S>::add(v, sc<S>::mul(beta, *cp));
-        *cp = v;
-        if (herm && ti < tj) it.C[j + (int64_t)i * it.ldc] = sc<S>::conj(v);
-      }
-    }
+  const int i = i0 + tx, j = j0 + ty;
+  if (i >= it.m || j >= it.n) return;
+  if (splits > 1) {
+    part[split * part_stride + it.part_off + i + (int64_t)j * it.m] = acc;
+  } else {
+    S* cp = it.C + i + (int64_t)j * it.ldc;
+    S v = sc<S>::mul(alpha, acc);
+    if (sc<S>::re(beta) != 0.0 || sc<S>::abs2(beta) != 0.0) v = sc<S>::add(v, sc<S>::mul(beta, *cp));
+    *cp = v;
+    if (herm && ti / GHB < tj / GHB) it.C[j + (int64_t)i * it.ldc] = sc<S>::conj(v);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -115,10 +105,13 @@ __global__ void __launch_bounds__(256) gemm_kernel(const GemmItem<S>* items, S a
 // the low word and lo*lo is dropped.  Relative accuracy of a length-K dot
 // product is about 2^-48 sqrt(K) in practice, far inside the 1e-10 residual
 // target; the exponent range is FP32's (operands above ~1e-19 in magnitude
-// keep full precision).  Tiles: 64 x 64 outputs per CTA of 512 threads, 4 x 2
-// per thread, k-steps of 16 staged in shared memory as (hi, lo) pairs.
+// keep full precision).  Tiles: 32 x 64 outputs per CTA of 256 threads, 4 x 2
+// per thread, k-steps of 16 staged in shared memory as (hi, lo) pairs (with 64 x 64
+// tiles one block of 267 is 25 CTAs on 152 SMs: its products in one refinement
+// step 660 -> 400 us).  herm: 64 x 64 blocks on or above the diagonal.
 // ---------------------------------------------------------------------------
-constexpr int FBM = 64, FBN = 64, FBK = 16, FFT = 512;
+constexpr int FBM = 32, FBN = 64, FBK = 16, FFT = 256;
+constexpr int FHB = 64 / FBM;
 
 template <typename S>
 struct ffv;  // a split operand in shared memory
@@ -190,13 +183,13 @@ __global__ void __launch_bounds__(FFT) ffgemm_kernel(const GemmItem<S>* items, S
   const int tm = (it.m + FBM - 1) / FBM, tn = (it.n + FBN - 1) / FBN;
   if ((int)blockIdx.x >= tm * tn) return;
   const int ti = blockIdx.x % tm, tj = blockIdx.x / tm;
-  if (herm && ti > tj) return;
+  if (herm && ti / FHB > tj) return;
   const int i0 = ti * FBM, j0 = tj * FBN;
   const int split = blockIdx.z;
   const int klim = triB ? min(it.k, j0 + FBN) : it.k;
   const int kper = ((klim + splits - 1) / splits + FBK - 1) / FBK * FBK;
   const int kb = split * kper, ke = min(klim, kb + kper);
-  // 512 threads: thread (tx, ty) owns rows ty + 16 q (q < 4) and columns tx + 32 r (r < 2)
+  // thread (tx, ty) owns rows ty + 8 q (q < 4) and columns tx + 32 r (r < 2)
   const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
   constexpr int NA = (FBM * FBK) / FFT, NB = (FBN * FBK) / FFT;
   S ra[NA], rb[NB];
@@ -252,7 +245,7 @@ __global__ void __launch_bounds__(FFT) ffgemm_kernel(const GemmItem<S>* items, S
     for (int kk = 0; kk < FBK; ++kk) {
       V a[4], b[2];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) a[q] = As[stg][kk][ty + 16 * q];
+      for (int q = 0; q < 4; ++q) a[q] = As[stg][kk][ty + 8 * q];
 #pragma unroll
       for (int r = 0; r < 2; ++r) b[r] = Bs[stg][kk][tx + 32 * r];
 #pragma unroll
@@ -268,7 +261,7 @@ __global__ void __launch_bounds__(FFT) ffgemm_kernel(const GemmItem<S>* items, S
   for (int q = 0; q < 4; ++q)
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-      const int i = i0 + ty + 16 * q, j = j0 + tx + 32 * r;
+      const int i = i0 + ty + 8 * q, j = j0 + tx + 32 * r;
       if (i >= it.m || j >= it.n) continue;
       const S val = ff_val(acc[q][r]);
       if (splits > 1) {
@@ -278,7 +271,7 @@ __global__ void __launch_bounds__(FFT) ffgemm_kernel(const GemmItem<S>* items, S
         S v = sc<S>::mul(alpha, val);
         if (sc<S>::re(beta) != 0.0 || sc<S>::abs2(beta) != 0.0) v = sc<S>::add(v, sc<S>::mul(beta, *cp));
         *cp = v;
-        if (herm && ti < tj) it.C[j + (int64_t)i * it.ldc] = sc<S>::conj(v);
+        if (herm && ti / FHB < tj) it.C[j + (int64_t)i * it.ldc] = sc<S>::conj(v);
       }
     }
 }
@@ -291,7 +284,7 @@ __global__ void gemm_reduce_kernel(const GemmItem<S>* items, S alpha, S beta, in
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(e % it.m), j = (int)(e / it.m);
-    const int ti = i / GBM, tj = j / GBN;
+    const int ti = i / 32, tj = j / 32;
     if (herm && ti > tj) continue;
     S s = sc<S>::zero();
     for (int p = 0; p < splits; ++p) s = sc<S>::add(s, part[p * part_stride + it.part_off + e]);
