@@ -352,6 +352,11 @@ __device__ __forceinline__ int cl_rank() { return (int)cg::this_cluster().block_
 __device__ __forceinline__ int cl_size() { return (int)cg::this_cluster().num_blocks(); }
 __device__ __forceinline__ void cl_sync() { cg::this_cluster().sync(); }
 __device__ __forceinline__ int cl_slice() { return blockIdx.x / cl_size(); }
+// thread index over the cluster with its warps dealt to the CTAs in turn, so that fewer warps of work than the
+// cluster has still spread over its SMs
+__device__ __forceinline__ int cl_dealt() {
+  return ((threadIdx.x >> 5) * cl_size() + cl_rank()) * 32 + (threadIdx.x & 31);
+}
 
 // Per launch, with `resident`, the widest shape whose nblk clusters are all
 // resident at once (a 16-CTA cluster needs 16 SMs of one GPC, so only a few
@@ -450,6 +455,21 @@ __device__ __forceinline__ double2 shfl_s(double2 v, int src) {
   return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
 
+// v - conj(a) b
+template <typename S>
+__device__ __forceinline__ S sub_mulcj(S v, S a, S b) {
+  return sc<S>::sub(v, sc<S>::mul(sc<S>::conj(a), b));
+}
+
+// Blocked right-looking factorization in panels of 32 columns, three cluster barriers per panel: (1) CTA 0
+// factors the diagonal block, (2) every CTA solves R_JJ^H R_JK = G_JK for its columns right of the panel,
+// (3) the trailing upper triangle gets G_KK -= R_JK^H R_JK.
+// FP64 latency bounds it: a warp instruction takes its pipe 64 clocks however few lanes it has, a division or
+// a square root about 600.  So (1) keeps the block's 528 entries one per thread, packed by rows from the last one
+// up (the entries still to be updated are the first ones: no idle warps), with two CTA barriers per column,
+// where one warp with a column per lane spent 5700 clocks per column; and (2) takes the reciprocals of
+// the diagonal from (1) instead of a division per entry.  Few elements are left in the later panels, hence
+// cl_dealt().  (Measured, complex order 267: 2843 -> 848 us for one block on 16 CTAs, 3170 -> 1254 us for 8 on 8.)
 template <typename S>
 __global__ void __launch_bounds__(1024) cholesky_kernel(const SmallDesc* desc, S* Gall, int* info, double* diag0,
                                                         double* minratio) {
@@ -457,54 +477,52 @@ __global__ void __launch_bounds__(1024) cholesky_kernel(const SmallDesc* desc, S
   const SmallDesc d = desc[t];
   const int m = d.m;
   S* G = Gall + d.off;
-  const int gid = cl_rank() * blockDim.x + threadIdx.x, gsz = cl_size() * blockDim.x;
+  const int gid = cl_dealt(), gsz = cl_size() * blockDim.x;
   if (diag0) {
     for (int i = gid; i < m; i += gsz) diag0[d.voff + i] = sc<S>::re(G[i + (int64_t)i * m]);
     cl_sync();
   }
-  // Blocked right-looking factorization in panels of CB columns, three cluster
-  // barriers per panel: (1) CTA 0 factors the diagonal block in shared memory,
-  // (2) every CTA solves R_JJ^H R_JK = G_JK for its columns right of the panel,
-  // (3) the trailing upper triangle gets G_KK -= R_JK^H R_JK.
   constexpr int CB = 32;
   __shared__ S Rjj[CB][CB + 1];  // R_JJ (row, col)
-  __shared__ int sh_bad;
+  __shared__ double rinv[CB];    // 1 / R_JJ(i, i)
+  __shared__ S rowj[CB];
+  __shared__ double sh_d;
   int bad = 0;
   for (int j0 = 0; j0 < m && !bad; j0 += CB) {
     const int nb = min(CB, m - j0);
     if (cl_rank() == 0) {
-      for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-        const int r = e % nb, c = e / nb;
-        Rjj[r][c] = G[(j0 + r) + (int64_t)(j0 + c) * m];
-      }
-      if (threadIdx.x == 0) sh_bad = 0;
+      // thread e holds entry (i, c), i <= c: rows from nb - 1 up, row i at (nb-1-i)(nb-i)/2 .. (its entries
+      // with the last columns first are its neighbours' below)
+      const int e = threadIdx.x;
+      int q = 0;  // rows before this entry's: q (q + 1) / 2 <= e
+      while ((q + 1) * (q + 2) / 2 <= e) ++q;
+      const int i = nb - 1 - q, c = i + (e - q * (q + 1) / 2);
+      const bool has = e < nb * (nb + 1) / 2;
+      S v = sc<S>::zero();
+      if (has) v = G[(j0 + i) + (int64_t)(j0 + c) * m];
+      if (has && i == 0 && c == 0) sh_d = sc<S>::re(v);
+      int fail = 0;
       __syncthreads();
-      if (threadIdx.x < 32) {  // one warp factors the diagonal block; lane c owns column c
-        const int lane = threadIdx.x;
-        for (int j = 0; j < nb; ++j) {
-          const double dj = sc<S>::re(Rjj[j][j]);
-          if (!((dj > 0.0) && isfinite(dj))) {
-            if (lane == 0) sh_bad = j0 + j + 1;
-            break;
-          }
-          const double r = sqrt(dj);
-          __syncwarp();
-          if (lane > j && lane < nb) Rjj[j][lane] = sc<S>::scale(Rjj[j][lane], 1.0 / r);
-          __syncwarp();
-          if (lane > j && lane < nb)
-            for (int i = j + 1; i <= lane; ++i)
-              Rjj[i][lane] = sc<S>::sub(Rjj[i][lane], sc<S>::mul(sc<S>::conj(Rjj[j][i]), Rjj[j][lane]));
-          __syncwarp();
-          if (lane == j) Rjj[j][j] = sc<S>::from_re(r);
-          __syncwarp();
+      for (int j = 0; j < nb; ++j) {
+        const double dj = sh_d;
+        if (!((dj > 0.0) && isfinite(dj))) {
+          fail = j0 + j + 1;
+          break;
         }
+        if (has && i == j) {
+          const double r = sqrt(dj), ri = 1.0 / r;
+          v = c == j ? sc<S>::from_re(r) : sc<S>::scale(v, ri);
+          rowj[c] = v;
+        }
+        __syncthreads();
+        if (has && i > j) {
+          v = sub_mulcj(v, rowj[i], rowj[c]);
+          if (i == j + 1 && c == j + 1) sh_d = sc<S>::re(v);
+        }
+        __syncthreads();
       }
-      __syncthreads();
-      for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-        const int r = e % nb, c = e / nb;
-        if (r <= c) G[(j0 + r) + (int64_t)(j0 + c) * m] = Rjj[r][c];
-      }
-      if (threadIdx.x == 0) info[t] = sh_bad;  // provisional; rewritten below
+      if (has) G[(j0 + i) + (int64_t)(j0 + c) * m] = v;
+      if (threadIdx.x == 0) info[t] = fail;  // provisional; rewritten below
     }
     cl_sync();
     bad = info[t];
@@ -512,7 +530,9 @@ __global__ void __launch_bounds__(1024) cholesky_kernel(const SmallDesc* desc, S
     // every CTA: R_JJ into shared memory, then one warp per column k of the row panel
     for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
       const int r = e % nb, c = e / nb;
-      Rjj[r][c] = r <= c ? G[(j0 + r) + (int64_t)(j0 + c) * m] : sc<S>::zero();
+      const S v = r <= c ? G[(j0 + r) + (int64_t)(j0 + c) * m] : sc<S>::zero();
+      Rjj[r][c] = v;
+      if (r == c) rinv[r] = 1.0 / sc<S>::re(v);
     }
     __syncthreads();
     const int k0 = j0 + nb;
@@ -525,9 +545,9 @@ __global__ void __launch_bounds__(1024) cholesky_kernel(const SmallDesc* desc, S
         S g = lane < nb ? G[(j0 + lane) + (int64_t)k * m] : sc<S>::zero();
         for (int i = 0; i < nb; ++i) {
           S xi = shfl_s(g, i);
-          xi = sc<S>::scale(xi, 1.0 / sc<S>::re(Rjj[i][i]));
+          xi = sc<S>::scale(xi, rinv[i]);
           if (lane == i) g = xi;
-          if (lane > i && lane < nb) g = sc<S>::sub(g, sc<S>::mul(sc<S>::conj(Rjj[i][lane]), xi));
+          if (lane > i && lane < nb) g = sub_mulcj(g, Rjj[i][lane], xi);
         }
         if (lane < nb) {
           G[(j0 + lane) + (int64_t)k * m] = g;
@@ -538,15 +558,19 @@ __global__ void __launch_bounds__(1024) cholesky_kernel(const SmallDesc* desc, S
       }
     }
     cl_sync();
-    // trailing update of the upper triangle: G(i,k) -= sum_l conj(R(l,i)) R(l,k), k0 <= i <= k
+    // trailing update of the upper triangle: G(i,k) -= sum_l conj(R(l,i)) R(l,k), k0 <= i <= k; columns paired
+    // shortest with longest, so that the lanes of a warp are all in use
     const int tt = m - k0;
-    for (int64_t e = gid; e < (int64_t)tt * tt; e += gsz) {
-      const int i = k0 + (int)(e % tt), k = k0 + (int)(e / tt);
-      if (i > k) continue;
+    for (int64_t e = gid; e < (int64_t)((tt + 1) / 2) * (tt + 1); e += gsz) {
+      const int q = (int)(e / (tt + 1)), x = (int)(e - (int64_t)q * (tt + 1));
+      const int kk = x <= q ? q : tt - 1 - q, ii = x <= q ? x : x - q - 1;  // columns q and tt-1-q
+      if (x > q && 2 * q == tt - 1) continue;  // an odd count: the middle column once
+      const int i = k0 + ii, k = k0 + kk;
       S v = G[i + (int64_t)k * m];
+#pragma unroll 8
       for (int l = 0; l < nb; ++l) {
         const S* pl = G + (int64_t)(j0 + l) * m;
-        v = sc<S>::sub(v, sc<S>::mul(sc<S>::conj(pl[i]), pl[k]));
+        v = sub_mulcj(v, pl[i], pl[k]);
       }
       G[i + (int64_t)k * m] = v;
     }
@@ -592,6 +616,10 @@ int launch_cholesky(int nblk, const SmallDesc* d_desc, S* G, int* info, cudaStre
 // T_ij = sum_{k=i+1..j} R_ik X_kj (kept transposed in the still-unused lower
 // tile (j,i), so every index stays inside the m x m block even when the last
 // tile is partial) and X_ij = -X_ii T_ij; two cluster barriers per distance.
+// FP64-pipe bound: at distance d there are (tiles - d) x 1024 entries, so the
+// warps are dealt to the CTAs in turn (dealt in runs, the long sums of the last
+// distances shared one SM).  Complex order 267: 1448 -> 477 us for one block,
+// 1448 -> 724 us for 8.
 // ---------------------------------------------------------------------------
 template <typename S>
 __global__ void __launch_bounds__(1024) triinv_kernel(const SmallDesc* desc, const S* Rall, S* Xall) {
@@ -600,20 +628,36 @@ __global__ void __launch_bounds__(1024) triinv_kernel(const SmallDesc* desc, con
   const int m = dsc.m;
   const S* R = Rall + dsc.off;
   S* X = Xall + dsc.off;
-  const int gid = cl_rank() * blockDim.x + threadIdx.x, gsz = cl_size() * blockDim.x;
+  const int gid = cl_dealt(), gsz = cl_size() * blockDim.x;
   const int nb = (m + 31) / 32;
   for (int64_t e = gid; e < (int64_t)m * m; e += gsz) X[e] = sc<S>::zero();
   cl_sync();
-  for (int it = gid; it < nb * 32; it += gsz) {
-    const int i = it / 32, c = it % 32;
-    const int j = 32 * i + c;
-    if (j >= m) continue;
-    X[j + (int64_t)j * m] = sc<S>::from_re(1.0 / sc<S>::re(R[j + (int64_t)j * m]));
-    for (int r = c - 1; r >= 0; --r) {
-      const int row = 32 * i + r;
-      S acc = sc<S>::zero();
-      for (int k = r + 1; k <= c; ++k) sc<S>::fma_(acc, R[row + (int64_t)(32 * i + k) * m], X[32 * i + k + (int64_t)j * m]);
-      X[row + (int64_t)j * m] = sc<S>::scale(acc, -1.0 / sc<S>::re(R[row + (int64_t)row * m]));
+  // diagonal tiles: tile i on CTA i mod G, its first warp, lane = column, the tile and the inverse in shared
+  // memory (from global memory, all tiles on CTA 0, this was half of the kernel's time)
+  __shared__ S Rt[32][33], Xt[32][33];
+  __shared__ double dinv[32];
+  for (int i = cl_rank(); i < nb; i += cl_size()) {
+    const int w = min(32, m - 32 * i);
+    const S* Ri = R + 32 * i + (int64_t)(32 * i) * m;
+    __syncthreads();
+    for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
+      const int r = e & 31, c = e >> 5;
+      Rt[r][c] = r < w && c < w && r <= c ? Ri[r + (int64_t)c * m] : sc<S>::zero();
+      if (r == c && r < w) dinv[r] = -1.0 / sc<S>::re(Ri[r + (int64_t)c * m]);
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      const int c = threadIdx.x;
+      for (int r = w - 1; r >= 0; --r) {
+        S acc = sc<S>::zero();
+#pragma unroll 4
+        for (int k = r + 1; k < w; ++k)
+          if (k <= c) sc<S>::fma_(acc, Rt[r][k], Xt[k][c]);
+        Xt[r][c] = r == c ? sc<S>::from_re(-dinv[r]) : r < c ? sc<S>::scale(acc, dinv[r]) : sc<S>::zero();
+      }
+      __syncwarp();
+      for (int q = 0; q < w; ++q)  // column q, lane = row
+        if (c <= q) X[32 * i + c + (int64_t)(32 * i + q) * m] = Xt[c][q];
     }
   }
   cl_sync();

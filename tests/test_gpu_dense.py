@@ -40,6 +40,27 @@ def test_cholqr_matches_oracle(device, cplx):
         off += m
 
 
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("sizes", [[1, 31, 32, 33], [63, 64, 65, 2], [159], [97, 100, 3, 128]])
+def test_cholqr_at_panel_edges(device, cplx, sizes):
+    """Orders around the 32-column panels and tiles, one block and several.  Gaussian columns with
+    m <= n/3: the condition number of R stays below 5, its error below 25 m eps."""
+    import paper_2012_00506_gb300 as pk
+    n = 480
+    Q0 = synth.random_subspace(n, sum(sizes), 29, cplx)
+    Q, R = pk.cholqr(block_to_dev(Q0, device), sizes, passes=1)
+    Qg = block_from_dev(Q)
+    off = 0
+    for t, m in enumerate(sizes):
+        Rg = R[t].cpu().numpy()
+        Qo, Ro, info = oracle.cholqr(Q0[:, off:off + m])
+        assert info == 0
+        assert np.all(np.tril(Rg, -1) == 0)
+        assert np.max(np.abs(Rg - Ro)) < 1e-12 * np.max(np.abs(Ro))
+        assert np.max(np.abs(Qg[:, off:off + m] - Qo)) < 1e-12
+        off += m
+
+
 def test_cholqr_breakdown(device):
     import paper_2012_00506_gb300 as pk
     Q0 = np.ones((64, 3))
