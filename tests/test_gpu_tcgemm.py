@@ -132,6 +132,20 @@ def test_tensor_agrees_with_floatfloat_and_fp64(pk):
         assert np.max(np.abs(r[pk.RR_FLOATFLOAT][t].cpu().numpy() - ref)) <= 5e-13 * scale
 
 
+@pytest.mark.parametrize("cplx,n,m", [(True, 250, 33), (False, 500, 65), (False, 31, 1)])
+@pytest.mark.parametrize("s", [-530, -512, -40, 400, 509])
+def test_power_of_two_scaling_is_exact(pk, cplx, n, m, s):
+    """The digits do not see a power of two: scaled operands give the scaled result, bit for bit, rounded
+    once where it is subnormal and infinite where it overflows (one k range, so no partial sums)."""
+    X = _blocks(n, [m], cplx, 71, scales=False)
+    X[m // 2] = 0.0
+    C = pk.block_gemm(pk.GEMM_GRAM, _t(pk, X), [m])[0].cpu().numpy()
+    D = pk.block_gemm(pk.GEMM_GRAM, _t(pk, X * 2.0 ** s), [m])[0].cpu().numpy()
+    with np.errstate(over="ignore"):
+        assert np.array_equal(D.real, np.ldexp(C.real, 2 * s))
+        assert np.array_equal(D.imag, np.ldexp(C.imag, 2 * s))
+
+
 @pytest.mark.parametrize("cplx", [True, False])
 def test_update_with_badly_scaled_columns(pk, cplx):
     """X = Q T with columns of Q spanning 16 decades and T undoing the scaling (the
