@@ -9,6 +9,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <cstring>
 #include <mutex>
 #include <vector>
 
@@ -123,6 +124,49 @@ struct tcs<double2> {
   __device__ static double im(double2 v) { return v.y; }
 };
 
+// Exponents come from the high words of the encodings: an FP64 maximum holds the FP64 pipe for 64 clocks a warp
+// (a pass over 240 MB took twice its memory time, a pass with ldexp seven times).  The largest high word of finite
+// normal numbers gives row_exponent() of the maximum; a row with a subnormal, an infinity or a NaN, or one
+// whose maximum is subnormal, goes through the FP64 loop instead.
+constexpr int kSpecial = 0x7FF00000;  // as an abs_hi value: the row takes the FP64 loop
+__device__ inline int abs_hi(double x) {
+  const int hi = __double2hiint(x) & 0x7FFFFFFF;
+  return hi < 0x00100000 && (hi | __double2loint(x)) ? kSpecial : hi;
+}
+template <typename S>
+__device__ inline int abs_hi2(S v) {
+  return tcs<S>::C ? max(abs_hi(tcs<S>::re(v)), abs_hi(tcs<S>::im(v))) : abs_hi(tcs<S>::re(v));
+}
+__device__ inline int hi_exponent(int hi) { return hi ? (hi >> 20) - 1022 : 0; }
+
+// row_exponent of max |x(k)|, k < n, by the whole CTA (valid on thread 0)
+template <typename S>
+__device__ inline int column_exponent(const S* x, int64_t n) {
+  __shared__ int redi[32];
+  __shared__ double red[32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  int mi = 0;
+#pragma unroll 8
+  for (int64_t k = threadIdx.x; k < n; k += blockDim.x) mi = max(mi, abs_hi2(x[k]));
+  mi = __reduce_max_sync(0xffffffffu, mi);
+  if (lane == 0) redi[warp] = mi;
+  __syncthreads();
+  mi = 0;
+  for (int w = 0; w < nw; ++w) mi = max(mi, redi[w]);
+  if (mi < kSpecial) return hi_exponent(mi);
+  double mx = 0.0;
+  for (int64_t k = threadIdx.x; k < n; k += blockDim.x) {
+    const S v = x[k];
+    mx = fmax(mx, fmax(fabs(tcs<S>::re(v)), fabs(tcs<S>::im(v))));
+  }
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) red[warp] = mx;
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int w = 1; w < nw; ++w) mx = fmax(mx, red[w]);
+  return row_exponent(mx);
+}
+
 // per listed block of a split launch
 struct SplitInfo {
   int64_t x_off;  // operand offset (elements of S)
@@ -146,18 +190,8 @@ __global__ void tc_colexp_kernel(int64_t n, const SplitInfo* info, const S* X, i
   const int j = blockIdx.x;
   if (j >= f.m) return;
   const S* x = X + f.x_off + (int64_t)j * n;
-  double mx = 0.0;
-  for (int64_t k = threadIdx.x; k < n; k += blockDim.x) {
-    const S v = x[k];
-    mx = fmax(mx, fmax(fabs(tcs<S>::re(v)), fabs(tcs<S>::im(v))));
-  }
-  __shared__ double red[32];
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
+  const int e = column_exponent(x, n);
   if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = fmax(mx, red[w]);
-    const int e = row_exponent(mx);
     constexpr int C = tcs<S>::C;
     if (f.a_row0 >= 0) ea[f.a_row0 + j] = e;
     if (f.b_row0 >= 0) {
@@ -217,19 +251,8 @@ __global__ void tc_colscale_kernel(int64_t n, const SplitInfo* info, const S* X,
   const int j = blockIdx.x;
   if (j >= f.m) return;
   const S* x = X + f.x_off + (int64_t)j * n;
-  double mx = 0.0;
-  for (int64_t k = threadIdx.x; k < n; k += blockDim.x) {
-    const S v = x[k];
-    mx = fmax(mx, fmax(fabs(tcs<S>::re(v)), fabs(tcs<S>::im(v))));
-  }
-  __shared__ double red[32];
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = fmax(mx, red[w]);
-    ec[f.c_off + j] = row_exponent(mx);
-  }
+  const int e = column_exponent(x, n);
+  if (threadIdx.x == 0) ec[f.c_off + j] = e;
 }
 
 // max |x(i, c)| 2^-c_c over row i (the block's m columns) -> exponent of A digit row i
@@ -239,6 +262,19 @@ __global__ void tc_rowexp_kernel(int64_t n, const SplitInfo* info, const S* X, c
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const S* x = X + f.x_off + i;
+  // the largest exponent of |x(i, c)| 2^-c_c; above the subnormal range it is frexp's (scaling by a power of two
+  // shifts it)
+  int me = -4096, special = 0;
+#pragma unroll 8
+  for (int c = 0; c < f.m; ++c) {
+    const int hi = abs_hi2(x[(int64_t)c * n]);
+    special |= hi >= kSpecial;
+    if (hi) me = max(me, hi_exponent(hi) - ec[f.c_off + c]);
+  }
+  if (!special && (me == -4096 || (me >= -1021 && me <= 1024))) {
+    ea[f.a_row0 + i] = me == -4096 ? 0 : me;
+    return;
+  }
   double mx = 0.0;
   for (int c = 0; c < f.m; ++c) {
     const S v = x[(int64_t)c * n];
@@ -347,14 +383,26 @@ __device__ inline S band_at(const S* ab, int64_t ldab, int b, int64_t n, int64_t
 }
 template <typename S>
 __global__ void tc_band_rowexp_kernel(int64_t n, int b, const S* ab, int64_t ldab, int* eband) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  // a warp per row (a thread per row: 75 us at n = 8192, b = 64, for 2 us of memory traffic; now 9 us)
+  const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
   if (i >= n) return;
+  const int64_t k0 = max((int64_t)0, i - b), k1 = min(n - 1, i + (int64_t)b);
+  int mi = 0;
+#pragma unroll 4
+  for (int64_t k = k0 + lane; k <= k1; k += 32) mi = max(mi, abs_hi2(band_at<S>(ab, ldab, b, n, i, k)));
+  mi = __reduce_max_sync(0xffffffffu, mi);
+  if (mi < kSpecial) {
+    if (lane == 0) eband[i] = hi_exponent(mi);
+    return;
+  }
   double mx = 0.0;
-  for (int64_t k = max((int64_t)0, i - b); k <= min(n - 1, i + (int64_t)b); ++k) {
+  for (int64_t k = k0 + lane; k <= k1; k += 32) {
     const S v = band_at<S>(ab, ldab, b, n, i, k);
     mx = fmax(mx, fmax(fabs(tcs<S>::re(v)), fabs(tcs<S>::im(v))));
   }
-  eband[i] = row_exponent(mx);
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) eband[i] = row_exponent(mx);
 }
 template <typename S>
 __global__ void tc_band_digits_kernel(int64_t n, int b, const S* ab, int64_t ldab, const int* eband, int lo, int W,
@@ -493,10 +541,26 @@ __device__ inline void tmem_wait16(uint32_t (&r)[16]) {
 // (n = 8192, 8 blocks of 141..267 complex columns, Gram + band + projection + update: 4.0 -> 2.53 ms, with the
 // epilogue of value() above.)
 // ---------------------------------------------------------------------------
+// item `item` (>= those asked for before with this l, the descriptor's index)
+__device__ inline TcItem item_at(const TcDesc* descs, int ndesc, int& l, int item) {
+  while (l + 1 < ndesc && item >= descs[l + 1].item0) ++l;
+  const TcDesc* d = descs + l;
+  int q = item - d->item0;
+  if (d->tm_n) return TcItem{l, q % d->tm_n, q / d->tm_n, 0};
+  const int split = q % d->nsplit;
+  q /= d->nsplit;
+  int tm = 0, left;
+  while (q >= (left = d->tn_n - d->tn_skip * tm)) {
+    q -= left;
+    ++tm;
+  }
+  return TcItem{l, tm, d->tn_skip * tm + q, split};
+}
+
 template <typename S>
 __global__ void __launch_bounds__(kThreads, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   const TcDesc* descs, const TcItem* items, int nitems, int plane_a, int plane_b, const int* ea,
+                   const TcDesc* descs, int ndesc, int nitems, int plane_a, int plane_b, const int* ea,
                    const int* eb, S* out, S* part, int* err) {
   constexpr int C = tcs<S>::C;
   extern __shared__ unsigned char smraw[];
@@ -540,14 +604,15 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0) {
     if (lane == 0) {
       // producer: all six digit tiles of A and of B for each stage of 32 reduction elements
-      int gs = 0;  // stages issued so far (all items)
+      int gs = 0, cur = 0;  // stages issued so far (all items)
       bool ok = true;
       for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-        const TcItem it = items[item];
-        const TcDesc d = descs[it.desc];
+        const TcItem it = item_at(descs, ndesc, cur, item);
+        const TcDesc& d = descs[it.desc];
         int k0;
         const int nst = stages_of(it, d, k0);
         const int ya = d.a_row0 + it.tm * BM, yb = d.b_row0 + it.tn * BN;
+        const int band = d.band, win = d.band_w, below = it.tm * BM - d.band_lo, next = d.band_half - win;
         for (int s = 0; s < nst; ++s) {
           const int G = gs, slot = G % kStages;
           if (!mbar_wait(empty0 + 8 * slot, ((G / kStages) & 1) ^ 1, err, lim)) { ok = false; break; }
@@ -556,7 +621,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int x = k0 + s * BK;
           // band products: the B coordinate follows the tile's window (it may start below 0 or end
           // past the data: TMA fills zeros there, and the band digits are zero outside the band)
-          const int xb = d.band ? x + it.tm * BM - d.band_lo + (x >= d.band_w ? d.band_half - d.band_w : 0) : x;
+          const int xb = band ? x + below + (x >= win ? next : 0) : x;
           for (int g = 0; g < kTcDigits; ++g) {
             tma_load_2d(sa + g * kATile, &tmA, x, g * plane_a + ya, full0 + 8 * slot);
             tma_load_2d(sa + kTcDigits * kATile + g * kBTile, &tmB, xb, g * plane_b + yb, full0 + 8 * slot);
@@ -615,10 +680,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       };
-      int gs = 0, gc = 0, ni = 0;  // stages, chunks and items consumed so far
+      int gs = 0, gc = 0, ni = 0, cur = 0;  // stages, chunks and items consumed so far
       for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x, ++ni) {
-        const TcItem it = items[item];
-        const TcDesc d = descs[it.desc];
+        const TcItem it = item_at(descs, ndesc, cur, item);
+        const TcDesc& d = descs[it.desc];
         int k0;
         const int nst = stages_of(it, d, k0);
         const int nchunk = (int)cdiv(nst, kChunk);
@@ -666,13 +731,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t lanebase = tbase + ((uint32_t)(32 * p) << 16);
     const int cA = C ? 16 * h : 32 * h, cB = C ? 32 + 16 * h : 32 * h + 16;
     bool ok = true;
-    int gc = 0;  // chunks read so far (all items)
+    int gc = 0, cur = 0;  // chunks read so far (all items)
     for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-      const TcItem it = items[item];
-      const TcDesc d = descs[it.desc];
-      int k0;
-      const int nst = stages_of(it, d, k0);
-      const int nchunk = (int)cdiv(nst, kChunk);
+      int nchunk;
+      {
+        const TcItem it = item_at(descs, ndesc, cur, item);
+        int k0;
+        nchunk = (int)cdiv(stages_of(it, descs[it.desc], k0), kChunk);
+      }
       // exact levels 0..4 of each entry as one integer in units of 2^-32 (|T| < 2^60 for 16384 elements)
       long long T[32];
 #pragma unroll
@@ -729,6 +795,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tfree);
+      // (asked for again: kept over the chunks, the item would spill registers)
+      const TcItem it = item_at(descs, ndesc, cur, item);
+      const TcDesc& d = descs[it.desc];
       const int i = it.tm * BM + 32 * p + lane;
       if (i < d.m) {
         const int er = ea[d.a_row0 + i] - 14;
@@ -767,8 +836,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // C = sum of the split partials (upper triangle only when tri), then written with ld ldc
 template <typename S>
-__global__ void tc_reduce_kernel(const TcDesc* descs, const int* list, S* out, const S* part, int tri) {
-  const TcDesc d = descs[list[blockIdx.y]];
+__global__ void tc_reduce_kernel(const TcDesc* descs, S* out, const S* part, int tri) {
+  const TcDesc d = descs[blockIdx.y];
   const int64_t mm = (int64_t)d.m * d.m;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < mm; idx += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(idx % d.m), j = (int)(idx / d.m);
@@ -781,8 +850,8 @@ __global__ void tc_reduce_kernel(const TcDesc* descs, const int* list, S* out, c
 
 // C(i, j) = conj(C(j, i)) for i > j; real diagonal
 template <typename S>
-__global__ void tc_mirror_kernel(const TcDesc* descs, const int* list, S* out) {
-  const TcDesc d = descs[list[blockIdx.y]];
+__global__ void tc_mirror_kernel(const TcDesc* descs, S* out) {
+  const TcDesc d = descs[blockIdx.y];
   const int64_t mm = (int64_t)d.m * d.m;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < mm; idx += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(idx % d.m), j = (int)(idx / d.m);
@@ -836,17 +905,33 @@ int make_map(CUtensorMap* map, void* base, int64_t k, int64_t pitch, int64_t row
 int rows_b_of(int cplx, int m) { return cplx ? 64 * (int)cdiv(m, 32) : (int)rup(m, 64); }
 int k2_update(int cplx, int m) { return cplx ? 2 * (int)rup(m, 16) : (int)rup(m, 32); }
 
+// the lists of one product call, in one copy: two SplitInfo and one TcDesc per block
+struct Upload {
+  std::vector<SplitInfo> info;  // those of the second operand from nl on
+  std::vector<TcDesc> desc;
+  explicit Upload(int nl) : info(2 * nl), desc(nl) {}
+  int send(const TcScratch& w, cudaStream_t st) const {
+    if ((int64_t)desc.size() > w.max_blocks) {
+      set_last_error_msg("tensor-core product: block list exceeds its scratch");
+      return PDESHEP_WORKSPACE_TOO_SMALL;
+    }
+    const size_t ni = sizeof(SplitInfo) * info.size(), nd = sizeof(TcDesc) * desc.size();
+    std::vector<char> all(ni + nd);
+    memcpy(all.data(), info.data(), ni);
+    memcpy(all.data() + ni, desc.data(), nd);
+    PD_CK(cudaMemcpyAsync(w.info, all.data(), ni + nd, cudaMemcpyHostToDevice, st));
+    return 0;
+  }
+  const SplitInfo* dinfo(const TcScratch& w, int second) const {
+    return (const SplitInfo*)w.info + (second ? desc.size() : 0);
+  }
+  const TcDesc* ddesc(const TcScratch& w) const { return (const TcDesc*)((const SplitInfo*)w.info + info.size()); }
+};
+
 template <typename S>
 int launch_products(const TcScratch& w, const CUtensorMap& ma, const CUtensorMap& mb, int plane_a, int plane_b,
-                    const std::vector<TcDesc>& hd, const std::vector<TcItem>& hi, const int* ea, S* out,
-                    cudaStream_t st) {
-  if (hi.empty()) return 0;
-  if ((int64_t)hi.size() > w.max_items || (int64_t)hd.size() > w.max_blocks) {
-    set_last_error_msg("tensor-core product: item list exceeds its scratch");
-    return PDESHEP_WORKSPACE_TOO_SMALL;
-  }
-  PD_CK(cudaMemcpyAsync(w.desc, hd.data(), sizeof(TcDesc) * hd.size(), cudaMemcpyHostToDevice, st));
-  PD_CK(cudaMemcpyAsync(w.items, hi.data(), sizeof(TcItem) * hi.size(), cudaMemcpyHostToDevice, st));
+                    const Upload& up, int nitems, const int* ea, S* out, cudaStream_t st) {
+  if (nitems <= 0) return 0;
   PD_CK(cudaFuncSetAttribute(tc_gemm_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
   static int nsm = 0;
   if (!nsm) {
@@ -854,10 +939,9 @@ int launch_products(const TcScratch& w, const CUtensorMap& ma, const CUtensorMap
     PD_CK(cudaGetDevice(&dev));
     PD_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   }
-  const int nitems = (int)hi.size();
   const int grid = std::min(nitems, std::max(1, nsm));  // one CTA per SM (222 KB shared memory each)
-  tc_gemm_kernel<S><<<(unsigned)grid, kThreads, kSmem, st>>>(ma, mb, w.desc, w.items, nitems, plane_a, plane_b, ea,
-                                                            w.eb, out, (S*)w.part, w.err);
+  tc_gemm_kernel<S><<<(unsigned)grid, kThreads, kSmem, st>>>(ma, mb, up.ddesc(w), (int)up.desc.size(), nitems, plane_a,
+                                                            plane_b, ea, w.eb, out, (S*)w.part, w.err);
   PD_CK_LAUNCH();
   return 0;
 }
@@ -873,14 +957,11 @@ TcScratch plan_tc_scratch(Arena& a, const TcShape& sh, int band_b) {
   TcScratch w;
   const int K = (int)sh.m.size();
   const int64_t n = sh.n;
-  int64_t ra = 0, rb = 0, ku = 32, tiles_h = 0, tiles_u = 0, part = 0;
+  int64_t ra = 0, rb = 0, ku = 32, part = 0;
   for (int m : sh.m) {
     ra += rup(m, BM);
     rb += rows_b_of(sh.cplx, m);
     ku = std::max<int64_t>(ku, k2_update(sh.cplx, m));
-    const int64_t tn = sh.cplx ? cdiv(m, 32) : cdiv(m, 64);
-    tiles_h += cdiv(m, BM) * tn;
-    tiles_u += cdiv(n, BM) * tn;
     part += (int64_t)m * m;
   }
   w.rows_a = ra;
@@ -899,7 +980,6 @@ TcScratch plan_tc_scratch(Arena& a, const TcShape& sh, int band_b) {
   }
   w.max_split = (int)std::max<int64_t>(8, cdiv((sh.cplx ? 2 : 1) * n, kMaxKSplit));
   w.max_blocks = K;
-  w.max_items = std::max<int64_t>(tiles_h * w.max_split, tiles_u);
   w.part_elems = part * w.max_split;
   w.da = a.take<unsigned short>((size_t)(kTcDigits * w.rows_a * w.pitch_a));
   w.du = a.take<unsigned short>((size_t)(kTcDigits * w.rows_u * w.pitch_u));
@@ -910,10 +990,7 @@ TcScratch plan_tc_scratch(Arena& a, const TcShape& sh, int band_b) {
   int64_t mtot = 0;
   for (int m : sh.m) mtot += m;
   w.ec = a.take<int>((size_t)mtot);
-  w.desc = a.take<TcDesc>((size_t)K);
-  w.items = a.take<TcItem>((size_t)w.max_items);
-  w.info = a.take<char>((size_t)K * 2 * sizeof(SplitInfo));
-  w.list = a.take<int>((size_t)K);
+  w.info = a.take<char>((size_t)K * (2 * sizeof(SplitInfo) + sizeof(TcDesc)));
   w.err = a.take<int>(1);
   w.part = a.take<char>((size_t)w.part_elems * (sh.cplx ? 16 : 8));
   if (band_b >= 0) {
@@ -942,52 +1019,28 @@ int tc_gemm_herm(const TcScratch& w, const TcShape& sh, const std::vector<int>& 
   }
   int mmax = 0;
   for (int t : blocks) mmax = std::max(mmax, sh.m[t]);
-  SplitInfo* dinfo = (SplitInfo*)w.info;
-  auto split = [&](const S* x, bool wa, bool wb) -> int {
-    std::vector<SplitInfo> inf(nl);
-    for (int l = 0; l < nl; ++l) {
-      const int t = blocks[l];
-      inf[l] = SplitInfo{x_off[t], sh.m[t], wa ? a0[t] : -1, wb ? b0[t] : -1, 0, 0};
-    }
-    PD_CK(cudaMemcpyAsync(dinfo, inf.data(), sizeof(SplitInfo) * nl, cudaMemcpyHostToDevice, st));
-    tc_colexp_kernel<S><<<dim3(mmax, nl), 256, 0, st>>>(n, dinfo, x, w.ea, w.eb);
-    PD_CK_LAUNCH();
-    tc_split_cols_kernel<S><<<dim3((unsigned)cdiv(n, 256), mmax, nl), 256, 0, st>>>(
-        n, dinfo, x, w.ea, w.eb, w.da, w.rows_a * w.pitch_a, w.pitch_a, w.db, w.rows_b * w.pitch_b, w.pitch_b);
-    PD_CK_LAUNCH();
-    return 0;
-  };
-  if (same_ab) {
-    PD_TRY(split(a, true, true));
-  } else {
-    if (!reuse_a) PD_TRY(split(a, true, false));
-    PD_TRY(split(b, false, true));
-  }
   // tiles and split-K
   const int k2 = (int)((C ? 2 : 1) * n);
-  int64_t tiles = 0;
-  auto tile_kept = [&](int m, int tm, int tn) {
-    const int cw = C ? 32 : 64;
-    return !triangle || (int64_t)cw * tn + cw - 1 >= (int64_t)BM * tm;
+  const int cw = C ? 32 : 64, tn_skip = triangle ? BM / cw : 0;  // column tiles left of the diagonal: skipped
+  auto tiles_of = [&](int m) {
+    int64_t c = 0;
+    for (int tm = 0; tm < cdiv(m, BM); ++tm) c += cdiv(m, cw) - tn_skip * tm;
+    return c;
   };
-  for (int t : blocks) {
-    const int m = sh.m[t], tn_n = (int)(C ? cdiv(m, 32) : cdiv(m, 64));
-    for (int tm = 0; tm < cdiv(m, BM); ++tm)
-      for (int tn = 0; tn < tn_n; ++tn) tiles += tile_kept(m, tm, tn);
-  }
+  int64_t tiles = 0;
+  for (int t : blocks) tiles += tiles_of(sh.m[t]);
   int nsplit = (int)std::max<int64_t>(1, cdiv(2 * 152, std::max<int64_t>(1, tiles)));
   nsplit = std::min(nsplit, (int)std::max<int64_t>(1, cdiv(k2, 512)));
   nsplit = std::max<int>(nsplit, (int)cdiv(k2, kMaxKSplit));
   nsplit = std::min(nsplit, w.max_split);
   const int ksplit = (int)rup(cdiv(k2, nsplit), kChunk * BK);
   nsplit = (int)cdiv(k2, ksplit);
-  std::vector<TcDesc> hd(nl);
-  std::vector<TcItem> hi;
-  std::vector<int> lst(nl);
-  int64_t poff = 0;
+  Upload up(nl);
+  int64_t poff = 0, nitems = 0;
   for (int l = 0; l < nl; ++l) {
     const int t = blocks[l], m = sh.m[t];
-    TcDesc& d = hd[l];
+    TcDesc& d = up.desc[l];
+    d = TcDesc{};
     d.a_row0 = a0[t];
     d.b_row0 = b0[t];
     d.m = m;
@@ -999,30 +1052,41 @@ int tc_gemm_herm(const TcScratch& w, const TcShape& sh, const std::vector<int>& 
     d.out_off = c_off[t];
     d.part_off = poff;
     poff += (int64_t)nsplit * m * m;
-    lst[l] = l;
-    const int tn_n = (int)(C ? cdiv(m, 32) : cdiv(m, 64));
-    for (int tm = 0; tm < cdiv(m, BM); ++tm)
-      for (int tn = 0; tn < tn_n; ++tn)
-        if (tile_kept(m, tm, tn))
-          for (int s = 0; s < nsplit; ++s) hi.push_back(TcItem{l, tm, tn, s});
+    d.item0 = (int)nitems;
+    d.tn_n = (int)cdiv(m, cw);
+    d.tn_skip = tn_skip;
+    nitems += tiles_of(m) * nsplit;
+    up.info[l] = SplitInfo{x_off[t], m, a0[t], same_ab ? b0[t] : -1, 0, 0};
+    up.info[nl + l] = SplitInfo{x_off[t], m, -1, b0[t], 0, 0};
   }
   if (poff > w.part_elems) {
     set_last_error_msg("tensor-core product: split partials exceed their scratch");
     return PDESHEP_WORKSPACE_TOO_SMALL;
   }
+  PD_TRY(up.send(w, st));
+  auto split = [&](const S* x, int second) -> int {
+    const SplitInfo* dinfo = up.dinfo(w, second);
+    tc_colexp_kernel<S><<<dim3(mmax, nl), 256, 0, st>>>(n, dinfo, x, w.ea, w.eb);
+    PD_CK_LAUNCH();
+    tc_split_cols_kernel<S><<<dim3((unsigned)cdiv(n, 256), mmax, nl), 256, 0, st>>>(
+        n, dinfo, x, w.ea, w.eb, w.da, w.rows_a * w.pitch_a, w.pitch_a, w.db, w.rows_b * w.pitch_b, w.pitch_b);
+    PD_CK_LAUNCH();
+    return 0;
+  };
+  if (same_ab || !reuse_a) PD_TRY(split(a, 0));
+  if (!same_ab) PD_TRY(split(b, 1));
   CUtensorMap ma, mb;
   PD_TRY(make_map(&ma, w.da, k2, w.pitch_a, kTcDigits * w.rows_a, BM));
   PD_TRY(make_map(&mb, w.db, k2, w.pitch_b, kTcDigits * w.rows_b, BN));
-  PD_TRY(launch_products<S>(w, ma, mb, (int)w.rows_a, (int)w.rows_b, hd, hi, w.ea, c, st));
-  if (nsplit > 1 || triangle) PD_CK(cudaMemcpyAsync(w.list, lst.data(), sizeof(int) * nl, cudaMemcpyHostToDevice, st));
+  PD_TRY(launch_products<S>(w, ma, mb, (int)w.rows_a, (int)w.rows_b, up, (int)nitems, w.ea, c, st));
   if (nsplit > 1) {
     const int g = (int)std::min<int64_t>(256, cdiv((int64_t)mmax * mmax, 256));
-    tc_reduce_kernel<S><<<dim3(g, nl), 256, 0, st>>>(w.desc, w.list, c, (const S*)w.part, triangle ? 1 : 0);
+    tc_reduce_kernel<S><<<dim3(g, nl), 256, 0, st>>>(up.ddesc(w), c, (const S*)w.part, triangle ? 1 : 0);
     PD_CK_LAUNCH();
   }
   if (triangle) {
     const int g = (int)std::min<int64_t>(256, cdiv((int64_t)mmax * mmax, 256));
-    tc_mirror_kernel<S><<<dim3(g, nl), 256, 0, st>>>(w.desc, w.list, c);
+    tc_mirror_kernel<S><<<dim3(g, nl), 256, 0, st>>>(up.ddesc(w), c);
     PD_CK_LAUNCH();
   }
   return 0;
@@ -1047,39 +1111,20 @@ int tc_gemm_update(const TcScratch& w, const TcShape& sh, const std::vector<int>
     mmax = std::max(mmax, sh.m[t]);
     kmax = std::max(kmax, k2_update(C, sh.m[t]));
   }
-  SplitInfo* dinfo = (SplitInfo*)w.info;
   std::vector<int> c0(K);
   for (int t = 0, c = 0; t < K; ++t) {
     c0[t] = c;
     c += sh.m[t];
   }
-  std::vector<SplitInfo> inf(nl);
-  for (int l = 0; l < nl; ++l) {
-    const int t = blocks[l];
-    inf[l] = SplitInfo{x_off[t], sh.m[t], (int)(t * npad), b0[t], k2_update(C, sh.m[t]), c0[t]};
-  }
-  PD_CK(cudaMemcpyAsync(dinfo, inf.data(), sizeof(SplitInfo) * nl, cudaMemcpyHostToDevice, st));
-  tc_colscale_kernel<S><<<dim3(mmax, nl), 256, 0, st>>>(n, dinfo, a, w.ec);
-  PD_CK_LAUNCH();
-  tc_rowexp_kernel<S><<<dim3((unsigned)cdiv(n, 256), nl), 256, 0, st>>>(n, dinfo, a, w.ec, w.eu);
-  PD_CK_LAUNCH();
-  const int mpmax = C ? kmax / 2 : kmax;
-  tc_split_rows_kernel<S><<<dim3((unsigned)cdiv(n, 32), (unsigned)cdiv(mpmax, 32), nl), 256, 0, st>>>(
-      n, dinfo, a, w.ec, w.eu, w.du, w.rows_u * w.pitch_u, w.pitch_u);
-  PD_CK_LAUNCH();
-  // T digits: the SplitInfo offsets point into the small blocks
-  std::vector<SplitInfo> tinf(inf);
-  for (int l = 0; l < nl; ++l) tinf[l].x_off = t_off[blocks[l]];
-  SplitInfo* dtinf = dinfo + nl;
-  PD_CK(cudaMemcpyAsync(dtinf, tinf.data(), sizeof(SplitInfo) * nl, cudaMemcpyHostToDevice, st));
-  tc_split_small_kernel<S><<<dim3(mmax, nl), 128, 0, st>>>(dtinf, tm, w.ec, w.eb, w.db, w.rows_b * w.pitch_u,
-                                                           w.pitch_u);
-  PD_CK_LAUNCH();
-  std::vector<TcDesc> hd(nl);
-  std::vector<TcItem> hi;
+  Upload up(nl);
+  int64_t nitems = 0;
   for (int l = 0; l < nl; ++l) {
     const int t = blocks[l], m = sh.m[t];
-    TcDesc& d = hd[l];
+    up.info[l] = SplitInfo{x_off[t], m, (int)(t * npad), b0[t], k2_update(C, m), c0[t]};
+    up.info[nl + l] = up.info[l];
+    up.info[nl + l].x_off = t_off[t];  // T digits: offsets into the small blocks
+    TcDesc& d = up.desc[l];
+    d = TcDesc{};
     d.a_row0 = (int)(t * npad);
     d.b_row0 = b0[t];
     d.m = (int)n;
@@ -1089,15 +1134,27 @@ int tc_gemm_update(const TcScratch& w, const TcShape& sh, const std::vector<int>
     d.nsplit = 1;
     d.ldc = (int)n;
     d.out_off = x_off[t];
-    d.part_off = 0;
-    const int tn_n = (int)(C ? cdiv(m, 32) : cdiv(m, 64));
-    for (int tn = 0; tn < tn_n; ++tn)
-      for (int tmi = 0; tmi < cdiv(n, BM); ++tmi) hi.push_back(TcItem{l, tmi, tn, 0});
+    d.item0 = (int)nitems;
+    d.tm_n = (int)cdiv(n, BM);
+    nitems += cdiv(n, BM) * cdiv(m, C ? 32 : 64);
   }
+  PD_TRY(up.send(w, st));
+  const SplitInfo* dinfo = up.dinfo(w, 0);
+  tc_colscale_kernel<S><<<dim3(mmax, nl), 256, 0, st>>>(n, dinfo, a, w.ec);
+  PD_CK_LAUNCH();
+  tc_rowexp_kernel<S><<<dim3((unsigned)cdiv(n, 256), nl), 256, 0, st>>>(n, dinfo, a, w.ec, w.eu);
+  PD_CK_LAUNCH();
+  const int mpmax = C ? kmax / 2 : kmax;
+  tc_split_rows_kernel<S><<<dim3((unsigned)cdiv(n, 32), (unsigned)cdiv(mpmax, 32), nl), 256, 0, st>>>(
+      n, dinfo, a, w.ec, w.eu, w.du, w.rows_u * w.pitch_u, w.pitch_u);
+  PD_CK_LAUNCH();
+  tc_split_small_kernel<S><<<dim3(mmax, nl), 128, 0, st>>>(up.dinfo(w, 1), tm, w.ec, w.eb, w.db, w.rows_b * w.pitch_u,
+                                                           w.pitch_u);
+  PD_CK_LAUNCH();
   CUtensorMap ma, mb;
   PD_TRY(make_map(&ma, w.du, w.pitch_u, w.pitch_u, kTcDigits * w.rows_u, BM));
   PD_TRY(make_map(&mb, w.db, w.pitch_u, w.pitch_u, kTcDigits * w.rows_b, BN));
-  return launch_products<S>(w, ma, mb, (int)w.rows_u, (int)w.rows_b, hd, hi, w.eu, c, st);
+  return launch_products<S>(w, ma, mb, (int)w.rows_u, (int)w.rows_b, up, (int)nitems, w.eu, c, st);
 }
 
 template <typename S>
@@ -1106,7 +1163,7 @@ int tc_band_split(const TcScratch& w, int64_t n, int b, const void* band, int64_
     set_last_error_msg("tensor-core band product: scratch planned without the band");
     return PDESHEP_WORKSPACE_TOO_SMALL;
   }
-  tc_band_rowexp_kernel<S><<<(unsigned)cdiv(n, 256), 256, 0, st>>>(n, b, (const S*)band, ldab, w.eband);
+  tc_band_rowexp_kernel<S><<<(unsigned)cdiv(n, 8), 256, 0, st>>>(n, b, (const S*)band, ldab, w.eband);
   PD_CK_LAUNCH();
   tc_band_digits_kernel<S><<<(unsigned)w.rows_band, 128, 0, st>>>(
       n, b, (const S*)band, ldab, w.eband, (int)w.band_lo, (int)w.band_w, w.dband, w.rows_band * w.pitch_band,
@@ -1131,24 +1188,13 @@ int tc_band_matmul(const TcScratch& w, const TcShape& sh, const std::vector<int>
   int mmax = 0;
   for (int t : blocks) mmax = std::max(mmax, sh.m[t]);
   const int64_t pitch = (C ? 2 : 1) * w.band_half;
-  SplitInfo* dinfo = (SplitInfo*)w.info;
-  std::vector<SplitInfo> inf(nl);
-  for (int l = 0; l < nl; ++l) {
-    const int t = blocks[l];
-    inf[l] = SplitInfo{x_off[t], sh.m[t], -1, b0[t], 0, 0};
-  }
-  PD_CK(cudaMemcpyAsync(dinfo, inf.data(), sizeof(SplitInfo) * nl, cudaMemcpyHostToDevice, st));
-  tc_colexp_kernel<S><<<dim3(mmax, nl), 256, 0, st>>>(n, dinfo, X, w.ea, w.eb);
-  PD_CK_LAUNCH();
-  tc_split_xcols_kernel<S><<<dim3((unsigned)cdiv(w.band_half, 256), mmax, nl), 256, 0, st>>>(
-      n, w.band_half, dinfo, X, w.eb, w.db, w.rows_b * pitch, pitch);
-  PD_CK_LAUNCH();
-  std::vector<TcDesc> hd(nl);
-  std::vector<TcItem> hi;
+  Upload up(nl);
+  int64_t nitems = 0;
   const int k2 = (int)((C ? 2 : 1) * w.band_w);
   for (int l = 0; l < nl; ++l) {
     const int t = blocks[l], m = sh.m[t];
-    TcDesc& d = hd[l];
+    up.info[l] = SplitInfo{x_off[t], m, -1, b0[t], 0, 0};
+    TcDesc& d = up.desc[l];
     d = TcDesc{};
     d.a_row0 = 0;
     d.b_row0 = b0[t];
@@ -1163,14 +1209,21 @@ int tc_band_matmul(const TcScratch& w, const TcShape& sh, const std::vector<int>
     d.band_lo = (int)w.band_lo;
     d.band_w = (int)w.band_w;
     d.band_half = (int)w.band_half;
-    const int tn_n = (int)(C ? cdiv(m, 32) : cdiv(m, 64));
-    for (int tn = 0; tn < tn_n; ++tn)
-      for (int tmi = 0; tmi < cdiv(n, BM); ++tmi) hi.push_back(TcItem{l, tmi, tn, 0});
+    d.item0 = (int)nitems;
+    d.tm_n = (int)cdiv(n, BM);
+    nitems += cdiv(n, BM) * cdiv(m, C ? 32 : 64);
   }
+  PD_TRY(up.send(w, st));
+  const SplitInfo* dinfo = up.dinfo(w, 0);
+  tc_colexp_kernel<S><<<dim3(mmax, nl), 256, 0, st>>>(n, dinfo, X, w.ea, w.eb);
+  PD_CK_LAUNCH();
+  tc_split_xcols_kernel<S><<<dim3((unsigned)cdiv(w.band_half, 256), mmax, nl), 256, 0, st>>>(
+      n, w.band_half, dinfo, X, w.eb, w.db, w.rows_b * pitch, pitch);
+  PD_CK_LAUNCH();
   CUtensorMap ma, mb;
   PD_TRY(make_map(&ma, w.dband, k2, w.pitch_band, kTcDigits * w.rows_band, BM));
   PD_TRY(make_map(&mb, w.db, pitch, pitch, kTcDigits * w.rows_b, BN));
-  return launch_products<S>(w, ma, mb, (int)w.rows_band, (int)w.rows_b, hd, hi, w.eband, Y, st);
+  return launch_products<S>(w, ma, mb, (int)w.rows_band, (int)w.rows_b, up, (int)nitems, w.eband, Y, st);
 }
 
 int tc_set_wait_polls(unsigned polls) {

@@ -52,6 +52,9 @@ struct TcDesc {
   // at 128 tm - band_lo ([Re | Im] windows for complex), B rows hold whole columns of X
   // ([Re | -Im] and [Im | Re] halves of band_half elements each); 0 for the other products
   int band, band_lo, band_w, band_half;
+  // work items (one tile over one k range each) item0, item0 + 1, ... of this block: row tiles fastest
+  // (tm_n > 0), or k ranges fastest, then column tiles tn >= tn_skip tm of the tn_n, then row tiles
+  int item0, tm_n, tn_n, tn_skip;
 };
 struct TcItem {
   int desc, tm, tn, split;
@@ -69,15 +72,12 @@ struct TcScratch {
   int* eu = nullptr;
   int* eb = nullptr;
   int* ec = nullptr;             // column exponents of the A operand of A T (equilibration)
-  TcDesc* desc = nullptr;
-  TcItem* items = nullptr;
-  char* info = nullptr;          // per-block split descriptors
-  int* list = nullptr;
+  char* info = nullptr;          // per-block lists: two split descriptors and a TcDesc each
   int* err = nullptr;            // set by a bounded wait that gave up
   void* part = nullptr;
   int64_t rows_a = 0, rows_b = 0, rows_u = 0, pitch_a = 0, pitch_b = 0, pitch_u = 0;
   int64_t rows_band = 0, pitch_band = 0, band_lo = 0, band_w = 0, band_half = 0;
-  int64_t max_items = 0, max_blocks = 0, part_elems = 0;
+  int64_t max_blocks = 0, part_elems = 0;
   int max_split = 1;
 };
 

@@ -184,3 +184,27 @@ def test_band_product_tensor_matches_fp64(pk, cplx, n, b, m):
     err = np.max(np.abs(Y - ref) / scale)
     print("band", cplx, n, b, m, err)
     assert err < 1e-13
+
+
+@pytest.mark.parametrize("cplx", [True, False])
+@pytest.mark.parametrize("n,m", [(300, 37), (129, 64)])
+def test_exponents_at_the_ends_of_the_range(pk, cplx, n, m):
+    """Columns of subnormal numbers, of the largest ones, of zeros, and rows whose scaled maximum is
+    subnormal take the FP64 loop for their exponents; the update by a permutation moves the columns, and
+    exactly (47 bits kept below a row's maximum; entries of magnitude 1 to 2 in one column and less than
+    2^-60 of it, or exactly representable, elsewhere)."""
+    g = np.random.default_rng(81)
+    X = g.integers(-8, 9, size=(m, n)).astype(np.float64)
+    if cplx:
+        X = X + 1j * g.integers(-8, 9, size=(m, n))
+    X[1] = X[1] * 2.0 ** -1070
+    X[2] = X[2] * 2.0 ** 1019
+    X[3] = 0.0
+    p = g.permutation(m)
+    T = np.zeros((m, m))
+    T[p, np.arange(m)] = 1.0
+    out = pk.block_gemm(pk.GEMM_UPDATE, _t(pk, X), [m], B=[_t(pk, T.astype(X.dtype))]).cpu().numpy()
+    ref = X[p]
+    big = np.abs(X) >= 2.0 ** -1022
+    # subnormal data counts as zero in the digits
+    assert np.array_equal(out, np.where(big[p], ref, 0))
