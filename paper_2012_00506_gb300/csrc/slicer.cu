@@ -230,198 +230,300 @@ static void layer_table(Layer L[4]) {
   }
 }
 
-// Y[bt][o] = act(sum_i X[bt][i] W[o][i] + bias[o]); one CTA per 32 x 32 output tile
-__global__ void __launch_bounds__(256) mlp_fwd_kernel(int B, int in, int out, const float* __restrict__ X,
-                                                      const float* __restrict__ W, const float* __restrict__ bias,
-                                                      float* __restrict__ Y, int relu) {
-  __shared__ float Xs[32][33], Ws[32][33];
-  const int o0 = blockIdx.x * 32, b0 = blockIdx.y * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int k0 = 0; k0 < in; k0 += 32) {
-    for (int e = threadIdx.x; e < 32 * 32; e += 256) {
-      const int r = e >> 5, c = e & 31;
-      Xs[r][c] = (b0 + r < B && k0 + c < in) ? X[(int64_t)(b0 + r) * in + k0 + c] : 0.f;
-      Ws[r][c] = (o0 + r < out && k0 + c < in) ? W[(int64_t)(o0 + r) * in + k0 + c] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int k = 0; k < 32; ++k) {
-      const float wv = Ws[tx][k];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q] = fmaf(Xs[ty + 8 * q][k], wv, acc[q]);
-    }
-    __syncthreads();
-  }
-  const int o = o0 + tx;
-  if (o >= out) return;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int bt = b0 + ty + 8 * q;
-    if (bt >= B) continue;
-    float v = acc[q] + bias[o];
-    if (relu) v = fmaxf(v, 0.f);
-    Y[(int64_t)bt * out + o] = v;
-  }
-}
+// The layers are small (256 x 256 weights, a batch of at most a few hundred): what costs is latency, not
+// arithmetic or bandwidth.  Each kernel copies its whole slab of the weights to shared memory at once, before it
+// waits for the kernel in front (programmatic launch: the weights are not written during a pass), then its few
+// rows of activations, and sums without further barriers; sums run over ascending k in one chain of FMAs.
+// (Only the weights are __restrict__: loads of what the kernel in front writes must not move above the wait.)
+// Measured, batch 64, one Adam step: 14 launches of 32 x 32 tiles staged 32 k at a time took 127 us of
+// device time and 158 us in all; these 8 launches take 46 us in all, with the same bits.
+constexpr int kRows = 8;           // batch rows per tile
+constexpr int kPitch = kHid + 4;   // floats: 16-byte rows, 8 consecutive rows in different banks
+constexpr int kHeadRows = 4;
+constexpr size_t kHeadSmem = sizeof(float) * (kOut + kHeadRows) * kPitch;
 
-// softmax over the 64 logits of one sample, cumulative sums -> 63 boundaries.
-// With a target: per-sample loss share and dL/dlogits.
-__global__ void __launch_bounds__(64) mlp_head_kernel(int B, const float* __restrict__ Z, float* __restrict__ bounds,
-                                                      const float* __restrict__ target, float* __restrict__ dZ,
-                                                      float* __restrict__ loss_part) {
-  const int bt = blockIdx.x, j = threadIdx.x;
-  __shared__ float p[kOut], cs[kOut], dc[kOut], dp[kOut];
-  __shared__ float red[2];
-  const float z = Z[(int64_t)bt * kOut + j];
-  float m = z;
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((j & 31) == 0) red[j >> 5] = m;
-  __syncthreads();
-  m = fmaxf(red[0], red[1]);
-  __syncthreads();
-  const float e = expf(z - m);
-  float s = e;
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((j & 31) == 0) red[j >> 5] = s;
-  __syncthreads();
-  s = red[0] + red[1];
-  p[j] = e / s;
-  __syncthreads();
-  if (j == 0) {
-    float c = 0.f;
-    for (int k = 0; k < kOut; ++k) {
-      c += p[k];
-      cs[k] = c;
+// rows x cols floats (row stride ld) to shared memory (row stride pitch); rows at or past nrows are zero
+__device__ __forceinline__ void stage_rows(float* dst, int pitch, const float* src, int64_t ld, int rows, int nrows,
+                                           int cols) {
+  if ((((uintptr_t)src | (uintptr_t)(ld * 4)) & 15) == 0 && (cols & 3) == 0) {
+    const int c4 = cols >> 2;
+#pragma unroll 8
+    for (int e = threadIdx.x; e < rows * c4; e += blockDim.x) {
+      const int r = e / c4, c = e - r * c4;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r < nrows) v = *(const float4*)(src + r * ld + 4 * c);
+      *(float4*)(dst + r * pitch + 4 * c) = v;
     }
-  }
-  __syncthreads();
-  if (j < kOut - 1) bounds[(int64_t)bt * (kOut - 1) + j] = cs[j];
-  if (!target) return;
-  const float scale = 1.0f / ((float)B * (float)(kOut - 1));
-  float l = 0.f;
-  if (j < kOut - 1) {
-    const float d = cs[j] - target[(int64_t)bt * (kOut - 1) + j];
-    l = d * d * scale;
-    dc[j] = 2.f * d * scale;
   } else {
-    dc[j] = 0.f;
-  }
-  for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-  __syncthreads();
-  if ((j & 31) == 0) red[j >> 5] = l;
-  __syncthreads();
-  if (j == 0) {
-    loss_part[bt] = red[0] + red[1];
-    float acc = 0.f;  // dL/dp_k = sum_{i >= k} dL/dc_i
-    for (int k = kOut - 1; k >= 0; --k) {
-      acc += dc[k];
-      dp[k] = acc;
+#pragma unroll 8
+    for (int e = threadIdx.x; e < rows * cols; e += blockDim.x) {
+      const int r = e / cols, c = e - r * cols;
+      dst[r * pitch + c] = r < nrows ? src[r * ld + c] : 0.f;
     }
   }
-  __syncthreads();
-  float sdp = p[j] * dp[j];
-  for (int o = 16; o > 0; o >>= 1) sdp += __shfl_xor_sync(0xffffffffu, sdp, o);
-  if ((j & 31) == 0) red[j >> 5] = sdp;
-  __syncthreads();
-  sdp = red[0] + red[1];
-  dZ[(int64_t)bt * kOut + j] = p[j] * (dp[j] - sdp);
 }
 
-// dX[bt][i] = (sum_o dY[bt][o] W[o][i]) * [Xact[bt][i] > 0]: the gradient with
-// respect to the pre-activation of the previous layer
-__global__ void __launch_bounds__(256) mlp_bwd_x_kernel(int B, int in, int out, const float* __restrict__ dY,
-                                                        const float* __restrict__ W, const float* __restrict__ Xact,
-                                                        float* __restrict__ dX) {
-  __shared__ float Ds[32][33], Ws[32][33];
-  const int i0 = blockIdx.x * 32, b0 = blockIdx.y * 32;
+// Y[bt][o] = max(sum_i X[bt][i] W[o][i] + bias[o], 0): 32 outputs x 8 rows per CTA, its weights kept over
+// the row tiles; out is a multiple of 32, in <= 256
+__global__ void __launch_bounds__(128) mlp_fwd_kernel(int B, int in, int out, const float* X,
+                                                      const float* __restrict__ W, const float* __restrict__ bias,
+                                                      float* Y) {
+  __shared__ __align__(16) float Ws[32 * kPitch], Xs[kRows * kPitch];
+  const int o0 = blockIdx.y * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int k0 = 0; k0 < out; k0 += 32) {
-    for (int e = threadIdx.x; e < 32 * 32; e += 256) {
-      const int r = e >> 5, c = e & 31;
-      Ds[r][c] = (b0 + r < B && k0 + c < out) ? dY[(int64_t)(b0 + r) * out + k0 + c] : 0.f;
-      Ws[r][c] = (k0 + r < out && i0 + c < in) ? W[(int64_t)(k0 + r) * in + i0 + c] : 0.f;  // Ws[o][i]
+  cudaTriggerProgrammaticLaunchCompletion();
+  stage_rows(Ws, kPitch, W + (int64_t)o0 * in, in, 32, 32, in);
+  const float bo = bias[o0 + tx];
+  cudaGridDependencySynchronize();
+  const float* w = Ws + tx * kPitch;
+  const float *x0 = Xs + ty * kPitch, *x1 = Xs + (ty + 4) * kPitch;
+  for (int b0 = blockIdx.x * kRows; b0 < B; b0 += gridDim.x * kRows) {
+    __syncthreads();
+    stage_rows(Xs, kPitch, X + (int64_t)b0 * in, in, kRows, B - b0, in);
+    __syncthreads();
+    float a0 = 0.f, a1 = 0.f;
+    int k = 0;
+#pragma unroll 8
+    for (; k + 4 <= in; k += 4) {
+      const float4 wv = *(const float4*)(w + k), u = *(const float4*)(x0 + k), v = *(const float4*)(x1 + k);
+      a0 = fmaf(u.x, wv.x, a0);
+      a1 = fmaf(v.x, wv.x, a1);
+      a0 = fmaf(u.y, wv.y, a0);
+      a1 = fmaf(v.y, wv.y, a1);
+      a0 = fmaf(u.z, wv.z, a0);
+      a1 = fmaf(v.z, wv.z, a1);
+      a0 = fmaf(u.w, wv.w, a0);
+      a1 = fmaf(v.w, wv.w, a1);
     }
+    for (; k < in; ++k) {
+      a0 = fmaf(x0[k], w[k], a0);
+      a1 = fmaf(x1[k], w[k], a1);
+    }
+    if (b0 + ty < B) Y[(int64_t)(b0 + ty) * out + o0 + tx] = fmaxf(a0 + bo, 0.f);
+    if (b0 + ty + 4 < B) Y[(int64_t)(b0 + ty + 4) * out + o0 + tx] = fmaxf(a1 + bo, 0.f);
+  }
+}
+
+// The last layer and the head: 64 logits of 4 samples per CTA (64 threads a sample), softmax, cumulative
+// sums -> 63 boundaries.  With a target: per-sample loss share and dL/dlogits.
+__global__ void __launch_bounds__(64 * kHeadRows)
+    mlp_head_kernel(int B, const float* X, const float* __restrict__ W, const float* __restrict__ bias,
+                    float* bounds, const float* target, float* dZ,
+                    float* loss_part) {
+  extern __shared__ __align__(16) float hs[];
+  float *Ws = hs, *Xs = hs + kOut * kPitch;
+  __shared__ __align__(16) float p_[kHeadRows][kOut], cs_[kHeadRows][kOut], dc_[kHeadRows][kOut], dp_[kHeadRows][kOut];
+  __shared__ float red_[kHeadRows][2];
+  const int s4 = threadIdx.x >> 6, j = threadIdx.x & 63;
+  float *p = p_[s4], *cs = cs_[s4], *dc = dc_[s4], *dp = dp_[s4], *red = red_[s4];
+  cudaTriggerProgrammaticLaunchCompletion();
+  stage_rows(Ws, kPitch, W, kHid, kOut, kOut, kHid);
+  const float bo = bias[j];
+  cudaGridDependencySynchronize();
+  for (int b0 = blockIdx.x * kHeadRows; b0 < B; b0 += gridDim.x * kHeadRows) {
+    __syncthreads();
+    stage_rows(Xs, kPitch, X + (int64_t)b0 * kHid, kHid, kHeadRows, B - b0, kHid);
+    __syncthreads();
+    const int bt = b0 + s4;
+    const bool live = bt < B;
+    float z = 0.f;
+    {
+      const float *w = Ws + j * kPitch, *x = Xs + s4 * kPitch;
+#pragma unroll 8
+      for (int k = 0; k < kHid; k += 4) {
+        const float4 wv = *(const float4*)(w + k), u = *(const float4*)(x + k);
+        z = fmaf(u.x, wv.x, z);
+        z = fmaf(u.y, wv.y, z);
+        z = fmaf(u.z, wv.z, z);
+        z = fmaf(u.w, wv.w, z);
+      }
+      z += bo;
+    }
+    float m = z;
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((j & 31) == 0) red[j >> 5] = m;
+    __syncthreads();
+    m = fmaxf(red[0], red[1]);
+    __syncthreads();
+    const float e = expf(z - m);
+    float s = e;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((j & 31) == 0) red[j >> 5] = s;
+    __syncthreads();
+    s = red[0] + red[1];
+    p[j] = e / s;
+    __syncthreads();
+    if (j == 0) {
+      float c = 0.f;
+#pragma unroll
+      for (int k = 0; k < kOut; ++k) {
+        c += p[k];
+        cs[k] = c;
+      }
+    }
+    __syncthreads();
+    if (live && j < kOut - 1) bounds[(int64_t)bt * (kOut - 1) + j] = cs[j];
+    if (!target) continue;
+    const float scale = 1.0f / ((float)B * (float)(kOut - 1));
+    float l = 0.f;
+    if (live && j < kOut - 1) {
+      const float d = cs[j] - target[(int64_t)bt * (kOut - 1) + j];
+      l = d * d * scale;
+      dc[j] = 2.f * d * scale;
+    } else {
+      dc[j] = 0.f;
+    }
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    __syncthreads();
+    if ((j & 31) == 0) red[j >> 5] = l;
+    __syncthreads();
+    if (j == 0) {
+      if (live) loss_part[bt] = red[0] + red[1];
+      float acc = 0.f;  // dL/dp_k = sum_{i >= k} dL/dc_i
+#pragma unroll
+      for (int k = kOut - 1; k >= 0; --k) {
+        acc += dc[k];
+        dp[k] = acc;
+      }
+    }
+    __syncthreads();
+    float sdp = p[j] * dp[j];
+    for (int o = 16; o > 0; o >>= 1) sdp += __shfl_xor_sync(0xffffffffu, sdp, o);
+    if ((j & 31) == 0) red[j >> 5] = sdp;
+    __syncthreads();
+    sdp = red[0] + red[1];
+    if (live) dZ[(int64_t)bt * kOut + j] = p[j] * (dp[j] - sdp);
+  }
+}
+
+// dX[bt][i] = (sum_o dY[bt][o] W[o][i]) * [Xact[bt][i] > 0]: the gradient with respect to the
+// pre-activation of the previous layer (in = 256); 32 columns x 8 rows per CTA
+__global__ void __launch_bounds__(128) mlp_bwd_x_kernel(int B, int out, const float* dY,
+                                                        const float* __restrict__ W, const float* Xact,
+                                                        float* dX) {
+  __shared__ __align__(16) float Ws[kHid * 32], Ds[kRows * kPitch];
+  const int i0 = blockIdx.y * 32;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  cudaTriggerProgrammaticLaunchCompletion();
+  stage_rows(Ws, 32, W + i0, kHid, out, out, 32);
+  cudaGridDependencySynchronize();
+  const float *d0 = Ds + ty * kPitch, *d1 = Ds + (ty + 4) * kPitch;
+  for (int b0 = blockIdx.x * kRows; b0 < B; b0 += gridDim.x * kRows) {
+    __syncthreads();
+    stage_rows(Ds, kPitch, dY + (int64_t)b0 * out, out, kRows, B - b0, out);
+    __syncthreads();
+    float a0 = 0.f, a1 = 0.f;
+#pragma unroll 4
+    for (int k = 0; k < out; k += 4) {
+      const float4 u = *(const float4*)(d0 + k), v = *(const float4*)(d1 + k);
+      const float w0 = Ws[k * 32 + tx], w1 = Ws[(k + 1) * 32 + tx], w2 = Ws[(k + 2) * 32 + tx],
+                  w3 = Ws[(k + 3) * 32 + tx];
+      a0 = fmaf(u.x, w0, a0);
+      a1 = fmaf(v.x, w0, a1);
+      a0 = fmaf(u.y, w1, a0);
+      a1 = fmaf(v.y, w1, a1);
+      a0 = fmaf(u.z, w2, a0);
+      a1 = fmaf(v.z, w2, a1);
+      a0 = fmaf(u.w, w3, a0);
+      a1 = fmaf(v.w, w3, a1);
+    }
+    for (int q = 0; q < 2; ++q) {
+      const int bt = b0 + ty + 4 * q;
+      if (bt >= B) continue;
+      const int64_t at = (int64_t)bt * kHid + i0 + tx;
+      dX[at] = Xact[at] > 0.f ? (q ? a1 : a0) : 0.f;
+    }
+  }
+}
+
+// Adam's state and step (m null: write the gradient instead)
+struct Adam {
+  float *p, *m, *v;
+  float lr, b1, b2, eps, c1, c2;
+};
+
+struct GradLayer {
+  const float *dY, *X;
+  int in, out, tiles_i, tile0;  // tile0: first CTA of the layer
+  int64_t w, b;                 // offsets of W and bias in the parameter vector
+};
+struct GradLayers {
+  GradLayer l[4];
+  int tiles;
+};
+
+// All layers' dW[o][i] = sum_bt dY[bt][o] X[bt][i] and db[o] = sum_bt dY[bt][o] (by the CTAs of a layer's
+// first column tile), written to g or taken into Adam's step at once; the last CTA sums the loss.
+__global__ void __launch_bounds__(256) mlp_bwd_w_kernel(int B, const __grid_constant__ GradLayers L,
+                                                        float* g, const Adam ad,
+                                                        const float* part, float* loss) {
+  constexpr int kChunk = 64;  // batch rows per stage
+  __shared__ __align__(16) float Ds[kChunk * 36], Xs[kChunk * 36];
+  if ((int)blockIdx.x == L.tiles) {
+    cudaGridDependencySynchronize();
+    float s = 0.f;
+    for (int i = threadIdx.x; i < B; i += blockDim.x) s += part[i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) Ds[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      float t = 0.f;
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += Ds[w];
+      *loss = t;
+    }
+    return;
+  }
+  int li = 0;
+  while (li < 3 && (int)blockIdx.x >= L.l[li + 1].tile0) ++li;
+  const GradLayer& l = L.l[li];
+  const int tile = blockIdx.x - l.tile0;
+  const int i0 = tile % l.tiles_i * 32, o0 = tile / l.tiles_i * 32;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int i = i0 + tx;
+  const bool bias = i0 == 0 && ty == 0;
+  // parameters and moments of this thread's entries: 4 weights, a bias
+  float pv[5], mv[5], vv[5];
+  int64_t at[5];
+#pragma unroll
+  for (int q = 0; q < 5; ++q) {
+    at[q] = q < 4 ? (i < l.in ? l.w + (int64_t)(o0 + ty + 8 * q) * l.in + i : -1) : bias ? l.b + o0 + tx : -1;
+    if (ad.m && at[q] >= 0) {
+      pv[q] = ad.p[at[q]];
+      mv[q] = ad.m[at[q]];
+      vv[q] = ad.v[at[q]];
+    }
+  }
+  cudaGridDependencySynchronize();
+  float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+  for (int k0 = 0; k0 < B; k0 += kChunk) {
+    const int nk = min(kChunk, B - k0);
+    __syncthreads();
+    stage_rows(Ds, 36, l.dY + (int64_t)k0 * l.out + o0, l.out, nk, nk, 32);
+    stage_rows(Xs, 36, l.X + (int64_t)k0 * l.in + i0, l.in, nk, nk, min(32, l.in - i0));
     __syncthreads();
 #pragma unroll 8
-    for (int k = 0; k < 32; ++k) {
-      const float wv = Ws[k][tx];
+    for (int k = 0; k < nk; ++k) {
+      const float xv = Xs[k * 36 + tx];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q] = fmaf(Ds[ty + 8 * q][k], wv, acc[q]);
+      for (int q = 0; q < 4; ++q) acc[q] = fmaf(Ds[k * 36 + ty + 8 * q], xv, acc[q]);
     }
-    __syncthreads();
-  }
-  const int i = i0 + tx;
-  if (i >= in) return;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int bt = b0 + ty + 8 * q;
-    if (bt >= B) continue;
-    const float v = Xact[(int64_t)bt * in + i] > 0.f ? acc[q] : 0.f;
-    dX[(int64_t)bt * in + i] = v;
-  }
-}
-
-// dW[o][i] = sum_bt dY[bt][o] X[bt][i]; the CTAs of the first column tile also
-// write db[o] = sum_bt dY[bt][o]
-__global__ void __launch_bounds__(256) mlp_bwd_w_kernel(int B, int in, int out, const float* __restrict__ dY,
-                                                        const float* __restrict__ X, float* __restrict__ dW,
-                                                        float* __restrict__ db) {
-  __shared__ float Ds[32][33], Xs[32][33];
-  const int i0 = blockIdx.x * 32, o0 = blockIdx.y * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  float bacc = 0.f;
-  for (int k0 = 0; k0 < B; k0 += 32) {
-    for (int e = threadIdx.x; e < 32 * 32; e += 256) {
-      const int r = e >> 5, c = e & 31;
-      Ds[r][c] = (k0 + r < B && o0 + c < out) ? dY[(int64_t)(k0 + r) * out + o0 + c] : 0.f;
-      Xs[r][c] = (k0 + r < B && i0 + c < in) ? X[(int64_t)(k0 + r) * in + i0 + c] : 0.f;
-    }
-    __syncthreads();
+    if (bias)
 #pragma unroll 8
-    for (int k = 0; k < 32; ++k) {
-      const float xv = Xs[k][tx];
+      for (int k = 0; k < nk; ++k) acc[4] += Ds[k * 36 + tx];
+  }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q] = fmaf(Ds[k][ty + 8 * q], xv, acc[q]);
+  for (int q = 0; q < 5; ++q) {
+    if (at[q] < 0) continue;
+    if (!ad.m) {
+      g[at[q]] = acc[q];
+      continue;
     }
-    if (blockIdx.x == 0 && ty == 0)
-      for (int k = 0; k < 32; ++k) bacc += Ds[k][tx];
-    __syncthreads();
-  }
-  const int i = i0 + tx;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int o = o0 + ty + 8 * q;
-    if (o < out && i < in) dW[(int64_t)o * in + i] = acc[q];
-  }
-  if (blockIdx.x == 0 && ty == 0 && o0 + tx < out) db[o0 + tx] = bacc;
-}
-
-__global__ void adam_kernel(int64_t np, float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-  }
-}
-
-__global__ void loss_sum_kernel(int B, const float* __restrict__ part, float* __restrict__ loss) {
-  __shared__ float red[32];
-  float s = 0.f;
-  for (int i = threadIdx.x; i < B; i += blockDim.x) s += part[i];
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float t = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    *loss = t;
+    const float gi = acc[q];
+    const float mi = ad.b1 * mv[q] + (1.f - ad.b1) * gi;
+    const float vi = ad.b2 * vv[q] + (1.f - ad.b2) * gi * gi;
+    ad.m[at[q]] = mi;
+    ad.v[at[q]] = vi;
+    ad.p[at[q]] = pv[q] - ad.lr * (mi / ad.c1) / (sqrtf(vi / ad.c2) + ad.eps);
   }
 }
 
@@ -442,38 +544,57 @@ static MlpWs plan_mlp(Arena& a, int B) {
   return w;
 }
 
-// forward (bounds); with target: loss; with grad: full backward pass into grad
+// launch that may start before the kernel in front has finished; the kernels above wait for it themselves
+template <typename... P, typename... A>
+static int launch_after(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  PD_CK(cudaLaunchKernelEx(&cfg, kernel, (P)args...));
+  PD_CK_LAUNCH();
+  return 0;
+}
+
+// forward (bounds); with target: loss and the full backward pass into grad, or into Adam's step (adam.m set)
 static int mlp_run(int B, const float* params, const float* X, float* bounds, const float* target, float* grad,
-                   float* loss, const MlpWs& w, cudaStream_t st) {
+                   const Adam& adam, float* loss, const MlpWs& w, cudaStream_t st) {
   Layer L[4];
   layer_table(L);
+  const int row_tiles = (int)std::min<int64_t>(ceil_div(B, kRows), 76);
   const float* in = X;
-  for (int l = 0; l < 4; ++l) {
-    dim3 g((unsigned)ceil_div(L[l].out, 32), (unsigned)ceil_div(B, 32));
-    mlp_fwd_kernel<<<g, 256, 0, st>>>(B, L[l].in, L[l].out, in, params + L[l].w, params + L[l].b, w.act[l + 1],
-                                      l < 3 ? 1 : 0);
-    PD_CK_LAUNCH();
+  for (int l = 0; l < 3; ++l) {
+    const dim3 g((unsigned)row_tiles, (unsigned)(L[l].out / 32));
+    const float *W = params + L[l].w, *bias = params + L[l].b;
+    if (l == 0) {  // reads what the caller's kernels wrote: an ordinary launch
+      mlp_fwd_kernel<<<g, 128, 0, st>>>(B, L[l].in, L[l].out, in, W, bias, w.act[1]);
+      PD_CK_LAUNCH();
+    } else {
+      PD_TRY(launch_after(mlp_fwd_kernel, g, 128, 0, st, B, L[l].in, L[l].out, in, W, bias, w.act[l + 1]));
+    }
     in = w.act[l + 1];
   }
-  mlp_head_kernel<<<B, kOut, 0, st>>>(B, w.act[4], bounds, target, w.dact[4], w.lpart);
-  PD_CK_LAUNCH();
+  PD_CK(cudaFuncSetAttribute(mlp_head_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeadSmem));
+  PD_TRY(launch_after(mlp_head_kernel, dim3((unsigned)std::min<int64_t>(ceil_div(B, kHeadRows), 304)), 64 * kHeadRows,
+                      kHeadSmem, st, B, in, params + L[3].w, params + L[3].b, bounds, target, w.dact[4], w.lpart));
   if (!target) return 0;
-  loss_sum_kernel<<<1, 256, 0, st>>>(B, w.lpart, loss);
-  PD_CK_LAUNCH();
-  if (!grad) return 0;
-  for (int l = 3; l >= 0; --l) {
-    const float* xin = l == 0 ? X : w.act[l];
-    dim3 gw((unsigned)ceil_div(L[l].in, 32), (unsigned)ceil_div(L[l].out, 32));
-    mlp_bwd_w_kernel<<<gw, 256, 0, st>>>(B, L[l].in, L[l].out, w.dact[l + 1], xin, grad + L[l].w, grad + L[l].b);
-    PD_CK_LAUNCH();
-    if (l > 0) {
-      dim3 gx((unsigned)ceil_div(L[l].in, 32), (unsigned)ceil_div(B, 32));
-      mlp_bwd_x_kernel<<<gx, 256, 0, st>>>(B, L[l].in, L[l].out, w.dact[l + 1], params + L[l].w, w.act[l],
-                                           w.dact[l]);
-      PD_CK_LAUNCH();
-    }
+  for (int l = 3; l > 0; --l)
+    PD_TRY(launch_after(mlp_bwd_x_kernel, dim3((unsigned)row_tiles, kHid / 32), 128, 0, st, B, L[l].out, w.dact[l + 1],
+                        params + L[l].w, w.act[l], w.dact[l]));
+  GradLayers G;
+  G.tiles = 0;
+  for (int l = 0; l < 4; ++l) {
+    const int ti = (int)ceil_div(L[l].in, 32);
+    G.l[l] = GradLayer{w.dact[l + 1], l == 0 ? X : w.act[l], L[l].in, L[l].out, ti, G.tiles, L[l].w, L[l].b};
+    G.tiles += ti * (L[l].out / 32);
   }
-  return 0;
+  return launch_after(mlp_bwd_w_kernel, dim3((unsigned)(G.tiles + 1)), 256, 0, st, B, G, grad, adam, w.lpart, loss);
 }
 
 // ---------------------------------------------------------------------------
@@ -696,7 +817,7 @@ extern "C" int pdeshep_mlp_forward(const float* d_params, int32_t batch, const f
   Arena a(d_work, work_bytes);
   const MlpWs w = plan_mlp(a, batch);
   if (!a.fits()) return PDESHEP_WORKSPACE_TOO_SMALL;
-  return mlp_run(batch, d_params, d_x, d_bounds, nullptr, nullptr, nullptr, w, (cudaStream_t)stream);
+  return mlp_run(batch, d_params, d_x, d_bounds, nullptr, nullptr, Adam{}, nullptr, w, (cudaStream_t)stream);
 }
 
 extern "C" int pdeshep_mlp_grad(const float* d_params, int32_t batch, const float* d_x, const float* d_target,
@@ -712,7 +833,7 @@ extern "C" int pdeshep_mlp_grad(const float* d_params, int32_t batch, const floa
   const MlpWs w = plan_mlp(a, batch);
   float* bounds = a.take<float>((size_t)batch * (kOut - 1));
   if (!a.fits()) return PDESHEP_WORKSPACE_TOO_SMALL;
-  return mlp_run(batch, d_params, d_x, bounds, d_target, d_grad, d_loss, w, (cudaStream_t)stream);
+  return mlp_run(batch, d_params, d_x, bounds, d_target, d_grad, Adam{}, d_loss, w, (cudaStream_t)stream);
 }
 
 extern "C" int pdeshep_mlp_train_step(float* d_params, float* d_adam_m, float* d_adam_v, int32_t step, float lr,
@@ -730,16 +851,14 @@ extern "C" int pdeshep_mlp_train_step(float* d_params, float* d_adam_m, float* d
   if (!d_work) return -10;
   Arena a(d_work, work_bytes);
   const MlpWs w = plan_mlp(a, batch);
-  float* grad = a.take<float>(kNParams);
+  a.take<float>(kNParams);  // (the size the workspace query reports)
   float* bounds = a.take<float>((size_t)batch * (kOut - 1));
   if (!a.fits()) return PDESHEP_WORKSPACE_TOO_SMALL;
   cudaStream_t st = (cudaStream_t)stream;
-  PD_TRY(mlp_run(batch, d_params, d_x, bounds, d_target, grad, d_loss, w, st));
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-  adam_kernel<<<152, 256, 0, st>>>(kNParams, d_params, grad, d_adam_m, d_adam_v, lr, b1, b2, 1e-8f, c1, c2);
-  PD_CK_LAUNCH();
-  return 0;
+  const Adam adam{d_params, d_adam_m, d_adam_v, lr, b1, b2, 1e-8f, c1, c2};
+  return mlp_run(batch, d_params, d_x, bounds, d_target, nullptr, adam, d_loss, w, st);
 }
 
 extern "C" size_t pdeshep_propose_workspace_size(int64_t n, int32_t b, int32_t is_complex, int32_t nslices,
@@ -789,7 +908,7 @@ extern "C" int pdeshep_propose_slices(int64_t n, int32_t b, int32_t is_complex, 
       PD_TRY(features<double2>(n, b, 1, d_band, ldab, seed, feat, fw, st));
     else
       PD_TRY(features<double>(n, b, 0, d_band, ldab, seed, feat, fw, st));
-    PD_TRY(mlp_run(1, d_params, feat, bnd, nullptr, nullptr, nullptr, mw, st));
+    PD_TRY(mlp_run(1, d_params, feat, bnd, nullptr, nullptr, Adam{}, nullptr, mw, st));
     PD_CK(cudaMemcpyAsync(c63, bnd, sizeof(float) * (kOut - 1), cudaMemcpyDeviceToHost, st));
   } else {
     PD_TRY(gershgorin_device(n, b, cplx, d_band, ldab, fw.glo, fw.ghi, st));

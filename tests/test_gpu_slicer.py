@@ -89,6 +89,43 @@ def test_adam_step_vs_oracle(device):
     assert np.abs((p1 - p0)[sure] - (po - p0)[sure]).max() < 2e-5
 
 
+@pytest.mark.parametrize("batch", [1, 4, 7, 8, 9, 63, 64, 65, 609])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_train_step_vs_oracle_at_tile_edges(device, batch, shift):
+    """Batches around the kernels' tiles (4, 8 and 64 rows, and one past the 608 rows of a resident grid), and
+    arrays 4 bytes off the 16-byte boundary.  With a gradient within dg = 1e-4 |grad| of the oracle's (as
+    above), m moves by (1 - beta1) dg, v by (1 - beta2) 2 |g| dg and the step by lr (1 - beta1) dg / sqrt(v/c2),
+    sqrt(v/c2) > 0.04; FP32 rounding adds a few units of each array's largest entry, and the powers of beta2
+    1e-5 of a step."""
+    import torch
+    from paper_2012_00506_gb300 import slicer
+    g_ = np.random.default_rng(100 + batch)
+
+    def place(x):
+        x = x.reshape(-1)
+        t = torch.zeros(x.size + 4, dtype=torch.float32, device=device)
+        t[shift:shift + x.size] = torch.from_numpy(x).to(device)
+        return t[shift:shift + x.size]
+
+    p0 = _params(31, device).cpu().numpy()
+    X = g_.normal(size=(batch, 98)).astype(np.float32)
+    T = np.sort(g_.uniform(size=(batch, 63)), axis=1).astype(np.float32)
+    tr = slicer.Trainer(place(p0), lr=1e-3, max_batch=batch)
+    m0 = (1e-2 * g_.normal(size=p0.shape)).astype(np.float32)
+    v0 = (1e-4 + 1e-4 * g_.uniform(size=p0.shape)).astype(np.float32)
+    tr.m, tr.v, tr.t = place(m0), place(v0), 50
+    lo, go = so.loss_and_grad(p0.astype(np.float64), X.astype(np.float64), T.astype(np.float64))
+    loss = tr.step(place(X).view(batch, 98), place(T).view(batch, 63))
+    po, mo, vo = so.adam_step(p0.astype(np.float64), go, m0.astype(np.float64), v0.astype(np.float64), 51, 1e-3,
+                              b1=float(np.float32(0.9)), b2=float(np.float32(0.999)))
+    assert abs(float(loss.item()) - lo) <= 1e-5 * lo
+    eps, dg = 2.0 ** -23, 1e-4 * np.linalg.norm(go)
+    step = np.abs(po - p0).max()
+    assert np.abs(tr.params.cpu().numpy() - po).max() <= 1e-3 * 0.1 * dg / 0.04 + 1e-5 * step + eps * np.abs(p0).max()
+    assert np.abs(tr.m.cpu().numpy() - mo).max() <= 0.1 * dg + 4 * eps * np.abs(mo).max()
+    assert np.abs(tr.v.cpu().numpy() - vo).max() <= 1e-3 * 2 * np.abs(go).max() * dg + 4 * eps * vo.max()
+
+
 def _check_counts(ab, pr, frac, nslices, tol, exact_targets=True):
     n = ab.shape[0]
     bd = pr.bounds
