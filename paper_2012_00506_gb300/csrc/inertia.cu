@@ -113,13 +113,68 @@ __device__ __forceinline__ void load_row(typename InertiaElem<CPLX>::T* W, int b
   }
 }
 
+// a / d rounded to nearest, in integers: the FP64 division is a chain of FP64 instructions of 64 clocks each
+// (about 600 clocks for a warp, and its quadrant's pipe is taken meanwhile), the division of two 53-bit
+// integers about 200 clocks of the integer pipes, and the reciprocal serves all entries of a column.
+// The reciprocal of the divisor's significand comes from one Newton step on a 23-bit estimate (relative error e:
+// e <= 2^-23 for the estimate plus 2^-24 for its argument, e^2 < 2^-44.8 after the step); the quotient to 54
+// bits follows from it and one correction by the remainder, which is exact modulo 2^64 and below 2^62.3; a last
+// comparison makes it the floor.  A quotient of two 53-bit numbers is never half-way between two of them, so its
+// 54th bit rounds it.  Zero, subnormal, infinite and NaN operands and results outside the normal range go
+// to the FP64 division (zero numerators, common in a band, give their zero at once).
+struct Divisor {
+  double d;
+  unsigned long long md, r1;  // significand (53 bits); 2^62 / (md / 2^53)
+  unsigned r0;                // 2^30 / (md / 2^53)
+};
+__device__ __forceinline__ Divisor divisor(double d) {
+  Divisor v;
+  v.d = d;
+  v.md = ((unsigned long long)__double_as_longlong(d) & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+  const unsigned dh = (unsigned)(v.md >> 21), dl = (unsigned)(v.md << 11);
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint2float_rn(dh)));
+  v.r0 = min(__float2uint_rz(r * 4611686018427387904.0f), 0x7FFFFFFFu);
+  // 1 - x r0 in units of 2^-52
+  const unsigned long long p = (unsigned long long)dh * v.r0 + (((unsigned long long)dl * v.r0) >> 32);
+  const int e = (int)((long long)((1ull << 62) - p) >> 10);
+  v.r1 = ((unsigned long long)v.r0 << 32) + (unsigned long long)(((long long)e * (int)v.r0) >> 20);
+  return v;
+}
+__device__ __noinline__ double quotient_special(double a, double d) { return __ddiv_rn(a, d); }
+__device__ __forceinline__ double quotient(double a, const Divisor& v) {
+  const unsigned long long ab = (unsigned long long)__double_as_longlong(a),
+                           db = (unsigned long long)__double_as_longlong(v.d);
+  const int ea = (int)(ab >> 52) & 0x7FF, ed = (int)(db >> 52) & 0x7FF;
+  const unsigned long long ma = (ab & 0xFFFFFFFFFFFFFull) | (1ull << 52), sign = (ab ^ db) & (1ull << 63);
+  const int less = ma < v.md;
+  const int e = ea - ed + 1023 - less;
+  const unsigned long long n = ma << less;  // n / md in [1, 2)
+  unsigned long long q = __umul64hi(n << 10, v.r1) >> 8;
+  long long rem = (long long)((n << 53) - q * v.md);
+  const int c = (int)(((long long)(int)(rem >> 32) * (int)v.r0) >> 51);
+  q += (long long)c;
+  rem -= (long long)((unsigned long long)(long long)c * v.md);
+  if (rem < 0)
+    --q;
+  else if ((unsigned long long)rem >= v.md)
+    ++q;
+  double x = __longlong_as_double((long long)(sign | (((unsigned long long)(e - 1) << 52) + ((q + 1) >> 1))));
+  const bool dnormal = (unsigned)(ed - 1) < 2046u;
+  if (dnormal && (ab << 1) == 0)
+    x = __longlong_as_double((long long)sign);
+  else if (!(dnormal && (unsigned)(ea - 1) < 2046u && e >= 1 && e <= 2046))
+    x = quotient_special(a, v.d);
+  return x;
+}
+
 // One CTA per shift, one column per step.  Shared memory: pair table (s,u)
 // packed as int32, the multipliers L[0..b], the ring heads h[0..b] and (if
 // `gwin` is null) the window rings W[(b+1)(b+2)/2].  It serves calls with enough
 // shifts to fill the GPU: its half-square window lets four CTAs of b = 64 complex
 // share an SM and hide each other's barriers, and it spends fewer FP64
-// instructions per column than the panel kernel below (504 shifts, n = 4096,
-// b = 64 complex: 23.5 us per column against 28.1).  Bands that no cluster's
+// instructions per column than the panel kernel below (504 shifts, n = 2048,
+// b = 64 complex: 22.6 us per column against 26.6).  Bands that no cluster's
 // shared memory holds also come here (window in the workspace).
 template <bool CPLX>
 __global__ void __launch_bounds__(256) inertia_kernel(int64_t n, int b, const double* __restrict__ band,
@@ -190,12 +245,15 @@ __global__ void __launch_bounds__(256) inertia_kernel(int64_t n, int b, const do
       if (dk < 0.0) ++neg;
       if (piv_out) piv_out[(int64_t)sid * n + k] = dk;
     }
-    for (int d = 1 + threadIdx.x; d <= kmax; d += blockDim.x) {
-      T a = W[ring_base(d, b) + h[d]];
-      if constexpr (CPLX)
-        L[d] = make_double2(__ddiv_rn(a.x, dk), __ddiv_rn(a.y, dk));
-      else
-        L[d] = __ddiv_rn(a, dk);
+    if (threadIdx.x < kmax) {
+      const Divisor by = divisor(dk);
+      for (int d = 1 + threadIdx.x; d <= kmax; d += blockDim.x) {
+        T a = W[ring_base(d, b) + h[d]];
+        if constexpr (CPLX)
+          L[d] = make_double2(quotient(a.x, by), quotient(a.y, by));
+        else
+          L[d] = quotient(a, by);
+      }
     }
     __syncthreads();
     for (int p = threadIdx.x; p < npairs; p += blockDim.x) {
@@ -274,11 +332,12 @@ __device__ __forceinline__ double pivot(double dk, double pivmin, int64_t& neg) 
 // Each entry sees the same rounded operations in the same (ascending column)
 // order as with one column at a time, so counts and pivots keep their bits.
 // Measured against one CTA per shift and one column per step (us per column, all
-// shifts of the call): b = 64 complex, 1 shift 1.5 against 6.7, 9 shifts 2.0
-// against 6.7, 63 shifts 4.5 against 6.8; b = 128 complex, 17 shifts 5.4 against
-// 22.6; b = 32 real, 64 shifts 1.2 against 1.55.  What remains at few shifts is
-// the chain of a column: a division and four dependent operations, about 1.2k of
-// 3k clocks, then the share of the updates (1k) and two cluster barriers per 8.
+// shifts of the call): b = 64 complex, 1 shift 1.4 against 6.6, 9 shifts 1.7
+// against 6.6, 63 shifts 4.3 against 6.6; b = 128 complex, 17 shifts 5.0 against
+// 22.2; b = 32 real, 64 shifts 0.93 against 1.48.  (With the FP64 division, 9 shifts
+// took 2.0 and 64 real ones 1.25.)  What remains at few shifts (b = 64 complex, 8 CTAs
+// a shift) is the chain of a column, a division and four dependent operations, 1.3k of
+// 3.6k clocks, the share of the updates (1.6k) and two cluster barriers per 8.
 // ---------------------------------------------------------------------------
 constexpr int kPan = 8;
 constexpr int kPanThreads = 256;
@@ -314,15 +373,6 @@ __device__ __forceinline__ double sub_prod(double v, double2 l, double2 a, int p
   return __dsub_rn(v, __dadd_rn(__dmul_rn(l1, a.x), __dmul_rn(l2, a.y)));
 }
 
-// a / d rounded to nearest; zeros (the division's slow path) are handled on the bits
-__device__ __forceinline__ double quotient(double a, double d) {
-  const long long ab = __double_as_longlong(a), db = __double_as_longlong(d);
-  const bool zero = (ab << 1) == 0;
-  const double q = __ddiv_rn(zero ? 1.0 : a, d);
-  const bool nan = (unsigned long long)(db << 1) > 0xffe0000000000000ull;
-  return zero && !nan ? __longlong_as_double((ab ^ db) & (long long)0x8000000000000000ull) : q;
-}
-
 template <bool CPLX, int NC>
 __global__ void __launch_bounds__(kPanThreads)
     inertia_panel_kernel(int64_t n, int b, const double* __restrict__ band, int64_t ldab,
@@ -356,31 +406,33 @@ __global__ void __launch_bounds__(kPanThreads)
     return i + ((rank - (int)i) & (G - 1));
   };
   auto slot_of = [&](int64_t i) -> int { return (int)((unsigned)(i >> lg) % (unsigned)nslot); };
-  // own rows r0 <= r < r0 + cnt requested (8-byte copies: the band is only known to be 8-byte aligned)
+  // own rows r0 <= r < r0 + cnt requested (8-byte copies: the band is only known to be 8-byte aligned), row
+  // number x by warp 1 + x mod 7: in the loop below warp 0 has the panel's first division meanwhile
   auto request_rows = [&](int64_t r0, int cnt) {
-    const int64_t r1 = r0 + cnt < n ? r0 + cnt : n;
-    int64_t r = first_own(r0);
-    if (r >= r1) return;
-    int q = slot_of(r);
-    for (int x = 0; r < r1; r += G, ++x) {  // row number x: its diagonal entry is copied by thread x mod 256
-      double* s = W + (size_t)q * rl;
-      for (int d = (tid - x) & (kPanThreads - 1); d <= b; d += kPanThreads) {
-        const int64_t j = r - d;
-        if (j < 0) break;
-        const double* p = band + NP * (d + j * ldab);
+    const int64_t r1 = r0 + cnt < n ? r0 + cnt : n, r = first_own(r0);
+    if (warp == 0 || r >= r1) return;
+    const int q0 = slot_of(r);
+    for (int x = warp - 1; r + (int64_t)x * G < r1; x += kPan - 1) {
+      const int64_t i = r + (int64_t)x * G;
+      const int q = q0 + x;  // (at most nslot rows are requested at once)
+      double* s = W + (size_t)(q >= nslot ? q - nslot : q) * rl;
+      const int last = i < b ? (int)i : b;
+      const double* p = band + NP * (lane + (i - lane) * ldab);
+      for (int d = lane; d <= last; d += 32, p += NP * 32 * (1 - ldab)) {
         cp_async8(s + NP * d, p);
         if (CPLX) cp_async8(s + NP * d + 1, p + 1);
       }
-      q = q + 1 == nslot ? 0 : q + 1;
     }
   };
   // ... and finished: the thread that copied a diagonal entry shifts it (own copies are visible to it)
   auto finish_rows = [&](int64_t r0, int cnt) {
     asm volatile("cp.async.wait_all;\n" ::: "memory");
-    const int64_t r1 = r0 + cnt < n ? r0 + cnt : n;
-    const int64_t r = first_own(r0);
-    for (int x = tid; r + (int64_t)x * G < r1; x += kPanThreads) {
-      double* s = W + (size_t)slot_of(r + (int64_t)x * G) * rl;
+    const int64_t r1 = r0 + cnt < n ? r0 + cnt : n, r = first_own(r0);
+    if (warp == 0 || lane > 0 || r >= r1) return;
+    const int q0 = slot_of(r);
+    for (int x = warp - 1; r + (int64_t)x * G < r1; x += kPan - 1) {
+      const int q = q0 + x;
+      double* s = W + (size_t)(q >= nslot ? q - nslot : q) * rl;
       s[0] = __dsub_rn(s[0], sigma);
       if (CPLX) s[1] = 0.0;
     }
@@ -393,16 +445,16 @@ __global__ void __launch_bounds__(kPanThreads)
   };
   // rows k .. k+kPan-1, columns k .. of them, to every CTA's triangle; q: the slot of the first own one
   auto send_triangle = [&](int64_t k, int q) {
-    for (int i = (rank - (int)k) & (G - 1); i < kPan && k + i < n; i += G) {
-      const double* s = W + (size_t)q * rl;
-      for (int e = tid; e < (kPan * NP << lg); e += kPanThreads) {
-        const int part = e % NP, c = (e / NP) % kPan, g = e / (NP * kPan);
-        if (c > i) continue;
-        const double v = i - c <= b ? s[NP * (i - c) + part] : 0.0;
-        double* t = G > 1 ? cl.map_shared_rank(Tri, g) : Tri;
-        t[(i * kPan + c) * NP + part] = v;
-      }
-      q = q + 1 == nslot ? 0 : q + 1;
+    const int i0 = (rank - (int)k) & (G - 1);
+    const int nown = i0 < kPan ? ((kPan - 1 - i0) >> lg) + 1 : 0;
+    for (int e = tid; e < nown * (kPan * NP << lg); e += kPanThreads) {
+      const int part = e % NP, c = (e / NP) % kPan, g = (e / (NP * kPan)) & (G - 1), x = (e / (NP * kPan)) >> lg;
+      const int i = i0 + (x << lg);
+      if (c > i || k + i >= n) continue;
+      const double* s = W + (size_t)(q + x >= nslot ? q + x - nslot : q + x) * rl;
+      const double v = i - c <= b ? s[NP * (i - c) + part] : 0.0;
+      double* t = G > 1 ? cl.map_shared_rank(Tri, g) : Tri;
+      t[(i * kPan + c) * NP + part] = v;
     }
   };
   request_rows(0, b + kPan);
@@ -424,7 +476,7 @@ __global__ void __launch_bounds__(kPanThreads)
     };
     const int T0 = off0 < nrows ? ((nrows - 1 - off0) >> lg) + 1 : 0;  // own rows among them: i0 + t G
     const int64_t new0 = k + kPan + b;
-    request_rows(new0, kPan);
+    if (NC > 1) request_rows(new0, kPan);
     // ---- the panel.  Its entries live in registers: chunk u of column j (32 lanes of rows: the
     // triangle's, then the own ones) belongs to warp (j + u) mod 8, so the divisions of a column and
     // the updates of the others spread over the SM's four FP64 pipes.
@@ -451,15 +503,17 @@ __global__ void __launch_bounds__(kPanThreads)
     for (int c = 0; c < pk; ++c) {
       // With one chunk per column the warp of column c has the pivot among its lanes and goes on to the
       // division at once; the other warps' updates by column c - 1 run beside it.
+      if (NC == 1 && c == 0) request_rows(new0, kPan);
       if (NC > 1 || warp == c) {
         const double dk = pivot(NC > 1 ? sh_d : __shfl_sync(0xffffffffu, v[0], c * NP), pivmin, neg);
+        const Divisor by = divisor(dk);
         const bool first = NC > 1 ? tid == 0 : lane == 0;
         if (piv_out && first && rank == 0) piv_out[(int64_t)sid * n + k + c] = dk;
 #pragma unroll
         for (int u = 0; u < NC; ++u)
           if (((warp - u) & (kPan - 1)) == c && u < chunks) {
             const bool on = rho[u] > c && rho[u] - c <= b;
-            const double l = quotient(on ? v[u] : 1.0, dk);
+            const double l = quotient(on ? v[u] : 1.0, by);
             if (on) {
               const int e = (c * lda + (32 * u + lane) / NP) * NP + part;
               ((double*)A)[e] = v[u];
@@ -662,7 +716,10 @@ static int panel_clusters(int b, int G) {
 // the panel's chain (a division and an update, in one warp per column or through two barriers), the
 // rest of a round (barriers, row entry, triangle), the CTA's share of the updates at 76 clocks per
 // warp instruction and FP64 pipe; CTAs that share an SM share its pipes.  `sms` is what clusters of G
-// reach at one CTA per SM.  At b = 64 complex the measured times cross at about 110 shifts.
+// reach at one CTA per SM.  Fitted to 254 calls (b = 8 .. 140, real and complex, 1 .. 504 shifts, every G): the
+// choice costs 1.1% over the best G on average, 30% at most, and is nowhere slower than one CTA per
+// shift.  At b = 64 complex the measured times cross between 63 shifts (4.3 us per column in clusters
+// of 4 or 2 against 6.6) and 110 (7.3 against 6.65).
 // beside: the counts run on a side stream next to factorizations that need whole SMs, and nobody waits
 // for them until two filter passes are done, so they keep to about 20 CTAs (9 shifts of n = 8192, b = 64
 // complex on 112 SMs stretched a factorization of 64 systems from 6.4 to 18 ms).
@@ -675,11 +732,11 @@ static int panel_cluster_size(int b, int nsigma, bool single_ok, bool beside) {
   int best = -1;
   double best_t = 0.0;
   if (single_ok) {
-    const double div = np * 9.0 * 19.0 * ceil_div(b, 32);
+    const double div = np * 221.0 * ceil_div(b, 32);
     const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(8, 227 * 1024 / (single_smem(b, CPLX) + 1024)));
     const int waves = (int)ceil_div(nsigma, 152 * per_sm);
     const double co = (double)ceil_div(std::min(nsigma, 152 * per_sm), 152);
-    best_t = waves * std::max(work + div + 2150.0 + 64.0 * ops, co * 1.1 * (work + div));
+    best_t = 0.92 * waves * std::max(work + div + 2280.0 + 11.5 * ops, co * (1.09 * work + div + 395.0));
     best = 0;
   }
   for (int G = 1, q = 0; G <= 16; G *= 2, ++q) {
@@ -689,9 +746,9 @@ static int panel_cluster_size(int b, int nsigma, bool single_ok, bool beside) {
     const int chunks = panel_shape(b, CPLX, G).chunks;
     const int waves = (int)ceil_div(nsigma, nc);
     const double co = (double)ceil_div((int64_t)std::min(nsigma, nc) * G, sms[q]);
-    const double upd = 1.2 * work / G, pan = chunks * (9.0 + 3.5 * ops) * 19.0 + 150.0;
-    const double chain = (chunks == 1 ? 1000.0 + 115.0 * ops : 1300.0 + 175.0 * ops) + 750.0;
-    const double t = waves * std::max((co > 1 ? 1.25 : 1.0) * (chain + upd), co * (upd + pan));
+    const double upd = 1.01 * work / G + 38.0, pan = chunks * (6.85 + 2.19 * ops) * 19.0 + 122.0;
+    const double chain = (chunks == 1 ? 525.0 + 82.5 * ops : 1660.0 + 227.0 * ops) + (G > 1 ? 547.0 : 375.0);
+    const double t = waves * std::max((co > 1 ? 1.35 : 1.0) * (chain + upd), co * (upd + pan));
     if (best < 0 || t < best_t) {
       best = G;
       best_t = t;

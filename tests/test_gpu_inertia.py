@@ -121,3 +121,40 @@ def test_panel_zero_pivots_and_nan(device):
         with pytest.raises(pk.PdeshepError) as e:
             pk.inertia(to_dev(ab, device), sig)
         assert e.value.status == 4
+
+
+@pytest.mark.parametrize("nsig", [1, 400])
+@pytest.mark.parametrize("kind", ["unit", "wide", "near", "edge"])
+def test_quotients_are_rounded_to_nearest(device, nsig, kind):
+    """The kernels divide in integers: 2 x 2 blocks [[d, a], [a, 0]] on the diagonal give the pivots d and
+    -fl(fl(a/d) a), whose bits show the quotient's.  Significands at random, next to each other and at
+    the ends of their range (a quotient next to 1, to 2 and to half-way points), exponents whose quotient is
+    subnormal, zero or infinite, one call per kernel (1 shift: cluster, 400: one CTA per shift)."""
+    import paper_2012_00506_gb300 as pk
+    m = 3000
+    g = np.random.default_rng(len(kind) + nsig)
+    sig = lambda: (1.0 + g.integers(0, 1 << 52, m).astype(np.float64) * 2.0 ** -52) * g.choice([-1.0, 1.0], m)
+    d, a = sig(), sig()
+    if kind == "wide":
+        d, a = np.ldexp(d, g.integers(-480, 480, m)), np.ldexp(a, g.integers(-480, 480, m))
+    elif kind == "near":
+        a = np.nextafter(d, d * g.choice([1.0, 2.0, 0.5], m)) * 2.0 ** g.integers(-3, 4, m).astype(np.float64)
+    elif kind == "edge":
+        u = g.integers(0, 4, m) * 2.0 ** -52
+        d = np.where(g.random(m) < 0.5, 1.0 + u, 2.0 - 2.0 ** -52 - u)
+        v = g.integers(0, 4, m) * 2.0 ** -52
+        a = np.where(g.random(m) < 0.5, 1.0 + v, 2.0 - 2.0 ** -52 - v)
+        e = g.choice([0, 0, 500, -520, -1040], m)
+        a, d = np.ldexp(a, e), np.ldexp(d, np.where(e == 0, g.choice([0, -1074 + 52, 700], m), 500))
+    a[::97] = 0.0
+    ab = np.zeros((2 * m, 2))
+    ab[0::2, 0] = d
+    ab[0::2, 1] = a
+    neg, piv = pk.inertia(to_dev(ab, device), np.zeros(nsig), pivots=True)
+    piv = piv.cpu().numpy()
+    with np.errstate(all="ignore"):
+        want = 0.0 - (a / d) * a
+    want = np.where(want == 0.0, -oracle.pivmin(ab), want)
+    for i in (0, nsig - 1):
+        assert np.array_equal(piv[i][0::2], d)
+        assert np.array_equal(piv[i][1::2], want, equal_nan=True)
