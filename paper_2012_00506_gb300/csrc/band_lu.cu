@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "band_lu.cuh"
+#include "quotient.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -109,12 +110,10 @@ __global__ void __launch_bounds__(kThreads) init_factor_kernel(FactorGeom g, int
 //    right of it (look-ahead of one); one cluster barrier per block column.  In
 //    FP64, where the updates of a block column take longer than a barrier, its
 //    columns are spread over the cluster as well (`spread`, a second barrier);
-//  * the panel lives in registers, and a column takes one barrier: each warp's
-//    candidate pivot (integer warp reductions on the bits of |re| + |im|) writes its
-//    row and its reciprocal beside its value, so after the barrier every thread has
-//    all it needs.  Rows do not move: each carries its logical index.  complex64: a
-//    thread per row (panel_lu_rows); complex128, where the FP64 pipes of all four
-//    quadrants are needed, a row in four threads (panel_lu_parts);
+//  * rows of the panel do not move: each carries its logical index.  complex64: a thread per row, the row in
+//    registers, every warp searching the column's entries itself (panel_lu_rows); complex128, where the
+//    FP64 pipes of all four quadrants are needed, a row in four threads and a warp that searches
+//    ahead (panel_lu_parts);
 //  * a warp updates NC columns on its own (gathered through the permutation,
 //    rows in registers), without barriers;
 //  * the inverses of the diagonal blocks that only the solves need are left to
@@ -124,7 +123,7 @@ __global__ void __launch_bounds__(kThreads) init_factor_kernel(FactorGeom g, int
 // substitution instead of the product with the inverse).
 // Measured, us per block column against one CTA with a panel in shared memory: complex64 b = 64, 8
 // systems 24.5 against 88, 64 systems 25 against 89, 256 systems 54 (two waves of 89 before); b = 128, 16
-// systems 30 against 151; complex128 b = 32, 8 systems 145 against 454, b = 128, 2 systems 282 against
+// systems 30 against 151; complex128 b = 32, 8 systems 81 against 454, b = 128, 2 systems 182 against
 // 1558.  What remains (b = 64) is the panel: 32 columns of about 1200 clocks, each a search (300), a
 // reciprocal (two dependent divisions, 170), two barriers and the row's updates (440).
 // ---------------------------------------------------------------------------
@@ -141,8 +140,9 @@ __device__ __forceinline__ C cmul_rn(C a, C b) {
 __device__ __forceinline__ unsigned long long pivot_key(float v) {
   return v == v ? (unsigned long long)__float_as_uint(v) + 1 : 0ull;
 }
-__device__ __forceinline__ unsigned long long pivot_key(double v) {
-  return v == v ? (unsigned long long)__double_as_longlong(v) + 1 : 0ull;
+__device__ __forceinline__ unsigned long long pivot_key(double v) {  // (an FP64 comparison takes 64 clocks)
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+  return (u << 1) <= 0xFFE0000000000000ull ? u + 1 : 0ull;
 }
 template <typename R>
 __device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k) {
@@ -158,17 +158,14 @@ __device__ __forceinline__ double2 shfl_c(double2 v, int src) {
   return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
 
-// One warp's candidate for the pivot of a column: its row (columns from the current one on), the
-// reciprocal of its entry, its key and logical row.
-template <typename C>
-struct alignas(16) PivotSlot {
-  C row[kTile];
-  C inv;
-  unsigned long long key;
-  int log, pad;
-};
-
 constexpr int kRowsMax = 256;  // panel rows that panel_lu_rows takes
+
+// One column's pivot, from the warp that searches to those that eliminate.
+template <typename C>
+struct Pivot {
+  C inv;
+  int row, log, ok;  // its row and logical row; whether there is one
+};
 
 // shared memory of one CTA
 template <typename C>
@@ -178,7 +175,9 @@ struct FactorSmem {
   C* Li;    // [T][T+1] rows of the inverse of the unit lower top block (complex64)
   C* top;   // [warps][2][NC][T] top rows of a warp's columns
   int* perm;            // [Pmax]
-  PivotSlot<C>* slot;   // panel_lu_parts: [2][warps]
+  unsigned long long* keys;  // panel_lu_parts: [2][Pmax] keys of the rows' entries of the current column
+  int* logs;            // ... [2][Pmax] and their logical rows
+  Pivot<C>* pivot;      // ... [2]
   C* U;                 // panel_lu_rows: [T][T+2] pivot rows, each from its column on
   C* col;               // ... [2][kRowsMax] the rows' entries of the current column
   unsigned* key;        // ... [2][kRowsMax] and their keys
@@ -191,7 +190,7 @@ __host__ __device__ inline size_t factor_cluster_smem(int Pmax, int nw, int nc) 
   const size_t base = sizeof(C) * ((size_t)kTile * (Pmax + 1) + (size_t)kTile * (kTile + 1) + (size_t)nw * 2 * nc * kTile) +
                       sizeof(int) * Pmax + 64;
   return base + (ROWS ? sizeof(C) * (kTile * (kTile + 2) + 2 * kRowsMax) + sizeof(int) * (3 * kRowsMax + kTile)
-                      : sizeof(PivotSlot<C>) * 2 * nw);
+                      : (sizeof(unsigned long long) + sizeof(int)) * 2 * Pmax + 2 * sizeof(Pivot<C>));
 }
 
 // complex64: LU with partial pivoting of the panel of block column K (rows K .. K+nbb), thread r holding
@@ -380,90 +379,154 @@ __device__ void store_panel_rows(const FactorGeom& g, const FactorPtr<float2>& f
   for (int e = threadIdx.x; e < Pmax; e += blockDim.x) pg[e] = (int16_t)(e < P ? sm.perm[e] : e);
 }
 
-// The same with a row in PARTS threads (columns i PARTS + part): complex128, and complex64 panels of
-// more than kRowsMax rows.  Results in sm.Pan (logical row order) / sm.perm and in global memory.
+// Reciprocal of a pivot by one warp, its parts' divisions in two lanes at once (lane 0: re, lane 1: im).
+// complex64 (Smith's form, whose bits the factors keep): two divisions in a row.
+__device__ __forceinline__ float pivot_reciprocal(float2 a, int lane) {
+  const bool big = fabsf(a.x) >= fabsf(a.y);
+  const float lo = big ? a.y : a.x, hi = big ? a.x : a.y;
+  const float r0 = lo / hi;
+  return (lane == 0 ? (big ? 1.0f : r0) : (big ? -r0 : -1.0f)) / fmaf(lo, r0, hi);
+}
+// complex128: conj(a) / |a|^2 of a scaled to |a| in [1, 2 sqrt 2) by an exact power of two, one division; the error
+// is no larger than Smith's (three roundings of the larger part either way).
+__device__ __forceinline__ double pivot_reciprocal(double2 a, int lane) {
+  const int ex = (__double2hiint(a.x) >> 20) & 0x7FF, ey = (__double2hiint(a.y) >> 20) & 0x7FF;
+  const int e = max(ex, ey);
+  if (e < 2 || e > 2044) {  // subnormal or next to overflow: Smith's form
+    const bool big = fabs(a.x) >= fabs(a.y);
+    const double lo = big ? a.y : a.x, hi = big ? a.x : a.y;
+    const double r0 = lo / hi;
+    return (lane == 0 ? (big ? 1.0 : r0) : (big ? -r0 : -1.0)) / fma(lo, r0, hi);
+  }
+  const double sc = __hiloint2double((2046 - e) << 20, 0);  // 2^(1023 - e)
+  const double x = a.x * sc, y = a.y * sc;
+  return (lane == 0 ? x : -y) * quotient(1.0, divisor(fma(x, x, y * y))) * sc;
+}
+
+// The same with a row in PARTS threads: complex128, and complex64 panels of more than kRowsMax rows.
+// FP64 issue bounds the complex128 panel (64 clocks a warp instruction and quadrant, so the row's entries can
+// stay in shared memory for nothing); the search and the reciprocal of a column are integer work (quotient.cuh), as
+// long again.  So the CTA's last warp searches the next column and takes its reciprocal while the others still
+// apply the current one: a warp has 32 rows (lane = row, where it was) and every PARTS-th column after
+// the current one, the first of them before the rest, with the keys of its entries.  Two named barriers carry
+// this: kKeys (the next column's keys are there; arrivals only) and kPivot (so is its pivot).  The loops stay rolled.
+// (With the rows in registers, eight unrolled bodies, a search per warp followed by one among the warps and
+// FP64 divisions, a block column of b = 32 took 145 us, b = 128 282 us; now 81 and 182.
+// The FP64 instructions of a column, 22 a warp on average and two warps a quadrant at b = 32, are 3.3k of its 4.8k clocks.)
+// Results in sm.Pan (logical row order) / sm.perm and in global memory.
 template <typename C, int PARTS>
 __device__ void panel_lu_parts(const FactorGeom& g, const FactorPtr<C>& f, int K, const FactorSmem<C>& sm, int* sh_status,
                          int32_t* ipiv) {
   using R = typename real_of<C>::type;
-  constexpr int T = kTile, NI = T / PARTS, RPW = 32 / PARTS;
+  constexpr int T = kTile, kPivot = 1, kKeys = 2;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nbb = min(g.bt, g.Nb - 1 - K);
   const int P = (nbb + 1) * T, Pmax = (g.bt + 1) * T, ldp = Pmax + 1;
-  const int nwp = (P + RPW - 1) / RPW;  // warps that hold rows
-  const int part = lane / RPW, r = warp * RPW + (lane & (RPW - 1));
-  const bool has = r < P;
-  C w[NI];
-#pragma unroll
-  for (int i = 0; i < NI; ++i)
-    w[i] = has ? f.tiles[g.tile_index(K + r / T, K) * g.tile_elems + (r & (T - 1)) + (i * PARTS + part) * T]
-               : cmk<C>(0, 0);
-  int mylog = has ? r : 0x7fffffff;
-  int par = 0;
-#pragma unroll
-  for (int i = 0; i < NI; ++i) {
-#pragma unroll 1
-    for (int pc = 0; pc < PARTS; ++pc, par ^= 1) {
-      const int c = i * PARTS + pc;
-      PivotSlot<C>* slots = sm.slot + par * (blockDim.x >> 5);
-      if (warp < nwp) {
-        const unsigned long long key = (part == pc && has && mylog >= c) ? pivot_key(cabs1(w[i])) : 0ull;
-        const unsigned long long m = warp_max_key<R>(key);
-        const int lg = __reduce_min_sync(0xffffffffu, key == m && key > 0 ? mylog : 0x7fffffff);
-        PivotSlot<C>& sl = slots[warp];
-        if (m > 0 && mylog == lg) {
-#pragma unroll
-          for (int q = i; q < NI; ++q) sl.row[q * PARTS + part] = w[q];
-        }
-        {
-          // reciprocal of the candidate (Smith's form), its parts' divisions in two lanes at once
-          const unsigned at = __ballot_sync(0xffffffffu, m > 0 && mylog == lg && part == pc);
-          const C a = shfl_c(w[i], at ? __ffs(at) - 1 : 0);
-          const bool big = fabs(a.x) >= fabs(a.y);
-          const R r0 = (big ? a.y : a.x) / (big ? a.x : a.y);
-          const R den = big ? a.x + a.y * r0 : a.x * r0 + a.y;
-          const R q = (lane == 0 ? (big ? R(1) : r0) : (big ? -r0 : R(-1))) / den;
-          if (lane < 2) ((R*)&sl.inv)[lane] = m > 1 ? q : R(0);
-        }
-        if (lane == 0) {
-          sl.key = m;
-          sl.log = lg;
-        }
-      }
-      __syncthreads();
-      if (warp < nwp) {
-        const unsigned long long kq = lane < nwp ? slots[lane].key : 0ull;
-        const int lq = lane < nwp ? slots[lane].log : 0x7fffffff;
-        const unsigned long long m = warp_max_key<R>(kq);
-        int p = __reduce_min_sync(0xffffffffu, kq == m && m > 0 ? lq : 0x7fffffff);
-        const unsigned who = __ballot_sync(0xffffffffu, kq == m && lq == p);
-        const bool ok = m > 1;  // a positive pivot
-        if (m == 0) p = c;      // nothing but NaN: no interchange
-        if (tid == 0) {
-          const int64_t k = (int64_t)K * T + c;
-          if (ipiv && k < g.n) ipiv[k] = (int32_t)((int64_t)K * T + p);
-          if (!ok && *sh_status == 0) *sh_status = (int)(k + 1);
-        }
-        if (ok) {
-          const PivotSlot<C>& sl = slots[__ffs(who) - 1];
-          C l = cmul_rn(w[i], sl.inv);
-          l = shfl_c(l, pc * RPW + (lane & (RPW - 1)));
-          if (has && mylog >= c && mylog != p) {
-            if (part == pc)
-              w[i] = l;
-            else if (part > pc)
-              cfms(w[i], l, sl.row[i * PARTS + part]);
-#pragma unroll
-            for (int q = i + 1; q < NI; ++q) cfms(w[q], l, sl.row[q * PARTS + part]);
-          }
-        }
-        mylog = mylog == p ? c : (mylog == c ? p : mylog);
-      }
+  const int part = warp / (nbb + 1), rg = warp - part * (nbb + 1), r = rg * T + lane;
+  const bool searcher = warp == (int)(blockDim.x >> 5) - 1;
+  const bool has = part < PARTS && !searcher;  // a short last panel leaves warps without rows
+  C* W = sm.Pan + r;  // this row; column q at q ldp
+  if (has) {
+    const C* src = f.tiles + g.tile_index(K + rg, K) * g.tile_elems + lane;
+#pragma unroll 4
+    for (int q = part; q < T; q += PARTS) W[q * ldp] = src[q * T];
+    if (part == 0) {
+      sm.keys[r] = pivot_key(cabs1(W[0]));
+      sm.logs[r] = r;
     }
   }
+  int mylog = r;
+  __syncthreads();
+  if (searcher) {
+#pragma unroll 1
+    for (int c = 0; c < T; ++c) {
+      if (c > 0) asm volatile("bar.sync %0, %1;" ::"n"(kKeys), "r"(P + 32) : "memory");
+      // the largest key, the lowest logical row on ties
+      const unsigned long long* kc = sm.keys + (c & 1) * Pmax;
+      const int* lc = sm.logs + (c & 1) * Pmax;
+      unsigned long long best = 0;
+      int blog = 0x7fffffff, brow = 0;
+      for (int x = lane; x < P; x += 32) {
+        const unsigned long long k = kc[x];
+        const int lg = lc[x];
+        if (k > best || (k == best && k > 0 && lg < blog)) {
+          best = k;
+          blog = lg;
+          brow = x;
+        }
+      }
+      const unsigned long long m = warp_max_key<R>(best);
+      unsigned who = __ballot_sync(0xffffffffu, best == m);
+      if (who & (who - 1)) {
+        const int p = __reduce_min_sync(0xffffffffu, best == m ? blog : 0x7fffffff);
+        who = __ballot_sync(0xffffffffu, best == m && blog == p);
+      }
+      const int at = __ffs(who) - 1;
+      const int rs = __shfl_sync(0xffffffffu, brow, at);
+      const bool ok = m > 1;                                              // a positive pivot
+      const int p = m == 0 ? c : __shfl_sync(0xffffffffu, blog, at);  // nothing but NaN: no interchange
+      Pivot<C>* out = sm.pivot + (c & 1);
+      if (ok) {
+        const R q = pivot_reciprocal(sm.Pan[rs + c * ldp], lane);
+        if (lane < 2) ((R*)&out->inv)[lane] = q;
+      }
+      if (lane == 0) {
+        out->row = rs;
+        out->log = p;
+        out->ok = ok;
+        const int64_t k = (int64_t)K * T + c;
+        if (ipiv && k < g.n) ipiv[k] = (int32_t)((int64_t)K * T + p);
+        if (!ok && *sh_status == 0) *sh_status = (int)(k + 1);
+      }
+      asm volatile("bar.arrive %0, %1;" ::"n"(kPivot), "r"(P * PARTS + 32) : "memory");
+    }
+  } else if (has) {
+    C l = cmk<C>(0, 0);
+    bool done = false;  // l is the row's multiplier of the previous column, still to be stored
+#pragma unroll 1
+    for (int c = 0; c < T; ++c) {
+      asm volatile("bar.sync %0, %1;" ::"n"(kPivot), "r"(P * PARTS + 32) : "memory");
+      const Pivot<C> pv = sm.pivot[c & 1];
+      if (part == 0 && done) W[(c - 1) * ldp] = l;  // (column c - 1 is read no more)
+      const bool act = mylog >= c && mylog != pv.log;
+      done = pv.ok && act;
+      mylog = mylog == pv.log ? c : (mylog == c ? pv.log : mylog);
+      const C* U = sm.Pan + pv.row;
+      l = cmul_rn(W[c * ldp], pv.inv);
+      int q = c + 1 + part;
+      if (part == 0 && q < T) {  // the next column first, with its keys
+        C x = W[q * ldp];
+        if (done) {
+          cfms(x, l, U[q * ldp]);
+          W[q * ldp] = x;
+        }
+        sm.keys[((c + 1) & 1) * Pmax + r] = mylog > c ? pivot_key(cabs1(x)) : 0ull;
+        sm.logs[((c + 1) & 1) * Pmax + r] = mylog;
+        asm volatile("bar.arrive %0, %1;" ::"n"(kKeys), "r"(P + 32) : "memory");
+        q += PARTS;
+      }
+      if (done) {
+#pragma unroll 2
+        for (; q < T; q += PARTS) {
+          C x = W[q * ldp];
+          cfms(x, l, U[q * ldp]);
+          W[q * ldp] = x;
+        }
+      }
+    }
+    if (part == 0 && done) W[(T - 1) * ldp] = l;
+  }
+  // rows to their logical places
+  C w[T / PARTS];
+  __syncthreads();
   if (has) {
 #pragma unroll
-    for (int i = 0; i < NI; ++i) sm.Pan[mylog + (i * PARTS + part) * ldp] = w[i];
+    for (int i = 0; i < T / PARTS; ++i) w[i] = W[(i * PARTS + part) * ldp];
+  }
+  __syncthreads();
+  if (has) {
+#pragma unroll
+    for (int i = 0; i < T / PARTS; ++i) sm.Pan[mylog + (i * PARTS + part) * ldp] = w[i];
     if (part == 0) sm.perm[mylog] = r;
   }
   __syncthreads();
@@ -659,8 +722,10 @@ __global__ void __launch_bounds__(MAXT, MINB)
     sm.win = sm.log + kRowsMax;
     sm.perm = sm.win + T;
   } else {
-    sm.slot = (PivotSlot<C>*)align16(sm.Pan + (size_t)T * ldp);
-    sm.perm = (int*)(sm.slot + 2 * nw);
+    sm.pivot = (Pivot<C>*)align16(sm.Pan + (size_t)T * ldp);
+    sm.keys = (unsigned long long*)(sm.pivot + 2);
+    sm.logs = (int*)(sm.keys + 2 * Pmax);
+    sm.perm = sm.logs + 2 * Pmax;
   }
   int32_t* piv = ipiv ? ipiv + (int64_t)sidx * g.n : nullptr;
   if (threadIdx.x == 0) sh_status = 0;
@@ -1235,7 +1300,7 @@ static bool factor_band_ok(const FactorGeom& g, size_t es) {
 template <typename C, int PARTS, int NCF, int NC, int MAXT, int MINB>
 static int launch_factor_cluster(const FactorGeom& g, int G, int spread, int nsys, const SysDesc* d_sys,
                                  char* factor_arena, int* d_status, int32_t* d_ipiv, cudaStream_t st) {
-  const int Pmax = (g.bt + 1) * kTile, threads = PARTS > 0 ? Pmax * PARTS : MAXT;
+  const int Pmax = (g.bt + 1) * kTile, threads = PARTS > 0 ? Pmax * PARTS + 32 : MAXT;
   const size_t smem = factor_cluster_smem<C, (PARTS <= 0)>(Pmax, threads / 32, NCF > NC ? NCF : NC);
   auto kern = factor_kernel<C, PARTS, NCF, NC, MAXT, MINB>;
   PD_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1272,8 +1337,8 @@ int launch_factor(const FactorGeom& g, int cplx, const void* band, int64_t ldab,
   // The cluster: as many CTAs as still shorten a block column, while all clusters run at once (76, 36
   // and 15 clusters of 2, 4 and 8 fit at one CTA per SM).  complex64: a second CTA takes the updates off
   // the panel's chain (b = 64: 34 -> 24.5 us per block column), at b > 64 four (68, 44, 30 us for 1, 2, 4);
-  // more change nothing.  complex128: every CTA shortens the updates (b = 32: 166, 151, 145 us for 2, 4,
-  // 8; b = 128: 1432, 1110, 394, 282 for 1 to 8).
+  // more change nothing.  complex128: every CTA shortens the updates (b = 32: 203, 106, 87, 81 us for 1 to 8;
+  // b = 128: 1316, 1117, 399, 183).
   const int most = sizeof(C) == sizeof(double2) ? 8 : g.bt > 2 ? 4 : 2;
   const int G = most >= 8 && nsys <= 15 ? 8 : most >= 4 && nsys <= 36 ? 4 : nsys <= 76 ? 2 : 1;
   if constexpr (sizeof(C) == sizeof(float2)) {
@@ -1286,7 +1351,7 @@ int launch_factor(const FactorGeom& g, int cplx, const void* band, int64_t ldab,
     else  // more systems than SMs: two per SM, with some registers spilled (256 systems, b = 64: 54 against 70 us)
       PD_TRY((launch_factor_cluster<C, 0, 4, 4, 256, 2>(g, G, 0, nsys, d_sys, factor_arena, d_status, d_ipiv, st)));
   } else {
-    PD_TRY((launch_factor_cluster<C, 4, 1, 1, 640, 1>(g, G, G > 1, nsys, d_sys, factor_arena, d_status, d_ipiv, st)));
+    PD_TRY((launch_factor_cluster<C, 4, 1, 1, 672, 1>(g, G, G > 1, nsys, d_sys, factor_arena, d_status, d_ipiv, st)));
   }
   diag_inverse_kernel<C><<<dim3((unsigned)g.Nb, (unsigned)nsys), 64, 0, st>>>(g, d_sys, factor_arena);
   PD_CK_LAUNCH();

@@ -136,3 +136,19 @@ def test_default_solve_width(device, precision, b, nshift, nrhs):
             Xo = oracle.band_solve(F, ip, b, Y, trans)
             err = np.max(np.abs(block_from_dev(X[s]) - Xo)) / np.max(np.abs(Xo))
             assert err < (1e-11 if precision == pk.FP64 else 1e-4), (s, trans, err)
+
+
+@pytest.mark.parametrize("n,b,cplx", [(70, 5, False), (200, 40, True)])
+@pytest.mark.parametrize("s", [-480, 470])
+def test_fp64_solve_scales_exactly(device, n, b, cplx, s):
+    """Band and shifts times a power of two: the pivots' reciprocals are taken on scaled values, so the
+    solution is scaled exactly (no entry of the factors leaves the normal range at these powers)."""
+    import paper_2012_00506_gb300 as pk
+    ab = synth.random_band(n, b, 77, cplx)
+    Y = synth.random_subspace(n, 6, 78, True)
+    z = np.array([0.3 + 0.2j, -0.7 + 0.01j])
+    f = 2.0 ** s
+    X, i0 = pk.shifted_solve(to_dev(ab, device), z, block_to_dev(Y, device), return_ipiv=True)
+    Z, i1 = pk.shifted_solve(to_dev(ab * f, device), z * f, block_to_dev(Y, device), return_ipiv=True)
+    assert np.array_equal(i0.cpu().numpy(), i1.cpu().numpy())
+    assert np.array_equal((Z * f).cpu().numpy(), X.cpu().numpy())
