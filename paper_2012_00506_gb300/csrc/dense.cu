@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "dense.cuh"
+#include "quotient.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -510,7 +511,7 @@ __global__ void __launch_bounds__(1024) cholesky_kernel(const SmallDesc* desc, S
           break;
         }
         if (has && i == j) {
-          const double r = sqrt(dj), ri = 1.0 / r;
+          const double r = sqrt(dj), ri = divide(1.0, r);
           v = c == j ? sc<S>::from_re(r) : sc<S>::scale(v, ri);
           rowj[c] = v;
         }
@@ -1572,6 +1573,13 @@ int small_gemm(bool conjA, const std::vector<SmallDesc>& blk, int max_m, S* cons
   return launch_gemm<S>(conjA, nb, d_items, max_m, max_m, max_m, one, zero, 1, nullptr, 0, st, herm, triB, ff);
 }
 
+// the larger absolute value of the parts, as its encoding (NaN above all; integer, since an FP64 maximum takes the
+// FP64 pipe for 64 clocks)
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+  return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+}
+__device__ __forceinline__ unsigned long long abs_bits(double2 v) { return max(abs_bits(v.x), abs_bits(v.y)); }
+
 // One refinement step of an approximate eigenvector matrix V of a Hermitian A
 // (Ogita & Aishima, "Iterative refinement for symmetric eigenvalue
 // decomposition", 2018); E overwrites S.  Their separation test uses one
@@ -1595,6 +1603,8 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
   // being separated, or -inf.  Grid (blocks, kOaSplit): CTA y of a block handles
   // columns y*nw + warp (stride kOaSplit*nw); est_out[block * kOaSplit + y] is its
   // partial maximum.  Every CTA computes the (identical) lambda itself.
+  // FP64 instructions bound it: 8 complex blocks of 267 took 165 us with two hypotenuses, two square roots and a
+  // division per pair, 102 without them, 72 with 36 CTAs per block instead of 16.
   // balanced (for a last step after coarser ones): E_ij as R_ij / 2 + (S_ij + (lambda_i + lambda_j)/2 R_ij) /
   // (lambda_j - lambda_i), the same value with an exactly antihermitian second term, so that its rounding does
   // not touch the orthogonality; and couplings below 1e-14 max|lambda| of pairs far apart (|gap| > 1e8 |c_ij|)
@@ -1632,7 +1642,7 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
       const int64_t e = i + (int64_t)j * m;
       S r = sc<S>::scale(P[e], -1.0);
       if (i == j) r = sc<S>::add(r, sc<S>::from_re(1.0));
-      rmax = fmax(rmax, sqrt(sc<S>::abs2(r)));
+      rmax = fmax(rmax, sc<S>::abs2(r));  // (the square root of the largest, below)
       S ev = sc<S>::scale(r, 0.5);
       if (i != j) {
         // c_ij and |c_ji| = |S_ij + lambda_i R_ij|: the pair is classified on the
@@ -1640,15 +1650,21 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
         // (E + E^H then equals R, which keeps the orthogonality correction exact)
         const double li = lam[i];
         const S c = sc<S>::add(Sm[e], sc<S>::scale(r, lj));
-        const double ca = fmax(sc<S>::absv(c), sc<S>::absv(sc<S>::add(Sm[e], sc<S>::scale(r, li))));
+        const S ct = sc<S>::add(Sm[e], sc<S>::scale(r, li));
         const double gap = lj - li;
+        // The largest part cm bounds ca = max(|c_ij|, |c_ji|) from both sides, cm <= ca < 1.4143 cm: most pairs are
+        // separated for certain, without the two hypotenuses (half of the kernel's FP64 instructions).
+        const double cm = __longlong_as_double((long long)max(abs_bits(c), abs_bits(ct)));
+        const bool apart = cm > tiny && fabs(gap) > 5.66 * cm;
+        const double ca = apart ? cm : fmax(sc<S>::absv(c), sc<S>::absv(ct));
         if (ca > tiny) {
-          if (fabs(gap) > 4.0 * ca) {
+          if (apart || fabs(gap) > 4.0 * ca) {
+            const double rg = divide(1.0, gap);
             if (balanced)
-              ev = sc<S>::add(ev, sc<S>::scale(sc<S>::add(Sm[e], sc<S>::scale(r, 0.5 * (li + lj))), 1.0 / gap));
+              ev = sc<S>::add(ev, sc<S>::scale(sc<S>::add(Sm[e], sc<S>::scale(r, 0.5 * (li + lj))), rg));
             else
-              ev = sc<S>::scale(c, 1.0 / gap);
-            emax = fmax(emax, sqrt(sc<S>::abs2(ev)));
+              ev = sc<S>::scale(c, rg);
+            emax = fmax(emax, sc<S>::abs2(ev));
           } else if (li >= lj) {
             rj = fmax(rj, li);
           }
@@ -1667,8 +1683,8 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
   }
   __syncthreads();
   if (lane == 0) {
-    red[0][warp] = emax;
-    red[1][warp] = rmax;
+    red[0][warp] = sqrt(emax);
+    red[1][warp] = sqrt(rmax);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -1681,9 +1697,12 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
   }
 }
 
-// W[:, rank(i)] = V[:, i] * phase, eigenvalues sorted ascending (rank sort, ties by index).
+// W[:, rank(i)] = V[:, i] * phase, eigenvalues sorted ascending (rank sort, ties by index); a warp per column, the
+// columns of a block over kSortSplit CTAs (FP64 comparisons and products bound it: on one CTA per block, 8
+// blocks of 267 took 324 us, now 27).
+constexpr int kSortSplit = 16;
 template <typename S>
-__global__ void __launch_bounds__(1024) sort_phase_kernel(const SmallDesc* desc, const S* Vall, const double* lam_in,
+__global__ void __launch_bounds__(256) sort_phase_kernel(const SmallDesc* desc, const S* Vall, const double* lam_in,
                                                           double* lam_out, S* Wall, const double* aux_in = nullptr,
                                                           double* aux_out = nullptr) {
   const SmallDesc d = desc[blockIdx.x];
@@ -1693,7 +1712,7 @@ __global__ void __launch_bounds__(1024) sort_phase_kernel(const SmallDesc* desc,
   const double* li = lam_in + d.voff;
   double* lo = lam_out + d.voff;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int i = warp; i < m; i += nw) {
+  for (int i = blockIdx.y * nw + warp; i < m; i += gridDim.y * nw) {
     int rank = 0;
     for (int j = lane; j < m; j += 32) rank += (li[j] < li[i]) || (li[j] == li[i] && j < i);
     for (int o = 16; o > 0; o >>= 1) rank += __shfl_down_sync(0xffffffffu, rank, o);
@@ -1907,7 +1926,7 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
     }
     act.swap(next);
   }
-  sort_phase_kernel<S><<<nblk, 1024, 0, st>>>(d_desc, V, w.lam32, lam, W, w.reach, w.reach_sorted);
+  sort_phase_kernel<S><<<dim3(nblk, kSortSplit), 256, 0, st>>>(d_desc, V, w.lam32, lam, W, w.reach, w.reach_sorted);
   PD_CK_LAUNCH();
   // Clusters: runs of sorted eigenvalues tied together by pairs that the
   // refinement could not separate (a run extends while the next eigenvalue is
