@@ -1403,6 +1403,10 @@ static int launch_solve_cw(const FactorGeom& g, int nitems, const SysDesc* d_sys
   PD_CK(cudaGetDevice(&dev));
   PD_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   PD_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem));
+  // complex128: no more blocks on an SM than every SM has items for.  One fills the FP64 pipes, and with a block
+  // per item some SMs took two at once while others had none (152 items among 160 halves, b = 32, n = 2000:
+  // 5.05 ms, now 2.7).  complex64 blocks hide one another's latency.
+  if (std::is_same<C, double2>::value) per_sm = std::min(per_sm, std::max(1, nitems / sms));
   const int grid = std::max(1, std::min(nitems, sms * std::max(1, per_sm)));
   PD_CK(cudaMemsetAsync(counter, 0, sizeof(int), st));
   kern<<<grid, kThreads, smem, st>>>(g, d_sys, factor_arena, rhs_arena, out_arena, d_items, nitems, counter);
