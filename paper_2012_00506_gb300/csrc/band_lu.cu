@@ -12,16 +12,16 @@
 // factor_kernel: a thread-block cluster per shifted system (the L2 level of the
 //   paper's parallelism is the batch dimension; the cluster is the L3 level,
 //   inside one factorization).  Per block column K: the panel ((bt+1)T x T) is
-//   factored in registers; the panel permutation is gathered into each trailing
+//   factored by one CTA; the panel permutation is gathered into each trailing
 //   block column on load; the top tile is multiplied by the inverted unit-lower
 //   diagonal block and the tiles below get the T-deep Schur update.
 // diag_inverse_kernel: the inverses of the diagonal blocks, so that every solve
 //   step is a tile product.
-// solve kernels: one thread block per (system, 32-column block of right-hand
-//   sides); forward L sweep then backward U sweep (trans = 0), or U^H then
+// solve kernels: one thread block per (system, block of 8 to 64 right-hand
+//   sides, solve_width); forward L sweep then backward U sweep (trans = 0), or U^H then
 //   L^H and the inverse permutation (trans = 1, the conjugate node conj(z)
 //   of a Hermitian band).  Factor tiles stream from L2/HBM through shared
-//   memory; each is reused by the 32 right-hand sides of the block.
+//   memory; each is reused by the right-hand sides of the block.
 #include <cooperative_groups.h>
 
 #include <algorithm>

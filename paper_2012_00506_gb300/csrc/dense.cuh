@@ -55,7 +55,7 @@ int cluster_ctas_used();
 template <typename S>
 int launch_triinv(int nblk, const SmallDesc* d_desc, const S* R, S* Rinv, cudaStream_t st);
 
-// Hermitian Jacobi: A and Aalt (scratch like A) are overwritten, eigenvalues
+// Hermitian Jacobi: A and Aalt (scratch like A) may be overwritten, eigenvalues
 // ascending into lam (offset voff), eigenvectors into Vout (same layout as A).
 // Vwork: scratch like A.  sweeps_out[t]: sweeps used or -1 if max_sweeps hit.
 template <typename S>

@@ -1,17 +1,17 @@
 // inertia.cu -- Sylvester inertia of B - sigma I by a pivot-free LDL^T (real)
-// or LDL^H (complex) factorization in FP64, one CTA per shift sigma.
+// or LDL^H (complex) factorization in FP64, many shifts sigma at once.
 //
 // The paper counts the eigenvalues of each slice from the inertia of
 // D - b_i I at both ends of the slice (Section 3.2, "Validation and Other
 // Details"), using a band LDL^H that keeps no L.  Here the count is computed
 // for many shifts at once: a thread-block cluster of 1 to 16 CTAs per shift
 // eliminates panels of 8 columns with the active window in (distributed) shared
-// memory (inertia_panel_kernel); bands too wide for that keep the window in a
-// per-shift slice of the workspace (L2 resident), one CTA per shift and one
-// column at a time (inertia_kernel).
+// memory (inertia_panel_kernel); calls with enough shifts to fill the GPU, and
+// bands too wide for a cluster (window in a per-shift slice of the workspace, L2
+// resident), take one CTA per shift and one column at a time (inertia_kernel).
 //
-// Every floating-point operation is an explicitly rounded __dmul_rn /
-// __dsub_rn / __ddiv_rn (no contraction), in the same order as the CPU
+// Every floating-point operation is explicitly rounded (__dmul_rn, __dsub_rn, no
+// contraction; quotients to nearest, quotient.cuh), in the same order as the CPU
 // reference, so the counts and pivots are bit-reproducible:
 //   d_k = W(k,k) (zero -> -pivmin);  l_i = W(i,k) / d_k;
 //   W(i,j) -= l_i * conj(W(j,k))  for k < j <= i <= k+b,
