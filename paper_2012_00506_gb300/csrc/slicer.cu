@@ -30,6 +30,7 @@
 // Loss: mean over the batch and the 63 boundaries of the squared error.
 // Optimiser: Adam (beta1 0.9, beta2 0.999, eps 1e-8, bias-corrected).
 // Parameter vector: for each layer, W (out x in, row-major) then bias (out).
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <algorithm>
@@ -39,6 +40,8 @@
 #include "dense.cuh"
 
 namespace pdeshep {
+
+namespace cg = cooperative_groups;
 
 // from inertia.cu
 int gershgorin_device(int64_t n, int b, int cplx, const void* band, int64_t ldab, double* d_lo, double* d_hi,
@@ -231,16 +234,19 @@ static void layer_table(Layer L[4]) {
 }
 
 // The layers are small (256 x 256 weights, a batch of at most a few hundred): what costs is latency, not
-// arithmetic or bandwidth.  Each kernel copies its whole slab of the weights to shared memory at once, before it
-// waits for the kernel in front (programmatic launch: the weights are not written during a pass), then its few
-// rows of activations, and sums without further barriers; sums run over ascending k in one chain of FMAs.
-// (Only the weights are __restrict__: loads of what the kernel in front writes must not move above the wait.)
+// arithmetic or bandwidth.  So one launch takes a pass through all layers and back: a cluster of 8 CTAs has 8
+// rows of the batch, each CTA the weights of 32 units of every layer (both ways, 162 KB, on their way to shared
+// memory from the start), and hands its activations to the other seven by distributed shared memory, a
+// cluster barrier per layer.  The weight gradients, which sum over the whole batch, are a second launch, with
+// the loss and Adam's step; it brings the parameters and moments before it waits for the first.  Sums run
+// over ascending k in one chain of FMAs.
 // Measured, batch 64, one Adam step: 14 launches of 32 x 32 tiles staged 32 k at a time took 127 us of
-// device time and 158 us in all; these 8 launches take 46 us in all, with the same bits.
-constexpr int kRows = 8;           // batch rows per tile
+// device time and 158 us in all; 8 launches, a layer each, 46 us in all; these two 31 us
+// (batches of 1, 120, 256: 25, 33, 72 us back to back; a layer a launch took 36, 50, 67), all with the same bits.
+constexpr int kRows = 8;           // batch rows per cluster
+constexpr int kUnits = kHid / 8;   // units of a hidden layer per CTA
 constexpr int kPitch = kHid + 4;   // floats: 16-byte rows, 8 consecutive rows in different banks
-constexpr int kHeadRows = 4;
-constexpr size_t kHeadSmem = sizeof(float) * (kOut + kHeadRows) * kPitch;
+constexpr int kPitch0 = kFeat + 2; // ... of the first layer's weights
 
 // rows x cols floats (row stride ld) to shared memory (row stride pitch); rows at or past nrows are zero
 __device__ __forceinline__ void stage_rows(float* dst, int pitch, const float* src, int64_t ld, int rows, int nrows,
@@ -263,25 +269,95 @@ __device__ __forceinline__ void stage_rows(float* dst, int pitch, const float* s
   }
 }
 
-// Y[bt][o] = max(sum_i X[bt][i] W[o][i] + bias[o], 0): 32 outputs x 8 rows per CTA, its weights kept over
-// the row tiles; out is a multiple of 32, in <= 256
-__global__ void __launch_bounds__(128) mlp_fwd_kernel(int B, int in, int out, const float* X,
-                                                      const float* __restrict__ W, const float* __restrict__ bias,
-                                                      float* Y) {
-  __shared__ __align__(16) float Ws[32 * kPitch], Xs[kRows * kPitch];
-  const int o0 = blockIdx.y * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+// the same by asynchronous copies, of rows x cols floats that exist
+__device__ __forceinline__ void request_rows(float* dst, int pitch, const float* src, int64_t ld, int rows, int cols) {
+  const unsigned d0 = (unsigned)__cvta_generic_to_shared(dst);
+  if ((((uintptr_t)src | (uintptr_t)(ld * 4)) & 15) == 0 && (cols & 3) == 0) {
+    const int c4 = cols >> 2;
+    for (int e = threadIdx.x; e < rows * c4; e += blockDim.x) {
+      const int r = e / c4, c = e - r * c4;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d0 + 4 * (r * pitch + 4 * c)),
+                   "l"(src + r * ld + 4 * c));
+    }
+  } else {
+    for (int e = threadIdx.x; e < rows * cols; e += blockDim.x) {
+      const int r = e / cols, c = e - r * cols;
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d0 + 4 * (r * pitch + c)),
+                   "l"(src + r * ld + c));
+    }
+  }
+  asm volatile("cp.async.commit_group;\n" ::);
+}
+template <int PENDING>
+__device__ __forceinline__ void arrived() {  // all but the last PENDING requests, for the whole CTA
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(PENDING) : "memory");
+  __syncthreads();
+}
+
+struct PassBuffers {
+  float* act[4];   // [1..3]: outputs of the hidden layers
+  float* dact[5];  // [1..4]: gradients with respect to the layers' sums
+};
+
+constexpr int kPassThreads = 256;  // 8 warps copy; 4 of them sum (lane = unit, a warp two rows)
+constexpr size_t kPassFloats = (size_t)kUnits * kPitch0 + 2 * kUnits * kPitch + (kOut / 8) * kPitch + kOut * kUnits +
+                               2 * kHid * kUnits + 2 * kRows * kPitch;
+
+// Forward pass (bounds) of the rows of each cluster, with a target also the loss shares and the gradients with
+// respect to every layer's sums.  Y[o] = max(sum_i X[i] W[o][i] + bias[o], 0); softmax over the 64 outputs of
+// the last layer, cumulative sums -> 63 boundaries; dX[i] = (sum_o dY[o] W[o][i]) * [X[i] > 0].
+__global__ void __cluster_dims__(8) __launch_bounds__(kPassThreads)
+    mlp_pass_kernel(int B, const float* __restrict__ params, const float* X, float* bounds, const float* target,
+                    const PassBuffers io, float* loss_part) {
+  extern __shared__ __align__(16) float ps[];
+  __shared__ float zb[kOut];  // the logits of this CTA's row
+  __shared__ __align__(16) float p_[4][kOut], cs_[4][kOut], dc_[4][kOut], dp_[4][kOut];
+  __shared__ float red_[4][2];
+  cg::cluster_group cl = cg::this_cluster();
+  const int g = (int)cl.block_rank(), tid = threadIdx.x, tx = tid & 31, ty = tid >> 5, u0 = g * kUnits;
+  constexpr int64_t w0 = 0, b0 = w0 + kHid * kFeat, w1 = b0 + kHid, b1 = w1 + kHid * kHid, w2 = b1 + kHid,
+                    b2 = w2 + kHid * kHid, w3 = b2 + kHid, b3 = w3 + kOut * kHid;
+  float* W0 = ps;                       // [units][kPitch0], then rows of W1, W2, of the last layer
+  float* W1 = W0 + kUnits * kPitch0;    // [units][kPitch]
+  float* W2 = W1 + kUnits * kPitch;
+  float* W3 = W2 + kUnits * kPitch;     // [8][kPitch]
+  float* V3 = W3 + (kOut / 8) * kPitch; // [64][units]: columns of the last layer's weights, then of W2, W1
+  float* V2 = V3 + kOut * kUnits;       // [256][units]
+  float* V1 = V2 + kHid * kUnits;
+  float* buf = V1 + kHid * kUnits;      // [2][rows][kPitch]: a layer's input, all units
+  request_rows(W0, kPitch0, params + w0 + (int64_t)u0 * kFeat, kFeat, kUnits, kFeat);
+  request_rows(W1, kPitch, params + w1 + (int64_t)u0 * kHid, kHid, kUnits, kHid);
+  request_rows(W2, kPitch, params + w2 + (int64_t)u0 * kHid, kHid, kUnits, kHid);
+  request_rows(W3, kPitch, params + w3 + (int64_t)g * (kOut / 8) * kHid, kHid, kOut / 8, kHid);
+  if (target) {
+    request_rows(V3, kUnits, params + w3 + u0, kHid, kOut, kUnits);
+    request_rows(V2, kUnits, params + w2 + u0, kHid, kHid, kUnits);
+    request_rows(V1, kUnits, params + w1 + u0, kHid, kHid, kUnits);
+  } else {  // (empty groups: the same counts below)
+    for (int q = 0; q < 3; ++q) asm volatile("cp.async.commit_group;\n" ::);
+  }
+  const float bias[3] = {params[b0 + u0 + tx], params[b1 + u0 + tx], params[b2 + u0 + tx]};
+  const float bias3 = params[b3 + g * (kOut / 8) + (tid & 7)];
   cudaTriggerProgrammaticLaunchCompletion();
-  stage_rows(Ws, kPitch, W + (int64_t)o0 * in, in, 32, 32, in);
-  const float bo = bias[o0 + tx];
-  cudaGridDependencySynchronize();
-  const float* w = Ws + tx * kPitch;
-  const float *x0 = Xs + ty * kPitch, *x1 = Xs + (ty + 4) * kPitch;
-  for (int b0 = blockIdx.x * kRows; b0 < B; b0 += gridDim.x * kRows) {
-    __syncthreads();
-    stage_rows(Xs, kPitch, X + (int64_t)b0 * in, in, kRows, B - b0, in);
-    __syncthreads();
-    float a0 = 0.f, a1 = 0.f;
+  cl.sync();  // every CTA runs: its shared memory may be written
+  // this thread's rows ty, ty + 4 of unit u0 + tx: to every CTA's buffer and to memory
+  const bool sums = tid < kPassThreads / 2;
+  auto give = [&](float* dst, float* out, int r0, float v0, float v1) {
+    if (!sums) return;
+    if (dst)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        float* d = cl.map_shared_rank(dst, c) + u0 + tx;
+        d[ty * kPitch] = v0;
+        d[(ty + 4) * kPitch] = v1;
+      }
+    if (r0 + ty < B) out[(int64_t)(r0 + ty) * kHid + u0 + tx] = v0;
+    if (r0 + ty + 4 < B) out[(int64_t)(r0 + ty + 4) * kHid + u0 + tx] = v1;
+  };
+  auto forward = [&](const float* W, int pitch, int in, const float* x, float& a0, float& a1) {
+    a0 = a1 = 0.f;
+    if (!sums) return;
+    const float *w = W + tx * pitch, *x0 = x + ty * kPitch, *x1 = x + (ty + 4) * kPitch;
     int k = 0;
 #pragma unroll 8
     for (; k + 4 <= in; k += 4) {
@@ -299,36 +375,51 @@ __global__ void __launch_bounds__(128) mlp_fwd_kernel(int B, int in, int out, co
       a0 = fmaf(x0[k], w[k], a0);
       a1 = fmaf(x1[k], w[k], a1);
     }
-    if (b0 + ty < B) Y[(int64_t)(b0 + ty) * out + o0 + tx] = fmaxf(a0 + bo, 0.f);
-    if (b0 + ty + 4 < B) Y[(int64_t)(b0 + ty + 4) * out + o0 + tx] = fmaxf(a1 + bo, 0.f);
-  }
-}
-
-// The last layer and the head: 64 logits of 4 samples per CTA (64 threads a sample), softmax, cumulative
-// sums -> 63 boundaries.  With a target: per-sample loss share and dL/dlogits.
-__global__ void __launch_bounds__(64 * kHeadRows)
-    mlp_head_kernel(int B, const float* X, const float* __restrict__ W, const float* __restrict__ bias,
-                    float* bounds, const float* target, float* dZ,
-                    float* loss_part) {
-  extern __shared__ __align__(16) float hs[];
-  float *Ws = hs, *Xs = hs + kOut * kPitch;
-  __shared__ __align__(16) float p_[kHeadRows][kOut], cs_[kHeadRows][kOut], dc_[kHeadRows][kOut], dp_[kHeadRows][kOut];
-  __shared__ float red_[kHeadRows][2];
-  const int s4 = threadIdx.x >> 6, j = threadIdx.x & 63;
-  float *p = p_[s4], *cs = cs_[s4], *dc = dc_[s4], *dp = dp_[s4], *red = red_[s4];
-  cudaTriggerProgrammaticLaunchCompletion();
-  stage_rows(Ws, kPitch, W, kHid, kOut, kOut, kHid);
-  const float bo = bias[j];
-  cudaGridDependencySynchronize();
-  for (int b0 = blockIdx.x * kHeadRows; b0 < B; b0 += gridDim.x * kHeadRows) {
-    __syncthreads();
-    stage_rows(Xs, kPitch, X + (int64_t)b0 * kHid, kHid, kHeadRows, B - b0, kHid);
-    __syncthreads();
-    const int bt = b0 + s4;
-    const bool live = bt < B;
-    float z = 0.f;
-    {
-      const float *w = Ws + j * kPitch, *x = Xs + s4 * kPitch;
+  };
+  auto backward = [&](const float* V, int out, const float* d, float& a0, float& a1) {
+    a0 = a1 = 0.f;
+    if (!sums) return;
+    const float *d0 = d + ty * kPitch, *d1 = d + (ty + 4) * kPitch;
+#pragma unroll 4
+    for (int k = 0; k < out; k += 4) {
+      const float4 u = *(const float4*)(d0 + k), v = *(const float4*)(d1 + k);
+      const float v0 = V[k * kUnits + tx], v1 = V[(k + 1) * kUnits + tx], v2 = V[(k + 2) * kUnits + tx],
+                  v3 = V[(k + 3) * kUnits + tx];
+      a0 = fmaf(u.x, v0, a0);
+      a1 = fmaf(v.x, v0, a1);
+      a0 = fmaf(u.y, v1, a0);
+      a1 = fmaf(v.y, v1, a1);
+      a0 = fmaf(u.z, v2, a0);
+      a1 = fmaf(v.z, v2, a1);
+      a0 = fmaf(u.w, v3, a0);
+      a1 = fmaf(v.w, v3, a1);
+    }
+  };
+  float *A = buf, *Bf = buf + kRows * kPitch;
+  for (int r0 = (blockIdx.x / 8) * kRows; r0 < B; r0 += (gridDim.x / 8) * kRows) {
+    float h[3][2];
+    stage_rows(A, kPitch, X + (int64_t)r0 * kFeat, kFeat, kRows, B - r0, kFeat);
+    arrived<6>();
+    forward(W0, kPitch0, kFeat, A, h[0][0], h[0][1]);
+    for (int q = 0; q < 2; ++q) h[0][q] = fmaxf(h[0][q] + bias[0], 0.f);
+    give(Bf, io.act[1], r0, h[0][0], h[0][1]);
+    arrived<5>();
+    cl.sync();
+    forward(W1, kPitch, kHid, Bf, h[1][0], h[1][1]);
+    for (int q = 0; q < 2; ++q) h[1][q] = fmaxf(h[1][q] + bias[1], 0.f);
+    give(A, io.act[2], r0, h[1][0], h[1][1]);
+    arrived<4>();
+    cl.sync();
+    forward(W2, kPitch, kHid, A, h[2][0], h[2][1]);
+    for (int q = 0; q < 2; ++q) h[2][q] = fmaxf(h[2][q] + bias[2], 0.f);
+    give(Bf, io.act[3], r0, h[2][0], h[2][1]);
+    arrived<3>();
+    cl.sync();
+    // the last layer: 8 outputs of 8 rows, each row's to the CTA of its number
+    if (tid < 64) {
+      const int o = tid & 7, row = tid >> 3;
+      const float *w = W3 + o * kPitch, *x = Bf + row * kPitch;
+      float z = 0.f;
 #pragma unroll 8
       for (int k = 0; k < kHid; k += 4) {
         const float4 wv = *(const float4*)(w + k), u = *(const float4*)(x + k);
@@ -337,8 +428,14 @@ __global__ void __launch_bounds__(64 * kHeadRows)
         z = fmaf(u.z, wv.z, z);
         z = fmaf(u.w, wv.w, z);
       }
-      z += bo;
+      cl.map_shared_rank(zb, row)[g * 8 + o] = z + bias3;
     }
+    cl.sync();
+    // head of row r0 + g (every 64 threads, the first ones write)
+    const int bt = r0 + g, j = tid & 63, s2 = tid >> 6;
+    const bool live = bt < B, writer = live && s2 == 0;
+    float *p = p_[s2], *cs = cs_[s2], *dc = dc_[s2], *dp = dp_[s2], *red = red_[s2];
+    const float z = zb[j];
     float m = z;
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((j & 31) == 0) red[j >> 5] = m;
@@ -362,77 +459,58 @@ __global__ void __launch_bounds__(64 * kHeadRows)
       }
     }
     __syncthreads();
-    if (live && j < kOut - 1) bounds[(int64_t)bt * (kOut - 1) + j] = cs[j];
-    if (!target) continue;
-    const float scale = 1.0f / ((float)B * (float)(kOut - 1));
-    float l = 0.f;
-    if (live && j < kOut - 1) {
-      const float d = cs[j] - target[(int64_t)bt * (kOut - 1) + j];
-      l = d * d * scale;
-      dc[j] = 2.f * d * scale;
-    } else {
-      dc[j] = 0.f;
-    }
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    __syncthreads();
-    if ((j & 31) == 0) red[j >> 5] = l;
-    __syncthreads();
-    if (j == 0) {
-      if (live) loss_part[bt] = red[0] + red[1];
-      float acc = 0.f;  // dL/dp_k = sum_{i >= k} dL/dc_i
-#pragma unroll
-      for (int k = kOut - 1; k >= 0; --k) {
-        acc += dc[k];
-        dp[k] = acc;
+    if (writer && j < kOut - 1) bounds[(int64_t)bt * (kOut - 1) + j] = cs[j];
+    if (target) {
+      const float scale = 1.0f / ((float)B * (float)(kOut - 1));
+      float l = 0.f;
+      if (live && j < kOut - 1) {
+        const float d = cs[j] - target[(int64_t)bt * (kOut - 1) + j];
+        l = d * d * scale;
+        dc[j] = 2.f * d * scale;
+      } else {
+        dc[j] = 0.f;
       }
+      for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+      __syncthreads();
+      if ((j & 31) == 0) red[j >> 5] = l;
+      __syncthreads();
+      if (j == 0) {
+        if (writer) loss_part[bt] = red[0] + red[1];
+        float acc = 0.f;  // dL/dp_k = sum_{i >= k} dL/dc_i
+#pragma unroll
+        for (int k = kOut - 1; k >= 0; --k) {
+          acc += dc[k];
+          dp[k] = acc;
+        }
+      }
+      __syncthreads();
+      float sdp = p[j] * dp[j];
+      for (int o = 16; o > 0; o >>= 1) sdp += __shfl_xor_sync(0xffffffffu, sdp, o);
+      if ((j & 31) == 0) red[j >> 5] = sdp;
+      __syncthreads();
+      sdp = red[0] + red[1];
+      const float dz = p[j] * (dp[j] - sdp);
+      for (int c = s2; c < 8; c += 4) cl.map_shared_rank(A, c)[g * kPitch + j] = dz;
+      if (writer) io.dact[4][(int64_t)bt * kOut + j] = dz;
+      arrived<2>();
+      cl.sync();
+      float d0, d1;
+      backward(V3, kOut, A, d0, d1);
+      d0 = h[2][0] > 0.f ? d0 : 0.f;
+      d1 = h[2][1] > 0.f ? d1 : 0.f;
+      give(Bf, io.dact[3], r0, d0, d1);
+      arrived<1>();
+      cl.sync();
+      backward(V2, kHid, Bf, d0, d1);
+      d0 = h[1][0] > 0.f ? d0 : 0.f;
+      d1 = h[1][1] > 0.f ? d1 : 0.f;
+      give(A, io.dact[2], r0, d0, d1);
+      arrived<0>();
+      cl.sync();
+      backward(V1, kHid, A, d0, d1);
+      give(nullptr, io.dact[1], r0, h[0][0] > 0.f ? d0 : 0.f, h[0][1] > 0.f ? d1 : 0.f);
     }
-    __syncthreads();
-    float sdp = p[j] * dp[j];
-    for (int o = 16; o > 0; o >>= 1) sdp += __shfl_xor_sync(0xffffffffu, sdp, o);
-    if ((j & 31) == 0) red[j >> 5] = sdp;
-    __syncthreads();
-    sdp = red[0] + red[1];
-    if (live) dZ[(int64_t)bt * kOut + j] = p[j] * (dp[j] - sdp);
-  }
-}
-
-// dX[bt][i] = (sum_o dY[bt][o] W[o][i]) * [Xact[bt][i] > 0]: the gradient with respect to the
-// pre-activation of the previous layer (in = 256); 32 columns x 8 rows per CTA
-__global__ void __launch_bounds__(128) mlp_bwd_x_kernel(int B, int out, const float* dY,
-                                                        const float* __restrict__ W, const float* Xact,
-                                                        float* dX) {
-  __shared__ __align__(16) float Ws[kHid * 32], Ds[kRows * kPitch];
-  const int i0 = blockIdx.y * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  cudaTriggerProgrammaticLaunchCompletion();
-  stage_rows(Ws, 32, W + i0, kHid, out, out, 32);
-  cudaGridDependencySynchronize();
-  const float *d0 = Ds + ty * kPitch, *d1 = Ds + (ty + 4) * kPitch;
-  for (int b0 = blockIdx.x * kRows; b0 < B; b0 += gridDim.x * kRows) {
-    __syncthreads();
-    stage_rows(Ds, kPitch, dY + (int64_t)b0 * out, out, kRows, B - b0, out);
-    __syncthreads();
-    float a0 = 0.f, a1 = 0.f;
-#pragma unroll 4
-    for (int k = 0; k < out; k += 4) {
-      const float4 u = *(const float4*)(d0 + k), v = *(const float4*)(d1 + k);
-      const float w0 = Ws[k * 32 + tx], w1 = Ws[(k + 1) * 32 + tx], w2 = Ws[(k + 2) * 32 + tx],
-                  w3 = Ws[(k + 3) * 32 + tx];
-      a0 = fmaf(u.x, w0, a0);
-      a1 = fmaf(v.x, w0, a1);
-      a0 = fmaf(u.y, w1, a0);
-      a1 = fmaf(v.y, w1, a1);
-      a0 = fmaf(u.z, w2, a0);
-      a1 = fmaf(v.z, w2, a1);
-      a0 = fmaf(u.w, w3, a0);
-      a1 = fmaf(v.w, w3, a1);
-    }
-    for (int q = 0; q < 2; ++q) {
-      const int bt = b0 + ty + 4 * q;
-      if (bt >= B) continue;
-      const int64_t at = (int64_t)bt * kHid + i0 + tx;
-      dX[at] = Xact[at] > 0.f ? (q ? a1 : a0) : 0.f;
-    }
+    cl.sync();  // the buffers are free, and nobody leaves while others write
   }
 }
 
@@ -567,26 +645,16 @@ static int mlp_run(int B, const float* params, const float* X, float* bounds, co
                    const Adam& adam, float* loss, const MlpWs& w, cudaStream_t st) {
   Layer L[4];
   layer_table(L);
-  const int row_tiles = (int)std::min<int64_t>(ceil_div(B, kRows), 76);
-  const float* in = X;
-  for (int l = 0; l < 3; ++l) {
-    const dim3 g((unsigned)row_tiles, (unsigned)(L[l].out / 32));
-    const float *W = params + L[l].w, *bias = params + L[l].b;
-    if (l == 0) {  // reads what the caller's kernels wrote: an ordinary launch
-      mlp_fwd_kernel<<<g, 128, 0, st>>>(B, L[l].in, L[l].out, in, W, bias, w.act[1]);
-      PD_CK_LAUNCH();
-    } else {
-      PD_TRY(launch_after(mlp_fwd_kernel, g, 128, 0, st, B, L[l].in, L[l].out, in, W, bias, w.act[l + 1]));
-    }
-    in = w.act[l + 1];
-  }
-  PD_CK(cudaFuncSetAttribute(mlp_head_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeadSmem));
-  PD_TRY(launch_after(mlp_head_kernel, dim3((unsigned)std::min<int64_t>(ceil_div(B, kHeadRows), 304)), 64 * kHeadRows,
-                      kHeadSmem, st, B, in, params + L[3].w, params + L[3].b, bounds, target, w.dact[4], w.lpart));
+  PassBuffers io = {};
+  for (int l = 1; l < 4; ++l) io.act[l] = w.act[l];
+  for (int l = 1; l < 5; ++l) io.dact[l] = w.dact[l];
+  const size_t smem = sizeof(float) * kPassFloats;
+  PD_CK(cudaFuncSetAttribute(mlp_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // 15 clusters of 8 CTAs run at once; they keep their weights over the rest of the batch
+  const int clusters = (int)std::min<int64_t>(ceil_div(B, kRows), 15);
+  mlp_pass_kernel<<<(unsigned)clusters * 8, kPassThreads, smem, st>>>(B, params, X, bounds, target, io, w.lpart);
+  PD_CK_LAUNCH();
   if (!target) return 0;
-  for (int l = 3; l > 0; --l)
-    PD_TRY(launch_after(mlp_bwd_x_kernel, dim3((unsigned)row_tiles, kHid / 32), 128, 0, st, B, L[l].out, w.dact[l + 1],
-                        params + L[l].w, w.act[l], w.dact[l]));
   GradLayers G;
   G.tiles = 0;
   for (int l = 0; l < 4; ++l) {

@@ -89,10 +89,10 @@ def test_adam_step_vs_oracle(device):
     assert np.abs((p1 - p0)[sure] - (po - p0)[sure]).max() < 2e-5
 
 
-@pytest.mark.parametrize("batch", [1, 4, 7, 8, 9, 63, 64, 65, 609])
+@pytest.mark.parametrize("batch", [1, 4, 7, 8, 9, 63, 64, 65, 120, 121, 609])
 @pytest.mark.parametrize("shift", [0, 1])
 def test_train_step_vs_oracle_at_tile_edges(device, batch, shift):
-    """Batches around the kernels' tiles (4, 8 and 64 rows, and one past the 608 rows of a resident grid), and
+    """Batches around the kernels' tiles (8 and 64 rows, the 120 rows of 15 clusters, several rounds of them), and
     arrays 4 bytes off the 16-byte boundary.  With a gradient within dg = 1e-4 |grad| of the oracle's (as
     above), m moves by (1 - beta1) dg, v by (1 - beta2) 2 |g| dg and the step by lr (1 - beta1) dg / sqrt(v/c2),
     sqrt(v/c2) > 0.04; FP32 rounding adds a few units of each array's largest entry, and the powers of beta2
