@@ -1580,6 +1580,25 @@ __device__ __forceinline__ unsigned long long abs_bits(double v) {
 }
 __device__ __forceinline__ unsigned long long abs_bits(double2 v) { return max(abs_bits(v.x), abs_bits(v.y)); }
 
+// lambda_i = S_ii / P_ii of the refinement step below (CTA y of a block: i in [64 y, 64 y + 64)).  mirror: the
+// products mirror their tiles off the diagonal, but those on it (32 x 32, or 64 x 64 in float-float) hold both
+// triangles with their own rounding, which E would divide by the gap: the lower one becomes the upper one's conjugate.
+template <typename S>
+__global__ void refined_values_kernel(const SmallDesc* desc, S* Sall, S* Pall, double* lamall, int mirror) {
+  const SmallDesc d = desc[blockIdx.x];
+  const int m = d.m, i0 = blockIdx.y * 64;
+  S *Sm = Sall + d.off, *P = Pall + d.off;
+  for (int i = i0 + threadIdx.x; i < min(m, i0 + 64); i += blockDim.x)
+    lamall[d.voff + i] = sc<S>::re(Sm[i + (int64_t)i * m]) / sc<S>::re(P[i + (int64_t)i * m]);
+  if (!mirror) return;
+  for (int e = threadIdx.x; e < 64 * 64; e += blockDim.x) {
+    const int i = i0 + (e & 63), j = i0 + (e >> 6);
+    if (i <= j || i >= m) continue;
+    Sm[i + (int64_t)j * m] = sc<S>::conj(Sm[j + (int64_t)i * m]);
+    P[i + (int64_t)j * m] = sc<S>::conj(P[j + (int64_t)i * m]);
+  }
+}
+
 // One refinement step of an approximate eigenvector matrix V of a Hermitian A
 // (Ogita & Aishima, "Iterative refinement for symmetric eigenvalue
 // decomposition", 2018); E overwrites S.  Their separation test uses one
@@ -1587,7 +1606,7 @@ __device__ __forceinline__ unsigned long long abs_bits(double2 v) { return max(a
 // coupling, which keeps the step quadratic on the separated pairs while the
 // others are left to the cluster treatment.
 template <typename S>
-__global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall, const S* Pall, double* lamall,
+__global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall, const S* Pall, const double* lamall,
                                                   double* est_out, double* reach_all, int balanced) {
   // One refinement step (Ogita and Aishima, 2018) for block t, given S = V^H A V
   // and P = V^H V of the current approximate eigenvectors V:
@@ -1602,7 +1621,8 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
   // reach_j = the largest lambda_i >= lambda_j (i != j) coupled to j without
   // being separated, or -inf.  Grid (blocks, kOaSplit): CTA y of a block handles
   // columns y*nw + warp (stride kOaSplit*nw); est_out[block * kOaSplit + y] is its
-  // partial maximum.  Every CTA computes the (identical) lambda itself.
+  // partial maximum.  lambda comes from refined_values_kernel: E overwrites S, its diagonal too, so a CTA that
+  // starts late cannot take it from here.
   // FP64 instructions bound it: 8 complex blocks of 267 took 165 us with two hypotenuses, two square roots and a
   // division per pair, 102 without them, 72 with 36 CTAs per block instead of 16.
   // balanced (for a last step after coarser ones): E_ij as R_ij / 2 + (S_ij + (lambda_i + lambda_j)/2 R_ij) /
@@ -1613,17 +1633,13 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
   const int m = d.m;
   S* Sm = Sall + d.off;
   const S* P = Pall + d.off;
-  double* lam = lamall + d.voff;
+  const double* lam = lamall + d.voff;
   double* reach = reach_all + d.voff;
   __shared__ double red[2][32];
   __shared__ double sh_l;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   double lmax = 0.0;
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    const double l = sc<S>::re(Sm[i + (int64_t)i * m]) / sc<S>::re(P[i + (int64_t)i * m]);
-    lam[i] = l;
-    lmax = fmax(lmax, fabs(l));
-  }
+  for (int i = threadIdx.x; i < m; i += blockDim.x) lmax = fmax(lmax, fabs(lam[i]));
   for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_down_sync(0xffffffffu, lmax, o));
   if (lane == 0) red[0][warp] = lmax;
   __syncthreads();
@@ -1891,6 +1907,8 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
       S* abc[3] = {V, V, w.T};  // P = V^H V  (in T)
       PD_TRY(small_gemm<S>(true, sub_d, max_m, abc, 1, 0, w.items, st, ff));
     }
+    refined_values_kernel<S><<<dim3(na, (max_m + 63) / 64), 256, 0, st>>>(dd, w.W64, w.T, w.lam32, w.rough);
+    PD_CK_LAUNCH();
     oa_kernel<S><<<dim3(na, kOaSplit), 256, 0, st>>>(dd, w.W64, w.T, w.lam32, w.delta, w.reach, w.rough);
     PD_CK_LAUNCH();
     for (auto& b : sub_d)

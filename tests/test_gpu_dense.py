@@ -132,3 +132,23 @@ def test_eigh_degenerate_spectra(device):
         assert np.max(np.abs(lam - np.linalg.eigvalsh(A))) < 1e-13 * nrm
         assert np.max(np.abs(A @ V - V * lam)) < 1e-12 * nrm
         assert np.max(np.abs(V.T @ V - np.eye(A.shape[0]))) < 1e-12
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("nblk,m", [(16, 130), (40, 33), (150, 20)])
+def test_eigh_many_blocks(device, cplx, nblk, m):
+    """More blocks than one wave of CTAs holds in the refinement and the sort: every block's eigenvalues and
+    vectors stand on their own."""
+    import torch
+    import paper_2012_00506_gb300 as pk
+    rng = np.random.default_rng(3 * nblk + m)
+    mats = []
+    for t in range(nblk):
+        A = rng.normal(size=(m - t % 3, m - t % 3)) + (1j * rng.normal(size=(m - t % 3, m - t % 3)) if cplx else 0)
+        mats.append(0.5 * (A + A.conj().T))
+    for A, (lam, V) in zip(mats, pk.eigh([torch.from_numpy(A).to(device) for A in mats])):
+        lam, V = lam.cpu().numpy(), V.cpu().numpy()
+        nrm = max(1.0, np.linalg.norm(A))
+        assert np.max(np.abs(lam - np.linalg.eigvalsh(A))) < 1e-13 * nrm
+        assert np.max(np.abs(V.conj().T @ V - np.eye(len(lam)))) < 1e-13
+        assert np.max(np.abs(A @ V - V * lam)) < 1e-13 * nrm
