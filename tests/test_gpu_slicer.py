@@ -89,7 +89,7 @@ def test_adam_step_vs_oracle(device):
     assert np.abs((p1 - p0)[sure] - (po - p0)[sure]).max() < 2e-5
 
 
-@pytest.mark.parametrize("batch", [1, 4, 7, 8, 9, 63, 64, 65, 120, 121, 609])
+@pytest.mark.parametrize("batch", [1, 4, 7, 8, 9, 63, 64, 65, 120, 609])
 @pytest.mark.parametrize("shift", [0, 1])
 def test_train_step_vs_oracle_at_tile_edges(device, batch, shift):
     """Batches around the kernels' tiles (8 and 64 rows, the 120 rows of 15 clusters, several rounds of them), and
