@@ -8,6 +8,7 @@
 // slice with the matrix in L2 and cluster barriers between phases.
 #include <cooperative_groups.h>
 
+#include <float.h>
 #include <stdlib.h>
 
 #include <algorithm>
@@ -1684,7 +1685,8 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
           } else if (li >= lj) {
             rj = fmax(rj, li);
           }
-        } else if (balanced && fabs(gap) > 1e8 * ca) {
+        } else if (balanced && ca > 0.0 && fabs(gap) > 1e8 * ca && fabs(gap) >= DBL_MIN) {
+          // (without coupling there is nothing to correct, and 1 / gap of a subnormal gap is infinite)
           ev = sc<S>::add(ev, sc<S>::scale(sc<S>::add(Sm[e], sc<S>::scale(r, 0.5 * (li + lj))), 1.0 / gap));
         }
       }

@@ -152,3 +152,19 @@ def test_eigh_many_blocks(device, cplx, nblk, m):
         assert np.max(np.abs(lam - np.linalg.eigvalsh(A))) < 1e-13 * nrm
         assert np.max(np.abs(V.conj().T @ V - np.eye(len(lam)))) < 1e-13
         assert np.max(np.abs(A @ V - V * lam)) < 1e-13 * nrm
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("d", [[1e-310, -1e-310], [1.0, -1.0, 3e-310, -3e-310], [5e-324, 0.0, 2.0, -2.0]])
+def test_eigh_subnormal_gaps(device, cplx, d):
+    """Diagonal matrices with eigenvalues a subnormal distance apart (the mean of the diagonal is 0 or harmless):
+    nothing has to be rotated, so eigenvalues and vectors are exact."""
+    import torch
+    import paper_2012_00506_gb300 as pk
+    A = np.diag(np.array(d, dtype=np.complex128 if cplx else np.float64))
+    (lam, V), = pk.eigh([torch.from_numpy(A).to(device)])
+    lam, V = lam.cpu().numpy(), V.cpu().numpy()
+    assert np.all(np.isfinite(V))
+    assert np.array_equal(np.abs(V) != 0, np.abs(V) == 1)
+    assert np.array_equal(V.conj().T @ V, np.eye(len(d)))
+    assert np.max(np.abs(lam - np.sort(d))) <= 2e-16 * np.max(np.abs(d))
