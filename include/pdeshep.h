@@ -467,9 +467,12 @@ int pdeshep_block_gemm(int32_t kind, int32_t arith, int64_t n, int32_t is_comple
 /* (offset sum_{u<t} m_u), eigenvectors into d_v (same layout as d_a), each   */
 /* scaled so its first largest-magnitude component is real positive.         */
 /* Cyclic Jacobi in parallel (round-robin) order on a thread-block cluster    */
-/* per block: FP32 sweeps give V32, then H = V32^H A V32 (FP64) is nearly     */
-/* diagonal and FP64 sweeps finish it (off(H) <= 1e-14 ||H||_F); the          */
-/* eigenvectors are V32 W.                                                    */
+/* per block gives FP32 starting vectors; refinement steps in FP64 (batched   */
+/* products) finish them, in large calls after up to three steps with         */
+/* float-float products (about 48 bits) that only bring the start closer:     */
+/* every eigenvalue and vector comes from a step in FP64.  Pairs the          */
+/* refinement leaves coupled are resolved by FP64 Jacobi on their columns, a  */
+/* block that does not converge by FP64 Jacobi on the whole of it.            */
 /* ------------------------------------------------------------------------ */
 size_t pdeshep_eigh_workspace_size(int32_t nblk, const int32_t* h_m, int32_t is_complex);
 int pdeshep_eigh(int32_t is_complex, int32_t nblk, const int32_t* h_m, void* d_a, double* d_lam,

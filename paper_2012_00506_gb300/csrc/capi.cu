@@ -211,7 +211,7 @@ static int eigh(int nblk, const int32_t* m, S* A, double* lam, S* V, void* work,
     mm = std::max(mm, (int)m[t]);
   }
   PD_CK(cudaMemcpyAsync(d_desc, desc.data(), sizeof(SmallDesc) * nblk, cudaMemcpyHostToDevice, st));
-  w.rough = 1;
+  w.coarse = 1;
   PD_TRY(eigh_mixed<S>(nblk, d_desc, desc.data(), mm, A, lam, V, w, st));
   std::vector<int> sw(nblk);
   PD_CK(cudaMemcpyAsync(sw.data(), w.sweeps, sizeof(int) * nblk, cudaMemcpyDeviceToHost, st));

@@ -1608,7 +1608,8 @@ __global__ void refined_values_kernel(const SmallDesc* desc, S* Sall, S* Pall, d
 // others are left to the cluster treatment.
 template <typename S>
 __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall, const S* Pall, const double* lamall,
-                                                  double* est_out, double* reach_all, int balanced) {
+                                                  double* est_out, double* reach_all, double coupled,
+                                                  int balanced) {
   // One refinement step (Ogita and Aishima, 2018) for block t, given S = V^H A V
   // and P = V^H V of the current approximate eigenvectors V:
   //   lambda_i = S_ii / P_ii, R = I - P, c_ij = S_ij + lambda_j R_ij,
@@ -1616,7 +1617,7 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
   //   E_ij = R_ij / 2                       otherwise (and on the diagonal),
   // and V <- V (I + E) (done by the caller).  A separated pair gets |E_ij| < 1/4
   // and converges quadratically.  A pair that is not separated although it is
-  // coupled (|c_ij| > 1e-14 max|lambda|) belongs to a cluster: its coupling is
+  // coupled (|c_ij| > `coupled` max|lambda|) belongs to a cluster: its coupling is
   // left alone here and resolved by the caller.  Outputs: est = max(|E_ij| over
   // separated pairs, |R_ij|), the size of the correction, and per column j
   // reach_j = the largest lambda_i >= lambda_j (i != j) coupled to j without
@@ -1626,9 +1627,9 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
   // starts late cannot take it from here.
   // FP64 instructions bound it: 8 complex blocks of 267 took 165 us with two hypotenuses, two square roots and a
   // division per pair, 102 without them, 72 with 36 CTAs per block instead of 16.
-  // balanced (for a last step after coarser ones): E_ij as R_ij / 2 + (S_ij + (lambda_i + lambda_j)/2 R_ij) /
+  // balanced (for a refinement whose first steps are coarser): E_ij as R_ij / 2 + (S_ij + (lambda_i + lambda_j)/2 R_ij) /
   // (lambda_j - lambda_i), the same value with an exactly antihermitian second term, so that its rounding does
-  // not touch the orthogonality; and couplings below 1e-14 max|lambda| of pairs far apart (|gap| > 1e8 |c_ij|)
+  // not touch the orthogonality; and couplings below `coupled` max|lambda| of pairs far apart (|gap| > 1e8 |c_ij|)
   // are corrected as well: the coarser steps leave some of that size.
   const SmallDesc d = desc[blockIdx.x];
   const int m = d.m;
@@ -1650,7 +1651,7 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
     sh_l = a;
   }
   __syncthreads();
-  const double tiny = 1e-14 * sh_l;
+  const double tiny = coupled * sh_l;
   double emax = 0.0, rmax = 0.0;
   for (int j = blockIdx.y * nw + warp; j < m; j += gridDim.y * nw) {
     const double lj = lam[j];
@@ -1876,20 +1877,13 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
   // separated pairs.  A block leaves the batch after the step whose correction was
   // below kRefineTol (what remains is of the order of its square); at most
   // kRefineSteps steps.
-  // w.rough: steps whose correction will be above kRefineTol by the square of the last one run their products
-  // in float-float: the next step corrects what that leaves (a block leaves only after a step in FP64, so S, P,
-  // lambda and the last correction are computed as before).  One of three or four steps is then in FP64
-  // (8 blocks of 267 complex columns: 4.4 ms a step against 2.4).
-  double est_max = 1.0;
   S* V = w.Vd;
   S* Vn = w.Vw;
   std::vector<double> drel(nblk, 1.0), est(nblk), estp((size_t)nblk * kOaSplit);
-  std::vector<int> act(nblk);
-  for (int t = 0; t < nblk; ++t) act[t] = t;
-  for (int it = 0; it < kRefineSteps && !act.empty(); ++it) {
+  std::vector<int> act, next;
+  // one step on the blocks of act; their corrections in est[0 ..)
+  auto refine_step = [&](int ff, double coupled) -> int {
     const int na = (int)act.size();
-    const bool rough = w.rough && it + 1 < kRefineSteps && est_max * est_max > kRefineTol;
-    const int ff = w.ff || rough;
     std::vector<SmallDesc> sub_d(na);
     for (int q = 0; q < na; ++q) sub_d[q] = all[act[q]];
     const SmallDesc* dd = d_desc;
@@ -1909,9 +1903,9 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
       S* abc[3] = {V, V, w.T};  // P = V^H V  (in T)
       PD_TRY(small_gemm<S>(true, sub_d, max_m, abc, 1, 0, w.items, st, ff));
     }
-    refined_values_kernel<S><<<dim3(na, (max_m + 63) / 64), 256, 0, st>>>(dd, w.W64, w.T, w.lam32, w.rough);
+    refined_values_kernel<S><<<dim3(na, (max_m + 63) / 64), 256, 0, st>>>(dd, w.W64, w.T, w.lam32, w.coarse);
     PD_CK_LAUNCH();
-    oa_kernel<S><<<dim3(na, kOaSplit), 256, 0, st>>>(dd, w.W64, w.T, w.lam32, w.delta, w.reach, w.rough);
+    oa_kernel<S><<<dim3(na, kOaSplit), 256, 0, st>>>(dd, w.W64, w.T, w.lam32, w.delta, w.reach, coupled, w.coarse);
     PD_CK_LAUNCH();
     for (auto& b : sub_d)
       PD_CK(cudaMemcpyAsync(Vn + b.off, V + b.off, sizeof(S) * (size_t)b.m * b.m, cudaMemcpyDeviceToDevice, st));
@@ -1935,14 +1929,36 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
       for (int c = 0; c < kOaSplit; ++c) est[q] = std::max(est[q], estp[(size_t)q * kOaSplit + c]);
     }
     if (rep) rep->refine_steps += 1;
-    std::vector<int> next;
-    est_max = 0.0;
-    for (int q = 0; q < na; ++q) {
-      drel[act[q]] = est[q];
-      if (!(est[q] < kRefineTol) || (rough && !w.ff)) {
-        next.push_back(act[q]);
-        est_max = std::max(est_max, est[q]);
+    return 0;
+  };
+  // w.coarse: the starting vectors are first improved by steps in float-float (8 blocks of 267 complex columns:
+  // 2.4 ms a step against 4.4).  A block leaves these when the next correction will be below kRefineTol, when
+  // its correction no longer falls to a quarter (nothing but pairs that float-float does not resolve is left), or after
+  // kCoarseSteps; every result then comes from the FP64 steps below, as from any other start.  S carries noise of
+  // about 1e-14 max|lambda| here, so pairs coupled below kCoarseCoupled are not rotated: a pair that close would
+  // be turned by noise / gap in every step, and its block would never leave (gaps of 1e-14 to 1e-10 of the spread
+  // took all ten steps and then the Jacobi sweeps).
+  if (w.coarse) {
+    std::vector<double> last(nblk, INFINITY);
+    for (int t = 0; t < nblk; ++t) act.push_back(t);
+    for (int it = 0; it < kCoarseSteps && !act.empty(); ++it) {
+      PD_TRY(refine_step(1, kCoarseCoupled));
+      next.clear();
+      for (size_t q = 0; q < act.size(); ++q) {
+        if (est[q] * est[q] > kRefineTol && est[q] <= 0.25 * last[act[q]]) next.push_back(act[q]);
+        last[act[q]] = est[q];
       }
+      act.swap(next);
+    }
+    act.clear();
+  }
+  for (int t = 0; t < nblk; ++t) act.push_back(t);
+  for (int it = 0; it < kRefineSteps && !act.empty(); ++it) {
+    PD_TRY(refine_step(w.ff, kCoupled));
+    next.clear();
+    for (size_t q = 0; q < act.size(); ++q) {
+      drel[act[q]] = est[q];
+      if (!(est[q] < kRefineTol)) next.push_back(act[q]);
     }
     act.swap(next);
   }

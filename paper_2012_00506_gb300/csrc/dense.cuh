@@ -93,7 +93,7 @@ struct EighScratch {
   int* csweeps;
   double* cjscratch;
   int ff = 0;               // float-float products in the refinement (set by the caller)
-  int rough = 0;            // FP64 refinement with its first steps in float-float (set by the caller)
+  int coarse = 0;           // FP64 refinement after a few steps in float-float (set by the caller)
 };
 // columns i0..i0+c-1 of the m x m block at element offset off (eigenvalues at voff)
 struct ClusterRef {
@@ -103,6 +103,9 @@ struct ClusterRef {
 constexpr int kMaxCluster = 64;
 constexpr int kRefineSteps = 10;
 constexpr double kRefineTol = 1e-8;
+constexpr double kCoupled = 1e-14;        // pairs with |c_ij| below this times max|lambda| count as uncoupled
+constexpr int kCoarseSteps = 3;           // float-float steps before the FP64 ones, at most
+constexpr double kCoarseCoupled = 1e-12;  // ... and their bound on |c_ij|
 constexpr int kOaSplit = 36;  // CTAs per block in one refinement step (8 warps a CTA: one column a warp up to m = 288)
 template <typename S>
 EighScratch<S> plan_eigh_scratch(Arena& a, int64_t msq, int64_t mtot, int nblk);

@@ -586,7 +586,7 @@ struct Feast {
     if (carve) {
       p = q;
       eig.ff = ff();
-      eig.rough = o->precision == PDESHEP_FP64;
+      eig.coarse = o->precision == PDESHEP_FP64;
     }
     return a.used();
   }

@@ -168,3 +168,27 @@ def test_eigh_subnormal_gaps(device, cplx, d):
     assert np.array_equal(np.abs(V) != 0, np.abs(V) == 1)
     assert np.array_equal(V.conj().T @ V, np.eye(len(d)))
     assert np.max(np.abs(lam - np.sort(d))) <= 2e-16 * np.max(np.abs(d))
+
+
+# Calls above and below the size from which the refinement's first steps are taken in float-float.
+@pytest.mark.parametrize("cplx,nblk,m", [(False, 2, 60), (True, 1, 160), (True, 6, 160), (False, 6, 267), (True, 2, 267)])
+@pytest.mark.parametrize("gap", [0.0, 1e-14, 1e-12, 1e-11, 1e-10])
+def test_eigh_of_doublets(device, cplx, nblk, m, gap):
+    """Blocks of close pairs (gap in units of the spread) and some simple eigenvalues."""
+    import torch
+    import paper_2012_00506_gb300 as pk
+    rng = np.random.default_rng(m + nblk)
+    mats = []
+    for t in range(nblk):
+        Q, _ = np.linalg.qr(rng.normal(size=(m, m)) + (1j * rng.normal(size=(m, m)) if cplx else 0))
+        pairs = m // 2 if t % 2 == 0 else 3
+        base = rng.uniform(-0.5, 0.5, pairs)
+        d = np.concatenate([base, base + gap, rng.uniform(-0.5, 0.5, m - 2 * pairs)])
+        A = (Q * d) @ Q.conj().T
+        mats.append(0.5 * (A + A.conj().T))
+    for A, (lam, V) in zip(mats, pk.eigh([torch.from_numpy(A).to(device) for A in mats])):
+        lam, V = lam.cpu().numpy(), V.cpu().numpy()
+        nrm = max(1.0, np.linalg.norm(A))
+        assert np.max(np.abs(lam - np.linalg.eigvalsh(A))) < 1e-13 * nrm
+        assert np.max(np.abs(V.conj().T @ V - np.eye(len(lam)))) < 1e-13
+        assert np.max(np.abs(A @ V - V * lam)) < 1e-13 * nrm

@@ -441,3 +441,48 @@ def test_trapezoid_rule_through_gpu_feast(device):
         assert oracle.subspace_sin_angle(V[:, off:off + cnt], o["evecs"][:, :cnt]) <= 1e-8
         assert oracle.orth_max(V[:, off:off + cnt]) <= orth_tol(n, 2)
         off += m0[i]
+
+
+def _doubled_band(n, b, cplx, seed, gap):
+    """Two interleaved copies of one band, the second shifted by gap: every eigenvalue is a doublet."""
+    ab = synth.random_band(n, b, seed, cplx)
+    two = np.zeros((2 * n, 2 * b + 1), dtype=ab.dtype)
+    two[0::2, 0::2] = ab
+    two[1::2, 0::2] = ab
+    two[1::2, 0] += gap
+    return ab, two
+
+
+# Orders of the projected matrices and slices of one call, small and large calls of the eigensolver.
+@pytest.mark.parametrize("cplx,pairs,nslices", [(False, 23, 2), (True, 23, 2), (False, 62, 20), (True, 62, 6),
+                                                (False, 103, 8), (True, 103, 3)])
+@pytest.mark.parametrize("gap", [0.0, 1e-14, 1e-12, 1e-11, 1e-10])
+def test_fp64_slices_of_doublets_need_no_fallback(device, cplx, pairs, nslices, gap):
+    """Close pairs (gap in units of a slice's width) in every slice: the refinement of the projected
+    eigenproblems converges by itself, on the blocks far from diagonal and on the others."""
+    import paper_2012_00506_gb300 as pk
+    n1, k0 = pairs * nslices + 60, 30
+    ab1, _ = _doubled_band(n1, 4, cplx, 90 + pairs, 0.0)
+    ev = np.linalg.eigvalsh(synth.band_to_dense(ab1))
+    ks = k0 + pairs * np.arange(nslices + 1)
+    bounds = [0.5 * (ev[k - 1] + ev[k]) for k in ks]
+    gap *= (bounds[-1] - bounds[0]) / nslices
+    ab1, ab = _doubled_band(n1, 4, cplx, 90 + pairs, gap)
+    m0 = [oracle.m0_rule(2 * pairs)] * nslices
+    X0 = synth.random_subspace(2 * n1, sum(m0), 6, cplx)
+    bnorm = float(np.max(np.abs(ev)))
+    r = pk.band_slice(to_dev(ab, device), bounds, m0, block_to_dev(X0, device), precision=pk.FP64, bnorm=bnorm,
+                      max_iter=30)
+    assert r.status == 0
+    st = r.stats
+    assert st["eig_refine_steps"] > 0
+    assert st["eig_fallback_unconverged"] == 0 and st["jacobi_sweeps64"] == 0, st
+    off = 0
+    for i in range(nslices):
+        assert r.counts[i] == r.nfound[i] == 2 * pairs
+        want = np.sort(np.concatenate([ev[ks[i]:ks[i + 1]], ev[ks[i]:ks[i + 1]] + gap]))
+        got = r.evals.cpu().numpy()[off:off + 2 * pairs]
+        X = block_from_dev(r.evecs)[:, off:off + 2 * pairs]
+        assert np.max(np.abs(got - want)) < 1e-12 * bnorm
+        assert oracle.orth_max(X) <= 1e-13
+        off += m0[i]
