@@ -1940,7 +1940,8 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
   // took all ten steps and then the Jacobi sweeps).
   if (w.coarse) {
     std::vector<double> last(nblk, INFINITY);
-    for (int t = 0; t < nblk; ++t) act.push_back(t);
+    for (int t = 0; t < nblk; ++t)  // (one FP64 step is enough for most blocks that start from the identity)
+      if (h_fp32 == nullptr || h_fp32[t]) act.push_back(t);
     for (int it = 0; it < kCoarseSteps && !act.empty(); ++it) {
       PD_TRY(refine_step(1, kCoarseCoupled));
       next.clear();

@@ -486,3 +486,22 @@ def test_fp64_slices_of_doublets_need_no_fallback(device, cplx, pairs, nslices, 
         assert np.max(np.abs(got - want)) < 1e-12 * bnorm
         assert oracle.orth_max(X) <= 1e-13
         off += m0[i]
+
+
+@pytest.mark.parametrize("cplx,count,nslices", [(False, 205, 8), (True, 205, 3), (True, 40, 2)])
+def test_fp64_slices_from_eigenvectors_take_one_refinement_step(device, cplx, count, nslices):
+    """Projected matrices that are diagonal to rounding start from the identity (no FP32 sweeps); one FP64
+    refinement step per Rayleigh-Ritz call is then enough."""
+    import paper_2012_00506_gb300 as pk
+    n = 200 + count * nslices + 160
+    ab = synth.random_band(n, 4, 5, cplx)
+    ev, V = np.linalg.eigh(synth.band_to_dense(ab))
+    ks = 100 + count * np.arange(nslices + 1)
+    bounds = [0.5 * (ev[k - 1] + ev[k]) for k in ks]
+    m0 = oracle.m0_rule(count)
+    cols = np.concatenate([np.arange(m0) + k - (m0 - count) // 2 for k in ks[:-1]])
+    r = pk.band_slice(to_dev(ab, device), bounds, [m0] * nslices, block_to_dev(V[:, cols], device), precision=pk.FP64,
+                      bnorm=float(np.max(np.abs(ev))))
+    assert r.status == 0 and list(r.nfound) == [count] * nslices
+    assert r.stats["jacobi_sweeps32"] == 0 and r.stats["jacobi_sweeps64"] == 0
+    assert r.stats["eig_refine_steps"] == r.stats["rr_calls"], r.stats
