@@ -1937,11 +1937,17 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
   // kCoarseSteps; every result then comes from the FP64 steps below, as from any other start.  S carries noise of
   // about 1e-14 max|lambda| here, so pairs coupled below kCoarseCoupled are not rotated: a pair that close would
   // be turned by noise / gap in every step, and its block would never leave (gaps of 1e-14 to 1e-10 of the spread
-  // took all ten steps and then the Jacobi sweeps).
+  // took all ten steps and then the Jacobi sweeps).  Below kCoarseWork the products are bound by their latency and the
+  // float-float ones are no shorter: a whole eigh of one complex block of 267 (7.6e7) 11.7 ms with, 11.3 without them, of
+  // 150 5.5 and 4.9, 8 complex ones of 80 (1.6e7) 3.5 and 3.35; of 4 complex ones of 200 (1.2e8) 8.65 and 9.7, 8 of
+  // 267 (6e8) 21.6 and 25.3, 8 real ones of 267 (1.5e8) 14.5 and 14.8.
   if (w.coarse) {
     std::vector<double> last(nblk, INFINITY);
     for (int t = 0; t < nblk; ++t)  // (one FP64 step is enough for most blocks that start from the identity)
       if (h_fp32 == nullptr || h_fp32[t]) act.push_back(t);
+    double work = 0.0;
+    for (int t : act) work += (double)all[t].m * all[t].m * all[t].m * (sizeof(S) == sizeof(double2) ? 4.0 : 1.0);
+    if (work < kCoarseWork) act.clear();
     for (int it = 0; it < kCoarseSteps && !act.empty(); ++it) {
       PD_TRY(refine_step(1, kCoarseCoupled));
       next.clear();

@@ -106,6 +106,7 @@ constexpr double kRefineTol = 1e-8;
 constexpr double kCoupled = 1e-14;        // pairs with |c_ij| below this times max|lambda| count as uncoupled
 constexpr int kCoarseSteps = 3;           // float-float steps before the FP64 ones, at most
 constexpr double kCoarseCoupled = 1e-12;  // ... and their bound on |c_ij|
+constexpr double kCoarseWork = 8e7;       // ... taken from this many real multiplications of one m x m product on
 constexpr int kOaSplit = 36;  // CTAs per block in one refinement step (8 warps a CTA: one column a warp up to m = 288)
 template <typename S>
 EighScratch<S> plan_eigh_scratch(Arena& a, int64_t msq, int64_t mtot, int nblk);
