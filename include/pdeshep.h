@@ -67,8 +67,8 @@ typedef struct {
   int32_t max_iter;        /* FEAST iterations per slice; default 20 */
   int32_t precision;       /* PDESHEP_FP64 or PDESHEP_MIXED; default PDESHEP_MIXED */
   int32_t refine_policy;   /* PDESHEP_REFINE_*; default PDESHEP_REFINE_RESIDUAL */
-  int32_t rhs_chunk;       /* right-hand sides per solve work item: 16, 32 or 64 (a thread per
-                              row of a 32-row tile, the window in shared memory), 128 (complex64
+  int32_t rhs_chunk;       /* right-hand sides per solve work item: 8 (PDESHEP_FP64 only), 16, 32 or 64 (a
+                              thread per row of a 32-row tile, the window in shared memory), 128 (complex64
                               factors only: a thread per right-hand side, the window in tensor
                               memory, b <= 128) or 256 (complex64 factors only: the tile products
                               on the tensor cores as bf16x6 MMAs into tensor memory, items of 128
@@ -92,7 +92,7 @@ typedef struct {
                               iteration */
   int32_t autotune;        /* 0 off; 1 use the tuned choice for this problem shape, measuring
                               it on first use; 2 measure again.  Tuned: the solve column block
-                              (16/32/64/128 and whether 256 serves the first passes, unless
+                              (FP64 8/16/32/64, mixed 16/32/64/128 and whether 256 serves the first passes, unless
                               rhs_chunk is set) and the split count of the tall Gram products
                               (2/4/8) */
   int32_t verbose;         /* 0 quiet */

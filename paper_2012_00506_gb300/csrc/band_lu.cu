@@ -1439,7 +1439,7 @@ int launch_solve_queued(const FactorGeom& g, int trans, int nitems, const SysDes
     case 128: return launch_solve_cw<C, 64, 0>(g, nitems, d_sys, factor_arena, rhs_arena, out_arena, queue, st);
     case 129: return launch_solve_cw<C, 64, 1>(g, nitems, d_sys, factor_arena, rhs_arena, out_arena, queue, st);
     default:
-      set_last_error_msg("right-hand-side block width must be 16, 32 or 64");
+      set_last_error_msg("right-hand-side block width must be 8 (FP64), 16, 32 or 64");
       return PDESHEP_CUDA_ERROR;
   }
 }
@@ -1476,7 +1476,7 @@ int launch_solve(const FactorGeom& g, int trans, int nsys, const SysDesc* h_sys,
   if (nsys <= 0) return 0;
   if (chunk <= 0) chunk = solve_width(g, sizeof(C), nsys, h_sys);
   if (chunk != 8 && chunk != 16 && chunk != 32 && chunk != 64 && chunk != kTmChunk && chunk != kTcChunk) {
-    set_last_error_msg("right-hand-side block width must be 16, 32, 64, 128 or 256");
+    set_last_error_msg("right-hand-side block width must be 8 (FP64), 16, 32, 64, 128 or 256");
     return PDESHEP_CUDA_ERROR;
   }
   int nitems = 0;

@@ -1599,7 +1599,7 @@ int check_slice_args(int64_t n, int32_t b, const void* d_band, int64_t ldab, int
   if (o && (!(o->tol > 0.0) || o->max_iter < 0 || (o->precision != PDESHEP_FP64 && o->precision != PDESHEP_MIXED) ||
             !(o->ellipse_ratio > 0.0) ||
             (o->rhs_chunk != 0 && o->rhs_chunk != 16 && o->rhs_chunk != 32 && o->rhs_chunk != 64 &&
-             o->rhs_chunk != 128 && o->rhs_chunk != 256) ||
+             o->rhs_chunk != 128 && o->rhs_chunk != 256 && !(o->rhs_chunk == 8 && o->precision == PDESHEP_FP64)) ||
             (o->rr_arith != PDESHEP_RR_FLOATFLOAT && o->rr_arith != PDESHEP_RR_FP64 &&
              o->rr_arith != PDESHEP_RR_TENSOR) || o->autotune < 0 ||
             o->autotune > 2 || (o->m0_resize != 0 && o->m0_resize != 1)))

@@ -505,3 +505,39 @@ def test_fp64_slices_from_eigenvectors_take_one_refinement_step(device, cplx, co
     assert r.status == 0 and list(r.nfound) == [count] * nslices
     assert r.stats["jacobi_sweeps32"] == 0 and r.stats["jacobi_sweeps64"] == 0
     assert r.stats["eig_refine_steps"] == r.stats["rr_calls"], r.stats
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+def test_fp64_rhs_block_widths_and_the_reported_one(device, cplx):
+    """FP64 solves give the same bits for work items of 8, 16, 32 and 64 right-hand sides, launched directly or from
+    graphs; the width a default call reports is one that a call accepts."""
+    import torch
+    import paper_2012_00506_gb300 as pk
+    ab, bounds, m0, X0 = _small_problem(device, cplx, n=700, b=9, ks=(40, 69, 110, 112))
+    band = to_dev(ab, device)
+    bn = oracle.spectral_norm(ab)
+    s = torch.cuda.Stream()
+    outs = []
+    with torch.cuda.stream(s):
+        def call(cw, graphs, precision=pk.FP64):
+            r = pk.band_slice(band, bounds, m0, block_to_dev(X0, device), precision=precision, bnorm=bn, rhs_chunk=cw,
+                              graphs=graphs, stream=s, max_iter=30)
+            s.synchronize()
+            assert r.status == 0 and list(r.nfound) == list(r.counts)
+            return r
+
+        for cw in (0, 8, 16, 32, 64):
+            for graphs in (0, 1):
+                r = call(cw, graphs)
+                assert cw == 0 or r.stats["rhs_chunk_used"] == cw
+                assert (r.stats["graph_launches"] > 0) == (graphs == 1)
+                outs.append(r)
+        used = outs[0].stats["rhs_chunk_used"]
+        outs.append(call(used, 0))
+        assert outs[-1].stats["rhs_chunk_used"] == used == 8
+        with pytest.raises(pk.PdeshepError) as e:
+            call(8, 0, pk.MIXED)
+        assert e.value.status == -15
+    for r in outs[1:]:
+        assert np.array_equal(r.evals.cpu().numpy(), outs[0].evals.cpu().numpy())
+        assert np.array_equal(r.evecs.cpu().numpy(), outs[0].evecs.cpu().numpy())
