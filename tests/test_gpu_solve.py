@@ -152,3 +152,21 @@ def test_fp64_solve_scales_exactly(device, n, b, cplx, s):
     Z, i1 = pk.shifted_solve(to_dev(ab * f, device), z * f, block_to_dev(Y, device), return_ipiv=True)
     assert np.array_equal(i0.cpu().numpy(), i1.cpu().numpy())
     assert np.array_equal((Z * f).cpu().numpy(), X.cpu().numpy())
+
+
+def test_fp64_pivot_reciprocals_are_correctly_rounded(device):
+    """Blocks [[z - a, -1], [-1, z - d]] with z = 2^-40 i and d = fl(1 / a): the second pivot is (z - d) minus the
+    reciprocal of the first.  In Smith's form the real part of that reciprocal is fl(1 / -a) = -d (the correction
+    y^2 / a is below a rounding of a), so the second pivot is imaginary to the last bit, and with it the
+    solution's second entry for (0, 1); an error of one unit in the last place would make its real part 1e-4 of it."""
+    import paper_2012_00506_gb300 as pk
+    nb = 500
+    a = 1.0 + np.random.default_rng(2).uniform(size=nb)
+    ab = np.zeros((2 * nb, 2))
+    ab[0::2, 0] = a
+    ab[0::2, 1] = 1.0
+    ab[1::2, 0] = 1.0 / a
+    Y = np.zeros((2 * nb, 1), dtype=np.complex128)
+    Y[1::2] = 1.0
+    X = block_from_dev(pk.shifted_solve(to_dev(ab, device), np.array([1j * 2.0 ** -40]), block_to_dev(Y, device))[0])
+    assert np.all(X[1::2].real == 0.0) and np.all(X[1::2].imag != 0.0)
