@@ -170,3 +170,41 @@ def test_fp64_pivot_reciprocals_are_correctly_rounded(device):
     Y[1::2] = 1.0
     X = block_from_dev(pk.shifted_solve(to_dev(ab, device), np.array([1j * 2.0 ** -40]), block_to_dev(Y, device))[0])
     assert np.all(X[1::2].real == 0.0) and np.all(X[1::2].imag != 0.0)
+
+
+# One case per panel kernel: at most 160 rows (with clusters, and two systems per SM), at most 256, wider; complex128.
+@pytest.mark.parametrize("b,nshift,precision", [(40, 3, 1), (40, 160, 1), (120, 2, 1), (200, 3, 1), (300, 2, 1),
+                                                (40, 2, 0), (70, 40, 0), (128, 80, 0)])
+@pytest.mark.parametrize("first", [0, 64])
+def test_ties_with_displaced_rows_take_the_lowest_logical_row(device, b, nshift, precision, first):
+    """Pairs of columns k, k + 1 of one panel: k takes its pivot (4) from row p, so row k moves down to p; the
+    largest entries of column k + 1 are then a 2 in row r and a 2 in the displaced row.  gbtrf takes the one that
+    stands higher now, row r if r < p, although the other row was the higher one before.  All numbers are
+    dyadic, so pivots and multipliers are exact in both precisions."""
+    import paper_2012_00506_gb300 as pk
+    rng = np.random.default_rng(b)
+    n = first + b + 70
+    groups = min(16, (b - 31) // 2)
+    rows = first + rng.permutation(np.arange(32, b + 1))[:2 * groups]
+    ab = np.zeros((n, b + 1))
+    want = first + np.arange(32)
+    displaced = 0
+    for q in range(groups):
+        k, p, r = first + 2 * q, rows[2 * q], rows[2 * q + 1]
+        ab[k, p - k] = 4.0
+        ab[k, 1] = 2.0
+        ab[k + 1, r - k - 1] = 2.0
+        want[2 * q:2 * q + 2] = p, min(p, r)
+        displaced += r < p
+    assert 2 <= displaced < groups
+    z = 1j * 0.5 ** (np.arange(nshift) % 3)
+    Y = synth.random_subspace(n, 2, 79, True)
+    X, ipiv = pk.shifted_solve(to_dev(ab, device), z, block_to_dev(Y, device), precision=precision, return_ipiv=True)
+    ipiv = ipiv.cpu().numpy()
+    for s in range(nshift):
+        assert np.array_equal(ipiv[s][first:first + 32], want)
+        if s < 3:
+            F, ip, info = oracle.band_lu(ab, z[s])
+            assert np.array_equal(ip[first:first + 32], want)
+            Xo = oracle.band_solve(F, ip, b, Y, 0)
+            assert np.max(np.abs(block_from_dev(X[s]) - Xo)) < (1e-11 if precision == 0 else 1e-4) * np.max(np.abs(Xo))
