@@ -126,6 +126,48 @@ def test_train_step_vs_oracle_at_tile_edges(device, batch, shift):
     assert np.abs(tr.v.cpu().numpy() - vo).max() <= 1e-3 * 2 * np.abs(go).max() * dg + 4 * eps * vo.max()
 
 
+def _rows_off_the_kinks(params, rng, batch):
+    """Input rows for which no unit's sum lies within its worst FP32 rounding error of zero, so that FP32 and FP64
+    take the same side of every ReLU: a k-term sum of products of values known to e errs by at most
+    (k + 2) 2^-24 (|W| (|x| + e) + |b|) + |W| e."""
+    X = rng.normal(size=(80 * batch, 98)).astype(np.float32)
+    x, e, ok = X.astype(np.float64), 0.0 * X, np.ones(len(X), dtype=bool)
+    for W, b in so.unpack(params)[:3]:
+        z = x @ W.T + b
+        e = (W.shape[1] + 2) * 2.0 ** -24 * ((np.abs(x) + e) @ np.abs(W).T + np.abs(b)) + e @ np.abs(W).T
+        ok &= np.all(np.abs(z) > e, axis=1)
+        x = np.maximum(z, 0.0)
+    assert ok.sum() >= batch, ok.mean()
+    return X[ok][:batch]
+
+
+@pytest.mark.parametrize("batch", [119, 120, 121, 128, 240, 241])
+def test_train_step_of_more_rows_than_the_clusters_hold(device, batch):
+    """Batches around the 120 rows that 15 clusters hold at once, with one live row in the last round, and around
+    twice that.  Bounds as in test_train_step_vs_oracle_at_tile_edges."""
+    import torch
+    from paper_2012_00506_gb300 import slicer
+    g_ = np.random.default_rng(700 + batch)
+    up = lambda x: torch.from_numpy(x).to(device)
+    p0 = _params(31, device).cpu().numpy()
+    X = _rows_off_the_kinks(p0.astype(np.float64), g_, batch)
+    T = np.sort(g_.uniform(size=(batch, 63)), axis=1).astype(np.float32)
+    tr = slicer.Trainer(up(p0), lr=1e-3, max_batch=batch)
+    m0 = (1e-2 * g_.normal(size=p0.shape)).astype(np.float32)
+    v0 = (1e-4 + 1e-4 * g_.uniform(size=p0.shape)).astype(np.float32)
+    tr.m, tr.v, tr.t = up(m0), up(v0), 50
+    lo, go = so.loss_and_grad(p0.astype(np.float64), X.astype(np.float64), T.astype(np.float64))
+    loss = tr.step(up(X), up(T))
+    po, mo, vo = so.adam_step(p0.astype(np.float64), go, m0.astype(np.float64), v0.astype(np.float64), 51, 1e-3,
+                              b1=float(np.float32(0.9)), b2=float(np.float32(0.999)))
+    assert abs(float(loss.item()) - lo) <= 1e-5 * lo
+    eps, dg = 2.0 ** -23, 1e-4 * np.linalg.norm(go)
+    step = np.abs(po - p0).max()
+    assert np.abs(tr.params.cpu().numpy() - po).max() <= 1e-3 * 0.1 * dg / 0.04 + 1e-5 * step + eps * np.abs(p0).max()
+    assert np.abs(tr.m.cpu().numpy() - mo).max() <= 0.1 * dg + 4 * eps * np.abs(mo).max()
+    assert np.abs(tr.v.cpu().numpy() - vo).max() <= 1e-3 * 2 * np.abs(go).max() * dg + 4 * eps * vo.max()
+
+
 def _check_counts(ab, pr, frac, nslices, tol, exact_targets=True):
     n = ab.shape[0]
     bd = pr.bounds
