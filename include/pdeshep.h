@@ -77,8 +77,8 @@ typedef struct {
                               ones); a nonzero value serves every filter pass.  0 = the first four
                               passes on the tensor cores where they apply and are not measured
                               slower, the later passes on the fastest FP32-FMA width (measured when
-                              autotune is on, else 16 or 32 by the number of systems and columns; FP64
-                              factors 8 to 64) */
+                              autotune is on, else 16, 32 or 128 by the number of systems and columns and
+                              by b; FP64 factors 8 to 64) */
   double ellipse_ratio;    /* vertical / horizontal semi-axis of the contour; default 0.3 */
   double bnorm;            /* ||B||_2 for the residual; <= 0: computed by the library */
   uint64_t seed;           /* start vectors drawn by the library when d_x0 is NULL (see

@@ -1438,28 +1438,41 @@ int launch_solve_queued(const FactorGeom& g, int trans, int nitems, const SysDes
   }
 }
 
-// The column block of the tiled solve for these systems: the least waves of items over 152 SMs times an
-// item's time.  complex128 is bound by its SM's FP64 pipe, an item's time by its columns (b = 32: 1.34,
-// 2.58, 5.04, 10.0 us per row for 8, 16, 32, 64 columns; 152 items of 8 run 3.8 times as fast as 40 of
-// 32).  complex64 items are bound by the chain of a step while they are alone on an SM (b = 64: 0.31, 0.42,
-// 0.69 us per row for 16, 32, 64) and by the SM's throughput when several share it (0.215, 0.35, 0.7 each);
-// 64 columns, and the 128 of the tensor-memory kernel (1.14), never won.
+// The column block of the solve for these systems, by an item's time and the items of 152 SMs.
+// complex128 is bound by its SM's FP64 pipe, an item's time by its columns (b = 32: 1.34, 2.58, 5.04, 10.0 us
+// per row for 8, 16, 32, 64 columns, in the same ratios from b = 8 to 128; 152 items of 8 run 3.8 times as fast as
+// 40 of 32).
+// complex64, us per row: items of 16 and 32 columns are bound by the chain of a step while they are alone on an SM and
+// by the SM's throughput when several share it, with a loss in the last, unfilled round; an item of 128 columns of the
+// tensor-memory kernel has an SM for itself.  Fitted to 144 calls (b = 16, 64, 128, 8 to 152 systems of 60 to
+// 384 columns): the choice costs 0.2% over the best width on average, 13% at most.  Few systems are fastest with 16
+// columns (b = 64, 8 of 200: 0.33 against 0.45 and 1.09), full rounds of 128 columns with 128 (b = 64, 64 of
+// 250: 1.52, 1.34, 1.12; b = 128, 128 of 250: 5.06, 4.47, 3.51).  64 columns never won.
 int solve_width(const FactorGeom& g, size_t es, int nsys, const SysDesc* h_sys) {
   const bool dbl = es == sizeof(double2);
   int best = 16;
   double best_t = 1e300;
-  for (int cw = dbl ? 8 : 16; cw <= (dbl ? 64 : 32); cw *= 2) {
-    if (cw > 16 && solve_smem_bytes(g, cw, es, 0) > 227 * 1024) break;
+  auto rounds = [&](int cw) {  // items per SM
     int64_t items = 0;
     for (int s = 0; s < nsys; ++s) items += ceil_div(h_sys[s].ncols, cw);
-    const double waves = (double)ceil_div(items, 152);
-    const double t = dbl ? waves * (0.1 + 0.155 * cw)
-                         : std::max(cw == 16 ? 0.31 : 0.42, waves * (cw == 16 ? 0.215 : 0.35));
-    if (t < best_t) {
-      best_t = t;
-      best = cw;
-    }
+    return (double)items / 152.0;
+  };
+  auto consider = [&](int cw, double t) {
+    if (t >= best_t) return;
+    best_t = t;
+    best = cw;
+  };
+  for (int cw = dbl ? 8 : 16; cw <= (dbl ? 64 : 32); cw *= 2) {
+    if (cw > 16 && solve_smem_bytes(g, cw, es, 0) > 227 * 1024) break;
+    const double r = rounds(cw);
+    if (dbl)
+      consider(cw, ceil(r) * (0.1 + 0.155 * cw));
+    else if (cw == 16)
+      consider(16, std::max(0.107 + 0.11 * g.bt, 0.11 + (0.0285 + 0.0816 * g.bt) * (0.65 * r + 0.35 * ceil(r))));
+    else
+      consider(32, std::max(0.13 + 0.155 * g.bt, 0.17 + (0.0343 + 0.1423 * g.bt) * (0.6 * r + 0.4 * ceil(r))));
   }
+  if (!dbl && solve_tm_supported(g)) consider(kTmChunk, ceil(rounds(kTmChunk)) * (0.49 + 0.3125 * g.bt));
   return best;
 }
 

@@ -541,3 +541,21 @@ def test_fp64_rhs_block_widths_and_the_reported_one(device, cplx):
     for r in outs[1:]:
         assert np.array_equal(r.evals.cpu().numpy(), outs[0].evals.cpu().numpy())
         assert np.array_equal(r.evecs.cpu().numpy(), outs[0].evecs.cpu().numpy())
+
+
+@pytest.mark.parametrize("nslices,b,m0,width", [(8, 128, 250, 128), (16, 120, 128, 128), (8, 64, 256, 128), (1, 128, 60, 16),
+                                                (8, 30, 120, 32)])
+def test_late_pass_width(device, nslices, b, m0, width):
+    """The default column block of the passes after the fourth: the tensor-memory kernel's where its items of 128
+    columns fill the SMs, else 16 or 32 (a tolerance out of reach keeps every slice active)."""
+    import paper_2012_00506_gb300 as pk
+    n = 640
+    ab = synth.random_band(n, b, 11, True)
+    ev = np.linalg.eigvalsh(synth.band_to_dense(ab))
+    ks = 40 + (30 if nslices > 8 else 50) * np.arange(nslices + 1)
+    bounds = [0.5 * (ev[k - 1] + ev[k]) for k in ks]
+    X0 = synth.random_subspace(n, m0 * nslices, 12, True)
+    r = pk.band_slice(to_dev(ab, device), bounds, [m0] * nslices, block_to_dev(X0, device), precision=pk.MIXED,
+                      bnorm=float(np.max(np.abs(ev))), tol=1e-18, max_iter=5, raise_on_error=False)
+    assert r.stats["iterations"] == 5 and r.stats["rhs_chunk_early"] == 256
+    assert r.stats["rhs_chunk_used"] == width, r.stats
