@@ -50,6 +50,23 @@ def test_forward_vs_oracle(device):
     assert np.all(np.diff(c, axis=1) >= 0)
 
 
+@pytest.mark.parametrize("shift", [0, 1])
+def test_forward_of_large_batches(device, shift):
+    """More than 960 rows take 32 x 32 tiles, a launch per layer: the same bits as parts that take the one launch, on
+    arrays that are aligned and arrays 4 bytes off."""
+    import torch
+    import paper_2012_00506_gb300 as pk
+    from paper_2012_00506_gb300 import slicer
+    p = _params(4, device)
+    X = torch.from_numpy(np.random.default_rng(8).normal(size=(2050 * 98 + 4,)).astype(np.float32)).to(device)
+    X = X[shift:shift + 2050 * 98].view(2050, 98)
+    parts = torch.cat([slicer.mlp_forward(p, X[i:i + 410]) for i in range(0, 2050, 410)])
+    for batch in (960, 961, 1023, 2050):
+        n0 = pk.kernel_launches()
+        got = slicer.mlp_forward(p, X[:batch])
+        assert pk.kernel_launches() - n0 == (1 if batch <= 960 else 5)
+        assert torch.equal(got, parts[:batch])
+
 @pytest.mark.parametrize("batch", [1, 37, 64])
 def test_gradient_vs_oracle(device, batch):
     import torch
