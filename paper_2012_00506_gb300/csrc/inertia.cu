@@ -657,15 +657,36 @@ static int panel_clusters(int b, int G) {
   return nc;
 }
 
+// CTAs of inertia_kernel that share an SM, cached per device and band.
+template <bool CPLX>
+static int single_per_sm(int b) {
+  static std::mutex mu;
+  static std::map<std::pair<int, int>, int> known;
+  int dev = 0, per = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  std::lock_guard<std::mutex> lk(mu);
+  const auto it = known.find(std::make_pair(dev, b));
+  if (it != known.end()) return it->second;
+  const size_t smem = single_smem(b, CPLX);
+  cudaError_t e = cudaFuncSetAttribute(inertia_kernel<CPLX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, inertia_kernel<CPLX>, 256, smem);
+  if (e != cudaSuccess) cudaGetLastError();
+  if (known.size() > 4096) known.clear();
+  return known[std::make_pair(dev, b)] = std::max(per, 1);
+}
+
 // The cluster size for nsigma shifts, or 0 for one CTA per shift and one column per step
 // (inertia_kernel): the least estimated clocks per column of a fit to measured times.  Panel kernel:
 // the panel's chain (a division and an update, in one warp per column or through two barriers), the
 // rest of a round (barriers, row entry, triangle), the CTA's share of the updates at 76 clocks per
 // warp instruction and FP64 pipe; CTAs that share an SM share its pipes.  `sms` is what clusters of G
-// reach at one CTA per SM.  Fitted to 254 calls (b = 8 .. 140, real and complex, 1 .. 504 shifts, every G): the
-// choice costs 1.1% over the best G on average, 30% at most, and is nowhere slower than one CTA per
-// shift.  At b = 64 complex the measured times cross between 63 shifts (4.3 us per column in clusters
-// of 4 or 2 against 6.6) and 110 (7.3 against 6.65).
+// reach at one CTA per SM.  One CTA per shift runs in rounds of all that fit on the chip, the last one with fewer to
+// an SM.  Checked on 605 calls (b = 0 .. 150, real and complex, 1 .. 2500 shifts, every G): the choice costs 1.5%
+// over the best G on average and is at most 6% slower than one CTA per shift.  (Rounds counted in full, and
+// at eight to an SM where registers allow five, sent calls of many shifts to the panel kernel, which has no
+// advantage there: n = 1000, b = 32 complex, 1500 shifts 22.7 ms against 16.3, b = 40, 504 shifts 11.8 against 10.0.)  At
+// b = 64 complex the measured times cross between 63 shifts (4.3 us per column in clusters of 4 or 2 against
+// 6.6) and 110 (7.3 against 6.65).  A diagonal band has nothing to update.
 // beside: the counts run on a side stream next to factorizations that need whole SMs, and nobody waits
 // for them until two filter passes are done, so they keep to about 20 CTAs (9 shifts of n = 8192, b = 64
 // complex on 112 SMs stretched a factorization of 64 systems from 6.4 to 18 ms).
@@ -678,11 +699,11 @@ static int panel_cluster_size(int b, int nsigma, bool single_ok, bool beside) {
   int best = -1;
   double best_t = 0.0;
   if (single_ok) {
+    if (b == 0) return 0;
     const double div = np * 221.0 * ceil_div(b, 32);
-    const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(8, 227 * 1024 / (single_smem(b, CPLX) + 1024)));
-    const int waves = (int)ceil_div(nsigma, 152 * per_sm);
-    const double co = (double)ceil_div(std::min(nsigma, 152 * per_sm), 152);
-    best_t = 0.92 * waves * std::max(work + div + 2280.0 + 11.5 * ops, co * (1.09 * work + div + 395.0));
+    const int per_sm = single_per_sm<CPLX>(b), rest = nsigma % (152 * per_sm);
+    auto round = [&](double co) { return std::max(work + div + 2280.0 + 11.5 * ops, co * (1.09 * work + div + 395.0)); };
+    best_t = 0.92 * (nsigma / (152 * per_sm) * round(per_sm) + (rest ? round((double)ceil_div(rest, 152)) : 0.0));
     best = 0;
   }
   for (int G = 1, q = 0; G <= 16; G *= 2, ++q) {
@@ -694,7 +715,8 @@ static int panel_cluster_size(int b, int nsigma, bool single_ok, bool beside) {
     const double co = (double)ceil_div((int64_t)std::min(nsigma, nc) * G, sms[q]);
     const double upd = 1.01 * work / G + 38.0, pan = chunks * (6.85 + 2.19 * ops) * 19.0 + 122.0;
     const double chain = (chunks == 1 ? 525.0 + 82.5 * ops : 1660.0 + 227.0 * ops) + (G > 1 ? 547.0 : 375.0);
-    const double t = waves * std::max((co > 1 ? 1.35 : 1.0) * (chain + upd), co * (upd + pan));
+    const double shared = co > 1 ? (CPLX && chunks > 1 ? 1.55 : 1.35) : 1.0;
+    const double t = (waves > 1 ? 1.02 : 1.0) * waves * std::max(shared * (chain + upd), co * (upd + pan));
     if (best < 0 || t < best_t) {
       best = G;
       best_t = t;

@@ -158,3 +158,20 @@ def test_quotients_are_rounded_to_nearest(device, nsig, kind):
     for i in (0, nsig - 1):
         assert np.array_equal(piv[i][0::2], d)
         assert np.array_equal(piv[i][1::2], want, equal_nan=True)
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("n,b", [(70, 0), (120, 3), (150, 24), (200, 56)])
+def test_counts_of_many_and_few_shifts_agree(device, n, b, cplx):
+    """Calls of one shift to several rounds of the chip (900, 1600) take different kernels: the same counts, and
+    the oracle's."""
+    import paper_2012_00506_gb300 as pk
+    ab = synth.random_band(n, b, 4000 + b, cplx)
+    lo, hi = oracle.gershgorin(ab)
+    sig = lo + (hi - lo) * (np.arange(1600) + 0.5) / 1600
+    band = to_dev(ab, device)
+    all_ = pk.inertia(band, sig)
+    assert np.array_equal(pk.inertia(band, sig[:900]), all_[:900])
+    assert np.array_equal(pk.inertia(band, sig[700:830]), all_[700:830])
+    for k in (3, 799, 1598):
+        assert pk.inertia(band, sig[k:k + 1])[0] == all_[k] == oracle.inertia(ab, sig[k])
