@@ -107,13 +107,13 @@ __global__ void __launch_bounds__(256) gemm_kernel(const GemmItem<S>* items, S a
 // the low word and lo*lo is dropped.  Relative accuracy of a length-K dot
 // product is about 2^-48 sqrt(K) in practice, far inside the 1e-10 residual
 // target; the exponent range is FP32's (operands above ~1e-19 in magnitude
-// keep full precision).  Tiles: 32 x 64 outputs per CTA of 256 threads, 4 x 2
-// per thread, k-steps of 16 staged in shared memory as (hi, lo) pairs (with 64 x 64
-// tiles one block of 267 is 25 CTAs on 152 SMs: its products in one refinement
-// step 660 -> 400 us).  herm: 64 x 64 blocks on or above the diagonal.
+// keep full precision).  Tiles: FBM x 64 outputs per CTA of 8 FBM threads, 4 x 2
+// per thread, k-steps of 16 staged in shared memory as (hi, lo) pairs; FBM = 32
+// (with 64 one block of 267 is 25 CTAs on 152 SMs: its products in one refinement
+// step took 660 us, 400 with 32), or 64 for complex products of many tiles
+// (ff_tall_tiles).  herm: 64 x 64 blocks on or above the diagonal.
 // ---------------------------------------------------------------------------
-constexpr int FBM = 32, FBN = 64, FBK = 16, FFT = 256;
-constexpr int FHB = 64 / FBM;
+constexpr int FBN = 64, FBK = 16;
 
 template <typename S>
 struct ffv;  // a split operand in shared memory
@@ -170,9 +170,10 @@ __device__ __forceinline__ double2 ff_val(const ffacc2& a) {
   return make_double2((double)a.rh + (double)a.rl, (double)a.ih + (double)a.il);
 }
 
-template <typename S, bool CA>
-__global__ void __launch_bounds__(FFT) ffgemm_kernel(const GemmItem<S>* items, S alpha, S beta, int splits,
-                                                    S* part, int64_t part_stride, int herm, int triB) {
+template <typename S, bool CA, int FBM>
+__global__ void __launch_bounds__(8 * FBM) ffgemm_kernel(const GemmItem<S>* items, S alpha, S beta, int splits,
+                                                        S* part, int64_t part_stride, int herm, int triB) {
+  constexpr int FFT = 8 * FBM, FHB = 64 / FBM, ROWS = FBM / 4;
   using V = typename ffv<S>::type;
   using ACC = typename std::conditional<std::is_same<S, double2>::value, ffacc2, ffacc1>::type;
   // two stages of the (hi, lo) tiles: the next k-step's operands are fetched
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(FFT) ffgemm_kernel(const GemmItem<S>* items, S
   const int klim = triB ? min(it.k, j0 + FBN) : it.k;
   const int kper = ((klim + splits - 1) / splits + FBK - 1) / FBK * FBK;
   const int kb = split * kper, ke = min(klim, kb + kper);
-  // thread (tx, ty) owns rows ty + 8 q (q < 4) and columns tx + 32 r (r < 2)
+  // thread (tx, ty) owns rows ty + ROWS q (q < 4) and columns tx + 32 r (r < 2)
   const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
   constexpr int NA = (FBM * FBK) / FFT, NB = (FBN * FBK) / FFT;
   S ra[NA], rb[NB];
@@ -247,7 +248,7 @@ __global__ void __launch_bounds__(FFT) ffgemm_kernel(const GemmItem<S>* items, S
     for (int kk = 0; kk < FBK; ++kk) {
       V a[4], b[2];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) a[q] = As[stg][kk][ty + 8 * q];
+      for (int q = 0; q < 4; ++q) a[q] = As[stg][kk][ty + ROWS * q];
 #pragma unroll
       for (int r = 0; r < 2; ++r) b[r] = Bs[stg][kk][tx + 32 * r];
 #pragma unroll
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(FFT) ffgemm_kernel(const GemmItem<S>* items, S
   for (int q = 0; q < 4; ++q)
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-      const int i = i0 + ty + 8 * q, j = j0 + tx + 32 * r;
+      const int i = i0 + ty + ROWS * q, j = j0 + tx + 32 * r;
       if (i >= it.m || j >= it.n) continue;
       const S val = ff_val(acc[q][r]);
       if (splits > 1) {
@@ -298,6 +299,27 @@ __global__ void gemm_reduce_kernel(const GemmItem<S>* items, S alpha, S beta, in
   }
 }
 
+// Whether a complex float-float product takes tiles of 64 rows: they split B's operands half as often but an SM holds one
+// (512 threads) where it holds two of 32 rows.  In units of a 64-row tile's time a 32-row tile takes 0.6 alone on
+// its SM and 1.11 beside another: 8 blocks of 267, n = 8192, Q W 10.9 ms against 12.3, one of 267, n = 5000, Q W
+// 0.97 ms against 1.09, Q^H Q 0.75 against 0.84; but one 267 x 267 product 325 us against 196, of 8 642
+// against 554.  Real tiles of 64 rows were never faster.
+static bool ff_tall_tiles(int max_m, int max_n, int nitems, int splits, int herm) {
+  const int64_t tn = ceil_div(max_n, FBN), t64 = ceil_div(max_m, 64), t32 = ceil_div(max_m, 32);
+  int64_t n64 = t64 * tn, n32 = t32 * tn;
+  if (herm) {  // blocks on or above the diagonal
+    n64 = n32 = 0;
+    for (int64_t j = 0; j < tn; ++j) {
+      n64 += std::min(t64, j + 1);
+      n32 += std::min(t32, 2 * (j + 1));
+    }
+  }
+  n64 *= (int64_t)nitems * splits;
+  n32 *= (int64_t)nitems * splits;
+  const int64_t rest = n32 % (2 * 152);
+  return (double)ceil_div(n64, 152) < 1.11 * (double)(n32 / (2 * 152)) + (rest > 152 ? 1.11 : rest > 0 ? 0.6 : 0.0);
+}
+
 template <typename S>
 int launch_gemm(bool conjA, int nitems, const GemmItem<S>* d_items, int max_m, int max_n, int max_k, S alpha,
                 S beta, int splits, S* part, int64_t part_stride, cudaStream_t st, int herm, int triB, int ff) {
@@ -305,15 +327,18 @@ int launch_gemm(bool conjA, int nitems, const GemmItem<S>* d_items, int max_m, i
   if (max_k <= 0) splits = 1;
   if (splits < 1) splits = 1;
   if (ff) {
-    dim3 grid((unsigned)(ceil_div(max_m, FBM) * ceil_div(max_n, FBN)), (unsigned)nitems, (unsigned)splits);
-    const size_t smem = 2 * sizeof(typename ffv<S>::type) * FBK * (FBM + FBN);
-    if (conjA) {
-      PD_CK(cudaFuncSetAttribute(ffgemm_kernel<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      ffgemm_kernel<S, true><<<grid, FFT, smem, st>>>(d_items, alpha, beta, splits, part, part_stride, herm, triB);
-    } else {
-      PD_CK(cudaFuncSetAttribute(ffgemm_kernel<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      ffgemm_kernel<S, false><<<grid, FFT, smem, st>>>(d_items, alpha, beta, splits, part, part_stride, herm, triB);
+    auto kern = conjA ? ffgemm_kernel<S, true, 32> : ffgemm_kernel<S, false, 32>;
+    int fbm = 32;
+    if constexpr (std::is_same<S, double2>::value) {
+      if (ff_tall_tiles(max_m, max_n, nitems, splits, herm)) {
+        kern = conjA ? ffgemm_kernel<S, true, 64> : ffgemm_kernel<S, false, 64>;
+        fbm = 64;
+      }
     }
+    const dim3 grid((unsigned)(ceil_div(max_m, fbm) * ceil_div(max_n, FBN)), (unsigned)nitems, (unsigned)splits);
+    const size_t smem = 2 * sizeof(typename ffv<S>::type) * FBK * (fbm + FBN);
+    PD_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<grid, 8 * fbm, smem, st>>>(d_items, alpha, beta, splits, part, part_stride, herm, triB);
   } else {
     dim3 grid((unsigned)(ceil_div(max_m, GBM) * ceil_div(max_n, GBN)), (unsigned)nitems, (unsigned)splits);
     if (conjA)

@@ -208,3 +208,23 @@ def test_exponents_at_the_ends_of_the_range(pk, cplx, n, m):
     big = np.abs(X) >= 2.0 ** -1022
     # subnormal data counts as zero in the digits
     assert np.array_equal(out, np.where(big[p], ref, 0))
+
+
+@pytest.mark.parametrize("sizes", [[267, 64, 65], [129, 128, 1, 200]])
+def test_float_float_tiles_agree(pk, sizes):
+    """Complex float-float products of many tiles take 64 rows to a tile, small ones 32: rows of X T do not depend
+    on it to the last bit, Gram matrices stay within the bound above."""
+    n = 5003
+    X = _blocks(n, sizes, True, 91, scales=False)
+    T = [_t(pk, t) for t in (_blocks(m, [m], True, 92 + m, scales=False) for m in sizes)]
+    Xd = _t(pk, X)
+    whole = pk.block_gemm(pk.GEMM_UPDATE, Xd, sizes, T, arith=pk.RR_FLOATFLOAT).cpu().numpy()
+    for i in (0, 300, 4700):
+        part = pk.block_gemm(pk.GEMM_UPDATE, Xd[:, i:i + 303].contiguous(), sizes, T, arith=pk.RR_FLOATFLOAT)
+        assert np.array_equal(part.cpu().numpy(), whole[:, i:i + 303])
+    off = 0
+    for m, g in zip(sizes, pk.block_gemm(pk.GEMM_GRAM, Xd, sizes, arith=pk.RR_FLOATFLOAT)):
+        A = X[off: off + m].T
+        nrm = np.linalg.norm(A, axis=0)
+        assert _rel_err(g.cpu().numpy(), A.conj().T @ A, nrm, nrm) <= 5e-13
+        off += m
