@@ -124,6 +124,8 @@ typedef struct {
 /* them as float-float (FP32 pairs, ~48-bit products, FP32 exponent range) on  */
 /* the FP32 pipes, which GB300 has 64x more of than FP64; FP64 keeps them in   */
 /* FP64 arithmetic.  Counts and residual tests are the same either way.       */
+/* (PDESHEP_FP64 calls are FP64 throughout, but for the FP32 starting vectors  */
+/* of the small eigenproblems and what brings them closer: see pdeshep_eigh.)  */
 #define PDESHEP_RR_FLOATFLOAT 0
 #define PDESHEP_RR_FP64 1
 #define PDESHEP_RR_TENSOR 2   /* bf16 digit products on the tensor cores (FP64-class) */

@@ -667,9 +667,9 @@ static int single_per_sm(int b) {
   std::lock_guard<std::mutex> lk(mu);
   const auto it = known.find(std::make_pair(dev, b));
   if (it != known.end()) return it->second;
-  const size_t smem = single_smem(b, CPLX);
-  cudaError_t e = cudaFuncSetAttribute(inertia_kernel<CPLX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, inertia_kernel<CPLX>, 256, smem);
+  cudaError_t e = cudaFuncSetAttribute(inertia_kernel<CPLX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, inertia_kernel<CPLX>, 256, single_smem(b, CPLX));
   if (e != cudaSuccess) cudaGetLastError();
   if (known.size() > 4096) known.clear();
   return known[std::make_pair(dev, b)] = std::max(per, 1);
@@ -754,7 +754,7 @@ int launch_inertia(int64_t n, int b, int cplx, const void* band, int64_t ldab, i
                 : launch_panel<false>(n, b, band, ldab, nsigma, d_sigma, amax, d_neg, d_piv, G, st);
   const size_t smem = single ? single_smem(b, cplx) : inertia_smem_base(b, cplx);
   auto kern = cplx ? inertia_kernel<true> : inertia_kernel<false>;
-  PD_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PD_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
   kern<<<nsigma, 256, smem, st>>>(n, b, (const double*)band, ldab, d_sigma, amax, d_neg, d_piv,
                                   single ? nullptr : gwin, gwin_stride);
   PD_CK_LAUNCH();
