@@ -1634,11 +1634,11 @@ __global__ void refined_values_kernel(const SmallDesc* desc, S* Sall, S* Pall, d
 template <typename S>
 __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall, const S* Pall, const double* lamall,
                                                   double* est_out, double* reach_all, double coupled,
-                                                  int balanced) {
+                                                  double sep, int balanced) {
   // One refinement step (Ogita and Aishima, 2018) for block t, given S = V^H A V
   // and P = V^H V of the current approximate eigenvectors V:
   //   lambda_i = S_ii / P_ii, R = I - P, c_ij = S_ij + lambda_j R_ij,
-  //   E_ij = c_ij / (lambda_j - lambda_i)   for a separated pair (|gap| > 4 max(|c_ij|, |c_ji|)),
+  //   E_ij = c_ij / (lambda_j - lambda_i)   for a separated pair (|gap| > sep max(|c_ij|, |c_ji|), sep >= 4),
   //   E_ij = R_ij / 2                       otherwise (and on the diagonal),
   // and V <- V (I + E) (done by the caller).  A separated pair gets |E_ij| < 1/4
   // and converges quadratically.  A pair that is not separated although it is
@@ -1698,10 +1698,10 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
         // The largest part cm bounds ca = max(|c_ij|, |c_ji|) from both sides, cm <= ca < 1.4143 cm: most pairs are
         // separated for certain, without the two hypotenuses (half of the kernel's FP64 instructions).
         const double cm = __longlong_as_double((long long)max(abs_bits(c), abs_bits(ct)));
-        const bool apart = cm > tiny && fabs(gap) > 5.66 * cm;
+        const bool apart = cm > tiny && fabs(gap) > 1.415 * sep * cm;
         const double ca = apart ? cm : fmax(sc<S>::absv(c), sc<S>::absv(ct));
         if (ca > tiny) {
-          if (apart || fabs(gap) > 4.0 * ca) {
+          if (apart || fabs(gap) > sep * ca) {
             const double rg = divide(1.0, gap);
             if (balanced)
               ev = sc<S>::add(ev, sc<S>::scale(sc<S>::add(Sm[e], sc<S>::scale(r, 0.5 * (li + lj))), rg));
@@ -1901,13 +1901,15 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
   // FP64 refinement of V (kept in Vd): each step roughly squares the error of the
   // separated pairs.  A block leaves the batch after the step whose correction was
   // below kRefineTol (what remains is of the order of its square); at most
-  // kRefineSteps steps.
+  // kRefineSteps steps.  What keeps a block longer is a pair that is separated while both its members are coupled to a
+  // third one that is not: its correction comes back in every step (3.5e-2 or 5e-3 in blocks of 162 with doublets,
+  // which then went to the full FP64 Jacobi).  With FP64 callers such pairs join the cluster from step kLateStep on.
   S* V = w.Vd;
   S* Vn = w.Vw;
   std::vector<double> drel(nblk, 1.0), est(nblk), estp((size_t)nblk * kOaSplit);
   std::vector<int> act, next;
   // one step on the blocks of act; their corrections in est[0 ..)
-  auto refine_step = [&](int ff, double coupled) -> int {
+  auto refine_step = [&](int ff, double coupled, double sep) -> int {
     const int na = (int)act.size();
     std::vector<SmallDesc> sub_d(na);
     for (int q = 0; q < na; ++q) sub_d[q] = all[act[q]];
@@ -1930,7 +1932,8 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
     }
     refined_values_kernel<S><<<dim3(na, (max_m + 63) / 64), 256, 0, st>>>(dd, w.W64, w.T, w.lam32, w.coarse);
     PD_CK_LAUNCH();
-    oa_kernel<S><<<dim3(na, kOaSplit), 256, 0, st>>>(dd, w.W64, w.T, w.lam32, w.delta, w.reach, coupled, w.coarse);
+    oa_kernel<S><<<dim3(na, kOaSplit), 256, 0, st>>>(dd, w.W64, w.T, w.lam32, w.delta, w.reach, coupled, sep,
+                                                        w.coarse);
     PD_CK_LAUNCH();
     for (auto& b : sub_d)
       PD_CK(cudaMemcpyAsync(Vn + b.off, V + b.off, sizeof(S) * (size_t)b.m * b.m, cudaMemcpyDeviceToDevice, st));
@@ -1974,7 +1977,7 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
     for (int t : act) work += (double)all[t].m * all[t].m * all[t].m * (sizeof(S) == sizeof(double2) ? 4.0 : 1.0);
     if (work < kCoarseWork) act.clear();
     for (int it = 0; it < kCoarseSteps && !act.empty(); ++it) {
-      PD_TRY(refine_step(1, kCoarseCoupled));
+      PD_TRY(refine_step(1, kCoarseCoupled, kApart));
       next.clear();
       for (size_t q = 0; q < act.size(); ++q) {
         if (est[q] * est[q] > kRefineTol && est[q] <= 0.25 * last[act[q]]) next.push_back(act[q]);
@@ -1986,7 +1989,7 @@ int eigh_mixed(int nblk, const SmallDesc* d_desc, const SmallDesc* h_desc, int m
   }
   for (int t = 0; t < nblk; ++t) act.push_back(t);
   for (int it = 0; it < kRefineSteps && !act.empty(); ++it) {
-    PD_TRY(refine_step(w.ff, kCoupled));
+    PD_TRY(refine_step(w.ff, kCoupled, w.coarse && it >= kLateStep ? kLateApart : kApart));
     next.clear();
     for (size_t q = 0; q < act.size(); ++q) {
       drel[act[q]] = est[q];

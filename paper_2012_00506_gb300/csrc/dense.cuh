@@ -104,6 +104,9 @@ constexpr int kMaxCluster = 64;
 constexpr int kRefineSteps = 10;
 constexpr double kRefineTol = 1e-8;
 constexpr double kCoupled = 1e-14;        // pairs with |c_ij| below this times max|lambda| count as uncoupled
+constexpr double kApart = 4.0;            // a pair is separated if its gap exceeds this times its coupling
+constexpr int kLateStep = 5;              // FP64 callers: from this step on ...
+constexpr double kLateApart = 1e4;        // ... this (corrections below sqrt(kRefineTol))
 constexpr int kCoarseSteps = 3;           // float-float steps before the FP64 ones, at most
 constexpr double kCoarseCoupled = 1e-12;  // ... and their bound on |c_ij|
 constexpr double kCoarseWork = 8e7;       // ... taken from this many real multiplications of one m x m product on
