@@ -1678,6 +1678,7 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
   __syncthreads();
   const double tiny = coupled * sh_l;
   double emax = 0.0, rmax = 0.0;
+  unsigned long long top = 0;  // the largest part of c_ij, c_ji and R_ij, NaN above all (the maxima pass over NaN)
   for (int j = blockIdx.y * nw + warp; j < m; j += gridDim.y * nw) {
     const double lj = lam[j];
     double rj = -INFINITY;
@@ -1686,6 +1687,7 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
       S r = sc<S>::scale(P[e], -1.0);
       if (i == j) r = sc<S>::add(r, sc<S>::from_re(1.0));
       rmax = fmax(rmax, sc<S>::abs2(r));  // (the square root of the largest, below)
+      top = max(top, abs_bits(r));
       S ev = sc<S>::scale(r, 0.5);
       if (i != j) {
         // c_ij and |c_ji| = |S_ij + lambda_i R_ij|: the pair is classified on the
@@ -1697,7 +1699,9 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
         const double gap = lj - li;
         // The largest part cm bounds ca = max(|c_ij|, |c_ji|) from both sides, cm <= ca < 1.4143 cm: most pairs are
         // separated for certain, without the two hypotenuses (half of the kernel's FP64 instructions).
-        const double cm = __longlong_as_double((long long)max(abs_bits(c), abs_bits(ct)));
+        const unsigned long long cb = max(abs_bits(c), abs_bits(ct));
+        const double cm = __longlong_as_double((long long)cb);
+        top = max(top, cb);
         const bool apart = cm > tiny && fabs(gap) > 1.415 * sep * cm;
         const double ca = apart ? cm : fmax(sc<S>::absv(c), sc<S>::absv(ct));
         if (ca > tiny) {
@@ -1721,6 +1725,7 @@ __global__ void __launch_bounds__(256) oa_kernel(const SmallDesc* desc, S* Sall,
     for (int o = 16; o > 0; o >>= 1) rj = fmax(rj, __shfl_down_sync(0xffffffffu, rj, o));
     if (lane == 0) reach[j] = rj;
   }
+  if (top >= 0x7FF0000000000000ull) emax = INFINITY;  // V or its products are not finite: never below the tolerance
   for (int o = 16; o > 0; o >>= 1) {
     emax = fmax(emax, __shfl_down_sync(0xffffffffu, emax, o));
     rmax = fmax(rmax, __shfl_down_sync(0xffffffffu, rmax, o));

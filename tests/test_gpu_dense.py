@@ -192,3 +192,23 @@ def test_eigh_of_doublets(device, cplx, nblk, m, gap):
         assert np.max(np.abs(lam - np.linalg.eigvalsh(A))) < 1e-13 * nrm
         assert np.max(np.abs(V.conj().T @ V - np.eye(len(lam)))) < 1e-13
         assert np.max(np.abs(A @ V - V * lam)) < 1e-13 * nrm
+
+
+@pytest.mark.parametrize("cplx,nblk,m", [(False, 6, 267), (True, 3, 200), (True, 1, 50), (False, 4, 90)])
+@pytest.mark.parametrize("scale", [1e-140, 1e-100, 1e-60, 1e-38, 1e-30, 1e18, 1e30, 1e37, 1e39, 1e100, 1e140])
+def test_eigh_of_any_scale(device, cplx, nblk, m, scale):
+    """Matrices far out of FP32's range or near its ends: the FP32 start is no help, the refinement may diverge
+    from it to infinity, and the block then has to be redone, never returned."""
+    import torch
+    import paper_2012_00506_gb300 as pk
+    rng = np.random.default_rng(1)
+    mats = []
+    for t in range(nblk):
+        A = rng.normal(size=(m, m)) + (1j * rng.normal(size=(m, m)) if cplx else 0)
+        mats.append(0.5 * (A + A.conj().T))
+    for A, (lam, V) in zip(mats, pk.eigh([torch.from_numpy(A * scale).to(device) for A in mats])):
+        lam, V = lam.cpu().numpy() / scale, V.cpu().numpy()
+        nrm = np.linalg.norm(A)
+        assert np.max(np.abs(lam - np.linalg.eigvalsh(A))) < 1e-13 * nrm
+        assert np.max(np.abs(V.conj().T @ V - np.eye(m))) < 1e-13
+        assert np.max(np.abs(A @ V - V * lam)) < 1e-13 * nrm
